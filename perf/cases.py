@@ -156,12 +156,16 @@ def _drop(c, rng):
 
 
 def _bubble(c, rng, frozen=False):
-    """Rising bubble in a no-slip box at 1/4 height, density ratio 1000, viscosity ratio 100."""
+    """Rising bubble in a no-slip box at 1/4 height: density ratio 1000, viscosity ratio 100; with FP16 storage the
+    paper's parameter set I (both 10), members of an ensemble in between."""
     base, L = _dims(c), c["levels"]
     D, r = len(base), 2 ** (c["levels"] - 1)
     nf = tuple(n * r for n in base)
     R = c["radius"] * r
-    prm = workloads.bubble_params(2 * R, 35.0, 10.0 * rng.uniform(0.8, 1.2), 1000.0, 100.0, Ma=0.01 if D == 2 else 0.005)
+    ratios = (1000.0, 100.0) if c["storage"] == "fp32" else (10.0, 10.0)
+    if c["kind"] == "ensemble":
+        ratios = (10.0 ** rng.uniform(1.0, 2.0), 10.0)
+    prm = workloads.bubble_params(2 * R, 35.0, 10.0 * rng.uniform(0.8, 1.2), *ratios, Ma=0.005)
     centre = [(n / 2 if a < D - 1 else n / 4) * r + rng.random() * 0.5 * r for a, n in enumerate(base)]
     dist = 16.0 if D == 2 else max(8.0, 2.0 * c["radius"])
     dref = [48.0] + [16.0] * (L - 2) if L > 2 else [dist] * (L - 1)
