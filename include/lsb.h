@@ -161,13 +161,16 @@ lsb_status lsb_use_graphs(lsb_grid *g, int enable);
 
 /*
  * Launch structure of the level-set update (Sec. 2.2 passes: extension sweeps,
- * TVD-RK3 transport, reinitialisation).  mode 0 (default): one launch per pass
- * (up to 16 per finest step).  mode 1: one persistent cooperative launch per
- * finest step that runs every pass over the band work list of all cases, with
- * a device-wide barrier between passes; the barrier's wait has an iteration
- * limit, and on expiry the kernel ends and the next synchronising call returns
- * LSB_ETIMEOUT.  Both modes give identical results.  Errors: LSB_EINVAL (bad
- * mode, or no cooperative launch on this device).
+ * TVD-RK3 transport, reinitialisation).  mode 0 (default): the passes and the
+ * classification's phase and cut-link passes in one launch per finest step, on
+ * stage arrays that need no band lookups (one thread-block cluster for a small
+ * band, a cooperative launch with bounded device-wide barriers otherwise).
+ * mode 1: one persistent cooperative launch per finest step that runs the
+ * level-set passes over the band work list of all cases with a lookup per
+ * stencil point, and a device-wide barrier between passes; the barrier's wait
+ * has an iteration limit, and on expiry the kernel ends and the next
+ * synchronising call returns LSB_ETIMEOUT.  Both modes give identical results.
+ * Errors: LSB_EINVAL (bad mode, or no cooperative launch on this device).
  */
 lsb_status lsb_set_driver(lsb_grid *g, int mode);
 

@@ -99,7 +99,9 @@ struct lsb_grid {
   int *d_work = nullptr;  // per level: the collide-and-stream's block counters (next, finished)
   int *d_counters = nullptr, *d_err = nullptr, *d_band = nullptr, *d_check = nullptr;
   int4 *d_band_info = nullptr;
-  unsigned *d_bar = nullptr;  // grid barrier of the persistent level-set kernel
+  unsigned *d_bar = nullptr;  // grid barriers: of the persistent level-set kernel, of the one-launch update
+  LsfLimits lsf_lim;
+  LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
   long long wait_limit = 1LL << 22;  // sleeps of ~64 ns before a device-side wait gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
@@ -146,7 +148,7 @@ struct lsb_grid {
   cudaStream_t side2[MAXL] = {};
   cudaEvent_t ev_free[MAXL] = {}, ev_fill[MAXL] = {}, ev_ring0[MAXL] = {}, ev_ring0_done[MAXL] = {};
   int early_fill = -1;  // level whose next ghost ring fills right after its collide
-  bool counters_turned[MAXL] = {};  // the level's classification counters already started
+  bool classified[MAXL] = {};  // the level's phases and cut links came with the level-set update
   bool init_done[MAXL] = {};        // the level's interface u~ came with the interface pass
   uint64_t gnodes[2][2] = {};
   // adjoint of the frozen-interface step: recording and reverse sweep
@@ -521,44 +523,40 @@ bool has_finest(const lsb_grid *g, int l) {
 #endif
 lsb_status classify(lsb_grid *g, int l, int init, bool refill = false) {
   if (!has_finest(g, l)) return LSB_OK;
-  // the band list the previous classification left is the set of blocks whose phases can
-  // change (phi moves on band cells only): keep its length, then clear the counters
-  // (the first extension sweep of this sub-step did it already; the phase pass clears the
-  // band count)
-  int *cnt = g->d_counters + l * NCOUNT;
-  if (init || !g->counters_turned[l]) {
-    CU(cudaMemcpyAsync(cnt + 5, cnt + 3, sizeof(int), cudaMemcpyDeviceToDevice, g->stream));
-    CU(cudaMemsetAsync(cnt, 0, sizeof(int) * 5, g->stream));
-  }
-  g->counters_turned[l] = false;
   Ctx C = make_ctx(g);
   BlockShape S = shape(g);
   WorkList &F = g->finest[l];
   const int *fl = F.d;
-  const int Q = g->Q, D = g->D, nt = g->nthreads;
-  // after creation or a regrid every finest block; otherwise the previous band's blocks
-  // (and, for the cut links, the blocks next to a flipped cell), walked from the lists
-  const int nlist = init ? F.n : std::max(1, std::min(F.n, 152 * LSB_CLS_CTAS));
-  RUN(8, 0, F.n, nt, run_classify_phase, Q, LN(g, nlist, nt), C, S, fl, F.n, l, init);
-  RUN(9, 0, F.n, nt, run_classify_links, Q, LN(g, nlist, nt), C, S, fl, F.n, l, init);
+  const int Q = g->Q, nt = g->nthreads;
+  if (init || !g->classified[l]) {
+    // the band list the previous classification left is the set of blocks whose phases can
+    // change (phi moves on band cells only): keep its length, then clear the counters
+    int *cnt = g->d_counters + l * NCOUNT;
+    CU(cudaMemcpyAsync(cnt + 5, cnt + 3, sizeof(int), cudaMemcpyDeviceToDevice, g->stream));
+    CU(cudaMemsetAsync(cnt, 0, sizeof(int) * 5, g->stream));
+    // after creation or a regrid every finest block; otherwise the previous band's blocks
+    // (and, for the cut links, the blocks next to a flipped cell), walked from the lists
+    const int nlist = init ? F.n : std::max(1, std::min(F.n, 152 * LSB_CLS_CTAS));
+    RUN(8, 0, F.n, nt, run_classify_phase, Q, LN(g, nlist, nt), C, S, fl, F.n, l, init);
+    RUN(9, 0, F.n, nt, run_classify_links, Q, LN(g, nlist, nt), C, S, fl, F.n, l, init);
+  }
+  g->classified[l] = false;
   // the band pass (a warp per block) and the curvature fit at the interface and the
   // flipped cells (and the refill of the flipped cells) share a launch
   const int gband = (F.n + 3) / 4;
   RUN(10, 0, F.n, 128, run_post_classify, Q, g->storage, LN(g, LSB_GEO_CTAS + gband, 128), C, fl, F.n, l,
       LSB_GEO_CTAS, refill ? 1 : 0);
-  (void)D;
   return LSB_OK;
 }
 
-// The precondition of the mirrored level-set passes, set in full: p1 = p2 = phi and
-// ut1 = ut2 = ut0 at every finest cell (after creation and after phi or u~ were
-// restored from a stored state).
+// The precondition of the mirrored level-set passes, set in full: p1 = p2 = phi and both
+// sweep buffers = ut0 at every finest cell (after creation and after phi or u~ were
+// restored from a stored state, or the persistent driver used the arrays as scratch).
 lsb_status ls_mirror(lsb_grid *g) {
-  const size_t b1 = sizeof(float) * (size_t)g->nfine, bD = b1 * g->D;
+  const size_t b1 = sizeof(float) * (size_t)g->nfine;
   CU(cudaMemcpyAsync(g->d_p1, g->d_phi, b1, cudaMemcpyDeviceToDevice, g->stream));
   CU(cudaMemcpyAsync(g->d_p2, g->d_phi, b1, cudaMemcpyDeviceToDevice, g->stream));
-  CU(cudaMemcpyAsync(g->d_ut[1], g->d_ut[0], bD, cudaMemcpyDeviceToDevice, g->stream));
-  CU(cudaMemcpyAsync(g->d_ut[2], g->d_ut[0], bD, cudaMemcpyDeviceToDevice, g->stream));
+  TRY(launched(g, run_ut_pack(g->D, LN(g, DYN_GRID, 256), g->d_ut[0], g->d_ut[1], g->d_ut[2], g->nfine)));
   g->ls_dirty = false;
   return LSB_OK;
 }
@@ -579,31 +577,45 @@ lsb_status levelset(lsb_grid *g, int l) {
         g->n_reinit, g->d_bar, g->wait_limit);
     return LSB_OK;
   }
-  // passes on mirrored stage arrays: the first sweep stores the plan, the others reuse
-  // it; the first transport stage commits u~; the first reinitialisation stage finds
-  // the frozen cells
   if (!g->init_done[l]) RUN(12, 0, 1, 128, run_ext_init, Q, LN(g, DYN_GRID, 128), C, l);
   g->init_done[l] = false;
-  const float *uin = g->d_ut[0];
-  for (int it = 0; it < g->n_ext; ++it) {
-    float *uout = g->d_ut[1 + (it & 1)];
-    if (it == 0) {
-      RUN(13, 0, nb, nt, run_ext_first, D, LN(g, nb, nt), C, S, l, uin, uout, 1);
-      g->counters_turned[l] = true;  // the classification of this sub-step finds them started
-    }
-    else RUN(13, 0, nb, nt, run_ext_sweep_mirror, D, LN(g, nb, nt), C, S, l, uin, uout);
-    uin = uout;
-  }
-  for (int st = 1; st <= 3; ++st) {
-    RUN(14, 0, nb, nt, run_adv_mirror, D, LN(g, nb, nt), C, S, l, st, uin);
-  }
   const bool due = g->reinit_every > 0 && ((g->fine_steps[l] + 1) % g->reinit_every == 0);
-  if (due && g->n_reinit > 0) {
-    for (int r = 0; r < g->n_reinit; ++r)
-      for (int st = 1; st <= 3; ++st) {
-        RUN(16, 0, nb, nt, run_reinit_mirror, Q, LN(g, nb, nt), C, S, l, st, r == 0 && st == 1 ? 1 : 0);
-      }
+  RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
+      (int)g->lds.size(), g->d_bar + 2);
+  g->classified[l] = true;
+  return LSB_OK;
+}
+
+// Shape of the one-launch level-set update of level l from the band its classification
+// just listed (the launch is right for any band; the shape only sets its speed).  Up to two
+// cells per thread of a 16-CTA cluster of 1024 threads the cluster's barrier wins (0.6 -
+// 1.0 us a pass against 1.4 us of the grid's); beyond, a pass is bound by its loads and a
+// grid over all SMs takes over.
+lsb_status plan_levelset(lsb_grid *g, int l) {
+  int nb = 0;
+  CU(cudaMemcpyAsync(&nb, g->d_counters + l * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  CU(cudaStreamSynchronize(g->stream));
+  nb = std::max(1, std::min(nb, g->band_cap));
+  nb += nb / 16;  // room for the band to grow until the next regrid
+  const int nt = g->nthreads, per = 1024 / nt;  // blocks of a full CTA
+  const LsfLimits &M = g->lsf_lim;
+  LsfPlan P;
+  if (nb <= M.cluster * per * 2 || M.grid == 0) {
+    P.coop = 0;
+    P.grid = 1;
+    while (P.grid < M.cluster && P.grid < nb) P.grid *= 2;
+    const int each = (nb + P.grid - 1) / P.grid;  // blocks per CTA
+    P.threads = nt * std::min(per, each);
+    P.kcap = std::min(M.kmax, (each + per - 1) / per);
+  } else {
+    P.coop = 1;
+    const int each = std::min(per, (nb + M.grid - 1) / M.grid);
+    P.threads = nt * each;
+    P.grid = std::min(M.grid, (nb + each - 1) / each);
+    P.kcap = std::min(M.kmax, (nb + P.grid * each - 1) / (P.grid * each));
   }
+  if ((int)g->lds.size() > M.max_ld) P.kcap = 0;
+  g->lsf[l] = P;
   return LSB_OK;
 }
 
@@ -1589,7 +1601,8 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
   ALLOC(g->d_p2, 4 * nf);
   ALLOC(g->d_s0, 4 * nf);
   ALLOC(g->d_frozen, nf);
-  for (int k = 0; k < 3; ++k) ALLOC(g->d_ut[k], 4 * D * nf);
+  ALLOC(g->d_ut[0], 4 * D * nf);
+  for (int k = 1; k < 3; ++k) ALLOC(g->d_ut[k], (D == 2 ? 8 : 16) * nf);  // sweep buffers: a vector per cell
   ALLOC(g->d_plan_v, 4 * D * nf);
   ALLOC(g->d_plan_f, nf);
   ALLOC(g->d_cmask, 4 * nf);
@@ -1621,7 +1634,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
     if (cudaDeviceGetStreamPriorityRange(&lo, &hi) == cudaSuccess) g->prio_hi = hi;
     else cudaGetLastError();
   }
-  ALLOC(g->d_bar, 2 * sizeof(unsigned));
+  ALLOC(g->d_bar, 4 * sizeof(unsigned));
   ALLOC(g->d_iface, sizeof(int2) * MAXL * g->list_cap);
   ALLOC(g->d_flip, sizeof(int2) * MAXL * g->list_cap);
   ALLOC(g->d_band, sizeof(int) * MAXL * (size_t)std::max(1, g->band_cap));
@@ -1652,7 +1665,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
       cuerr(cudaMemset(g->d_bflag, 0, g->nblock_total), "bflag") ||
       cuerr(cudaMemset(g->d_err, 0, sizeof(int)), "err") ||
       cuerr(cudaMemset(g->d_work, 0, sizeof(int) * 2 * MAXL), "work") ||
-      cuerr(cudaMemset(g->d_bar, 0, 2 * sizeof(unsigned)), "barrier") ||
+      cuerr(cudaMemset(g->d_bar, 0, 4 * sizeof(unsigned)), "barrier") ||
       cuerr(cudaMemset(g->d_counters, 0, sizeof(int) * MAXL * NCOUNT), "counters") ||
       cuerr(cudaMemset(g->d_cmask, 0, 4 * nf), "cmask") ||
       cuerr(cudaMemset(g->d_nvec, 0, 4 * D * nf), "nvec") ||
@@ -1663,8 +1676,8 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
     lsb_destroy(g);
     return LSB_ECUDA;
   }
-  for (int k = 0; k < 3; ++k)
-    if (cuerr(cudaMemset(g->d_ut[k], 0, 4 * D * nf), "ut")) { lsb_destroy(g); return LSB_ECUDA; }
+  // (the sweep buffers are filled from it by ls_mirror)
+  if (cuerr(cudaMemset(g->d_ut[0], 0, 4 * D * nf), "ut")) { lsb_destroy(g); return LSB_ECUDA; }
   // phi: dense caller array -> padded finest array
   for (int c = 0; c < n_cases; ++c) {
     const LevelDev &F = g->lds[g->cases[c].ld0 + g->cases[c].L - 1];
@@ -1677,6 +1690,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
     pr.kind = cudaMemcpyDeviceToDevice;
     if (cuerr(cudaMemcpy3D(&pr), "phi0 copy")) { lsb_destroy(g); return LSB_ECUDA; }
   }
+  if (cuerr(prepare_levelset_fused(g->Q, &g->lsf_lim), "level-set launch")) { lsb_destroy(g); return LSB_ECUDA; }
   s = build_tensor_maps(g);
   if (s == LSB_OK) s = ls_mirror(g);
   if (s == LSB_OK) s = regrid(g, true);
@@ -2526,7 +2540,10 @@ lsb_status regrid(lsb_grid *g, bool initial) {
   TRY(collect_cells(g));
   drop_graphs(g);
   CU(cudaMemsetAsync(g->d_bflag, 0, g->nblock_total, g->stream));
-  for (int l = 0; l < g->Lmax; ++l) TRY(classify(g, l, 1));
+  for (int l = 0; l < g->Lmax; ++l) {
+    TRY(classify(g, l, 1));
+    if (has_finest(g, l)) TRY(plan_levelset(g, l));
+  }
   return LSB_OK;
 }
 

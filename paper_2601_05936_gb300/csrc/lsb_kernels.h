@@ -103,12 +103,21 @@ cudaError_t run_ext_iter(int D, Launch L, Ctx C, BlockShape S, int glevel, const
 cudaError_t run_adv_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage);
 cudaError_t run_reinit_prep(int Q, Launch L, Ctx C, BlockShape S, int glevel);
 cudaError_t run_reinit_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage);
-// forward passes on mirrored stage arrays (no band lookups; see lsb_ls.cu)
-cudaError_t run_ext_first(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *uin, float *uout,
-                          int turn);
-cudaError_t run_ext_sweep_mirror(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *uin, float *uout);
-cudaError_t run_adv_mirror(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage, const float *ufin);
-cudaError_t run_reinit_mirror(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, int prep);
+// The level-set update and the classification's phase and link passes of a finest sub-step
+// in one launch (see k_levelset_fused).  LsfLimits: what the device allows (kmax slots of
+// 1024 threads in shared memory, CTAs of a cooperative launch or 0, largest cluster);
+// LsfPlan: one level's launch.
+struct LsfLimits {
+  int kmax = 0, grid = 0, cluster = 0, max_ld = 0;
+};
+struct LsfPlan {
+  int coop = 0, grid = 1, threads = 0, kcap = 1;
+};
+cudaError_t prepare_levelset_fused(int Q, LsfLimits *out);
+// ut0's planes into the interleaved sweep buffers (n finest cells)
+cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n);
+cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
+                               unsigned *bar);
 // the curvature fit of the interface and flipped cells on CTAs [0, gg) (each flipped cell
 // then refilled when refill is set) and the band pass on the rest, one launch
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,

@@ -23,6 +23,38 @@ __device__ __forceinline__ bool in_band(const Ctx &C, const LevelDev &L, const B
 }
 
 // ------------------------------------------------------------------ classification
+// A cell that changed phase: into the flip list, and the blocks around it that the previous
+// band does not hold into the check list (the band flags tested here are those of the
+// previous classification, which no thread of the phase pass changes).
+template <int Q>
+__device__ __forceinline__ void list_flip(const Ctx &C, const LevelDev &L, const BlockShape &S, int glevel, int ld,
+                                       long long c, int x, int y, int z) {
+  using LT = Lat<Q>;
+  constexpr int D = LT::D;
+  int e = atomicAdd(&C.counters[glevel * NCOUNT + 2], 1);
+  if (e < C.list_cap) C.flip_list[(long long)glevel * C.list_cap + e] = make_int2(ld, (int)c);
+  else atomicOr(C.err, ERR_LIST_OVF);
+  for (int k = 0; k < Q; ++k) {
+    int sx = x + LT::cx(k), sy = y + LT::cy(k), sz = z + LT::cz(k);
+    if (!(wrap(L, 0, sx) && wrap(L, 1, sy) && (D == 2 || wrap(L, 2, sz)))) continue;
+    const int nb = L.block_off + block_of(L, sx, sy, sz, S);
+    // set BF_CHECK once per block (compare-and-swap on the flag's word) and list it
+    unsigned *wp = reinterpret_cast<unsigned *>(C.bflag + (nb & ~3));
+    const int sh = (nb & 3) * 8;
+    unsigned old = *reinterpret_cast<volatile unsigned *>(wp);
+    while (!(((old >> sh) & 0xffu) & (BF_BAND | BF_CHECK))) {
+      const unsigned seen = atomicCAS(wp, old, old | ((unsigned)BF_CHECK << sh));
+      if (seen == old) {
+        const int slot = atomicAdd(&C.counters[glevel * NCOUNT + 4], 1);
+        if (slot < C.band_cap) C.check_list[(long long)glevel * C.band_cap + slot] = nb;
+        else atomicOr(C.err, ERR_BAND_OVF);
+        break;
+      }
+      old = seen;
+    }
+  }
+}
+
 // Pass 1: phase of every leaf cell from phi (liquid iff phi < 0); flipped cells
 // are listed.  init = 1 (after creation or regrid): all blocks, no flips,
 // previous = current.  Otherwise only blocks of the previous band (they keep the band
@@ -62,34 +94,117 @@ __global__ void k_classify_phase(Ctx C, BlockShape S, const int *list, int nlist
     uint8_t nt = (tg & (TAG_LEAF | TAG_RLAYER | TAG_GHOST)) | (gas ? TAG_GAS : 0) | (prev ? TAG_PREVGAS : 0) |
                  (flip ? TAG_FLIP : 0);
     C.tag[L.cell_off + c] = nt;
-    if (flip) {
-      int e = atomicAdd(&C.counters[glevel * NCOUNT + 2], 1);
-      if (e < C.list_cap) C.flip_list[(long long)glevel * C.list_cap + e] = make_int2(C.blk_ld[gb], (int)c);
-      else atomicOr(C.err, ERR_LIST_OVF);
-      // the blocks around the flip that the previous band does not hold: the band flags
-      // tested here are those of the previous classification, which no thread of this pass
-      // changes
-      for (int k = 0; k < Q; ++k) {
-        int sx = x + LT::cx(k), sy = y + LT::cy(k), sz = z + LT::cz(k);
-        if (!(wrap(L, 0, sx) && wrap(L, 1, sy) && (D == 2 || wrap(L, 2, sz)))) continue;
-        const int nb = L.block_off + block_of(L, sx, sy, sz, S);
-        // set BF_CHECK once per block (compare-and-swap on the flag's word) and list it
-        unsigned *wp = reinterpret_cast<unsigned *>(C.bflag + (nb & ~3));
-        const int sh = (nb & 3) * 8;
-        unsigned old = *reinterpret_cast<volatile unsigned *>(wp);
-        while (!(((old >> sh) & 0xffu) & (BF_BAND | BF_CHECK))) {
-          const unsigned seen = atomicCAS(wp, old, old | ((unsigned)BF_CHECK << sh));
-          if (seen == old) {
-            const int slot = atomicAdd(&C.counters[glevel * NCOUNT + 4], 1);
-            if (slot < C.band_cap) C.check_list[(long long)glevel * C.band_cap + slot] = nb;
-            else atomicOr(C.err, ERR_BAND_OVF);
-            break;
-          }
-          old = seen;
-        }
-      }
+    if (flip) list_flip<Q>(C, L, S, glevel, C.blk_ld[gb], c, x, y, z);
+  }
+}
+
+// Offsets from a cell to its neighbours at -1 and +1 along each axis (wrapped on periodic
+// axes), and a mask of the sides that lie behind a wall (bit 2 a: -1, bit 2 a + 1: +1).
+struct NearOff {
+  int m[3], p[3];
+  unsigned wall;
+};
+template <int D>
+__device__ __forceinline__ NearOff near_off(const int crd[3], const int n[3], unsigned per, unsigned p0, unsigned p01) {
+  NearOff o;
+  o.wall = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    o.m[a] = o.p[a] = 0;
+    if (a >= D) continue;
+    const int str = a == 0 ? 1 : (int)(a == 1 ? p0 : p01);
+    const bool w = (per >> a) & 1u;
+    o.m[a] = crd[a] > 0 ? -str : (n[a] - 1) * str;
+    o.p[a] = crd[a] < n[a] - 1 ? str : -(n[a] - 1) * str;
+    if (!w && crd[a] == 0) o.wall |= 1u << (2 * a);
+    if (!w && crd[a] == n[a] - 1) o.wall |= 2u << (2 * a);
+  }
+  return o;
+}
+// The offset to the neighbour in direction (x, y, z); out: it lies behind a wall.
+__device__ __forceinline__ int off_to(const NearOff &o, int x, int y, int z, bool &out) {
+  const unsigned need = (x < 0 ? 1u : (x > 0 ? 2u : 0u)) | (y < 0 ? 4u : (y > 0 ? 8u : 0u)) | (z < 0 ? 16u : (z > 0 ? 32u : 0u));
+  out = (o.wall & need) != 0;
+  return (x < 0 ? o.m[0] : (x > 0 ? o.p[0] : 0)) + (y < 0 ? o.m[1] : (y > 0 ? o.p[1] : 0)) +
+         (z < 0 ? o.m[2] : (z > 0 ? o.p[2] : 0));
+}
+__device__ __forceinline__ unsigned per_mask(const LevelDev &L) {
+  return (L.per[0] ? 1u : 0u) | (L.per[1] ? 2u : 0u) | (L.per[2] ? 4u : 0u);
+}
+
+// Cut mask of a cell with tag tg (tag pointer tc at the cell): bit k set when the source
+// x - c_k is a leaf of the other phase (no source through a wall).
+template <int Q>
+__device__ __forceinline__ uint32_t cut_mask(const uint8_t *tc, uint8_t tg, const NearOff &o) {
+  using LT = Lat<Q>;
+  uint32_t m = 0;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    if (k == LT::REST) continue;
+    bool out;
+    const int off = off_to(o, -LT::cx(k), -LT::cy(k), -LT::cz(k), out);
+    const uint8_t ts = tc[out ? 0 : off];  // a cell is never of the other phase to itself
+    if ((ts & TAG_LEAF) && ((ts ^ tg) & TAG_GAS)) m |= 1u << k;
+  }
+  return m;
+}
+
+// The same for a cell with every source in the box.
+template <int Q>
+__device__ __forceinline__ uint32_t cut_mask_inner(const uint8_t *tc, uint8_t tg, long long p0, long long p01) {
+  using LT = Lat<Q>;
+  uint32_t m = 0;
+#pragma unroll
+  for (int k = 0; k < Q; ++k) {
+    if (k == LT::REST) continue;
+    const uint8_t ts = tc[-(LT::cx(k) + LT::cy(k) * p0 + LT::cz(k) * p01)];
+    if ((ts & TAG_LEAF) && ((ts ^ tg) & TAG_GAS)) m |= 1u << k;
+  }
+  return m;
+}
+
+// Slots of a warp's cut links and interface cells in the lists (one atomic pair per warp;
+// every lane of the warp calls this), then the entries, the link base and TAG_IFACE of the
+// cell (ld, c) with cut mask m; fc and tc: its finest-level and tag indices.
+__device__ __forceinline__ void list_links(const Ctx &C, int glevel, uint32_t m, int ld, int c, long long fc,
+                                           long long tc, uint8_t tg) {
+  const int lane = threadIdx.x & 31;
+  const unsigned wcells = __ballot_sync(0xffffffffu, m != 0);
+  if (!wcells) return;
+  const int np = __popc(m);
+  int incl = np;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += t;
+  }
+  const int wlinks = __shfl_sync(0xffffffffu, incl, 31);
+  int lbase = 0, cbase0 = 0;
+  if (lane == 0) {
+    lbase = atomicAdd(&C.counters[glevel * NCOUNT + 0], wlinks);
+    cbase0 = atomicAdd(&C.counters[glevel * NCOUNT + 1], __popc(wcells));
+  }
+  lbase = __shfl_sync(0xffffffffu, lbase, 0);
+  cbase0 = __shfl_sync(0xffffffffu, cbase0, 0);
+  if (!m) return;
+  const int base = lbase + incl - np;
+  if ((long long)base + np > C.link_cap) atomicOr(C.err, ERR_LINK_OVF);
+  C.cbase[fc] = base;
+  // the link list: one entry per cut link, in link-buffer order
+  const int2 cell = make_int2(ld, c);
+  uint32_t mm = m;
+  for (int r = 0; mm; ++r) {
+    const int k = __ffs(mm) - 1;
+    mm &= mm - 1u;
+    if ((long long)base + r < C.link_cap) {
+      C.link_cell[C.link_list_off[glevel] + base + r] = cell;
+      C.link_dir[C.link_list_off[glevel] + base + r] = (uint8_t)k;
     }
   }
+  C.tag[tc] = tg | TAG_IFACE;
+  const int e = cbase0 + __popc(wcells & ((1u << lane) - 1u));
+  if (e < C.list_cap) C.iface_list[(long long)glevel * C.list_cap + e] = cell;
+  else atomicOr(C.err, ERR_LIST_OVF);
 }
 
 // Pass 2: cut mask of every leaf cell (bit k: source x - c_k is a leaf of the
@@ -129,67 +244,13 @@ __global__ void k_classify_links(Ctx C, BlockShape S, const int *list, int nlist
       c = cidx(L, x, y, z);
       tg = C.tag[L.cell_off + c];
       if (tg & TAG_LEAF) {
-        const bool inner = x >= 1 && x + 1 < L.n[0] && y >= 1 && y + 1 < L.n[1] && (D == 2 || (z >= 1 && z + 1 < L.n[2]));
-        if (inner) {  // every source inside the box: direct offsets
-          const long long p0 = L.p[0], p01 = (long long)L.p[0] * L.p[1];
-          const uint8_t *tc = C.tag + L.cell_off + c;
-#pragma unroll
-          for (int k = 0; k < Q; ++k) {
-            if (k == LT::REST) continue;
-            const uint8_t ts = tc[-(LT::cx(k) + LT::cy(k) * p0 + LT::cz(k) * p01)];
-            if ((ts & TAG_LEAF) && ((ts & TAG_GAS) != (tg & TAG_GAS))) m |= 1u << k;
-          }
-        } else {
-          for (int k = 0; k < Q; ++k) {
-            if (k == LT::REST) continue;
-            int sx = x - LT::cx(k), sy = y - LT::cy(k), sz = z - LT::cz(k);
-            if (!(wrap(L, 0, sx) && wrap(L, 1, sy) && (D == 2 || wrap(L, 2, sz)))) continue;
-            const uint8_t ts = C.tag[L.cell_off + cidx(L, sx, sy, sz)];
-            if ((ts & TAG_LEAF) && ((ts & TAG_GAS) != (tg & TAG_GAS))) m |= 1u << k;
-          }
-        }
+        const int crd[3] = {x, y, z};
+        m = cut_mask<Q>(C.tag + L.cell_off + c, tg,
+                        near_off<D>(crd, L.n, per_mask(L), (unsigned)L.p[0], (unsigned)(L.p[0] * L.p[1])));
         C.cmask[L.fine_off + c] = m;
       }
     }
-    // slots in the link list and the interface list, one atomic per warp (every lane
-    // of the CTA is here: the block-level branch above is uniform)
-    const int lane = threadIdx.x & 31;
-    const int np = __popc(m);
-    int incl = np;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int t = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += t;
-    }
-    const int wlinks = __shfl_sync(0xffffffffu, incl, 31);
-    const unsigned wcells = __ballot_sync(0xffffffffu, m != 0);
-    int lbase = 0, cbase0 = 0;
-    if (lane == 0 && wcells) {
-      lbase = atomicAdd(&C.counters[glevel * NCOUNT + 0], wlinks);
-      cbase0 = atomicAdd(&C.counters[glevel * NCOUNT + 1], __popc(wcells));
-    }
-    lbase = __shfl_sync(0xffffffffu, lbase, 0);
-    cbase0 = __shfl_sync(0xffffffffu, cbase0, 0);
-    if (m) {
-      const int base = lbase + incl - np;
-      if ((long long)base + np > C.link_cap) atomicOr(C.err, ERR_LINK_OVF);
-      C.cbase[L.fine_off + c] = base;
-      // the link list: one entry per cut link, in link-buffer order
-      const int2 cell = make_int2(C.blk_ld[gb], (int)c);
-      uint32_t mm = m;
-      for (int r = 0; mm; ++r) {
-        const int k = __ffs(mm) - 1;
-        mm &= mm - 1u;
-        if ((long long)base + r < C.link_cap) {
-          C.link_cell[C.link_list_off[glevel] + base + r] = cell;
-          C.link_dir[C.link_list_off[glevel] + base + r] = (uint8_t)k;
-        }
-      }
-      C.tag[L.cell_off + c] = tg | TAG_IFACE;
-      const int e = cbase0 + __popc(wcells & ((1u << lane) - 1u));
-      if (e < C.list_cap) C.iface_list[(long long)glevel * C.list_cap + e] = make_int2(C.blk_ld[gb], (int)c);
-      else atomicOr(C.err, ERR_LIST_OVF);
-    }
+    list_links(C, glevel, m, C.blk_ld[gb], (int)c, L.fine_off + c, L.cell_off + c, tg);
     const bool any = __syncthreads_or(m != 0);
     if (threadIdx.x == 0) C.bflag[gb] = any ? BF_IFACE : 0;
   }
@@ -482,9 +543,7 @@ __global__ void k_ext_iter(Ctx C, BlockShape S, int glevel, const float *uin, fl
 // plan, values, upwind neighbours) is latency-bound and the band holds only a few blocks
 // per resident CTA: one cell per thread (LSB_EXT_U blocks at once) at three CTAs per SM
 // measured faster than two blocks per thread at two CTAs per SM (more CTAs in flight).
-// MIRROR: the forward step's stage arrays equal ut0 outside the band, so every
-// upwind neighbour reads uin (no band bit of the plan consulted).
-template <int D, bool MIRROR = false>
+template <int D>
 __global__ void __launch_bounds__(512, LSB_EXT_MINB) k_ext_plan(Ctx C, BlockShape S, int glevel, const float *__restrict__ uin,
                                                      float *__restrict__ uout) {
   LSB_GRID_WAIT();
@@ -547,7 +606,7 @@ __global__ void __launch_bounds__(512, LSB_EXT_MINB) k_ext_plan(Ctx C, BlockShap
         } else {
           cn = c[k] + dir * (a == 0 ? 1LL : (a == 1 ? (long long)L.p[0] : (long long)L.p[0] * L.p[1]));
         }
-        const float *src = (MIRROR || ((pf[k] >> (3 + a)) & 1)) ? ui : C.ut0 + fo[k];
+        const float *src = ((pf[k] >> (3 + a)) & 1) ? ui : C.ut0 + fo[k];
 #pragma unroll
         for (int b = 0; b < D; ++b) un[k][a][b] = __ldg(src + b * NF + cn);
       }
@@ -708,16 +767,18 @@ __global__ void k_reinit_prep(Ctx C, BlockShape S, int glevel) {
   d_reinit_prep<Q>(C, S, glevel);
 }
 
-// HJ-WENO5 one-sided derivative (Jiang & Peng 2000) from the five differences.
-// Constant divisions are multiplications by the reciprocals, and the three weights
-// gamma_k / (s_k + eps)^2 are formed as gamma_k prod_{j != k} (s_j + eps)^2 (the
-// same normalised weights, one division instead of four).
-__device__ __forceinline__ float weno5(float v1, float v2, float v3, float v4, float v5) {
-  const float eps = 1e-6f;
+// HJ-WENO5 one-sided derivative (Jiang & Peng 2000) from the five differences: the three
+// candidates, and their weighted mean.  Constant divisions are multiplications by the
+// reciprocals, and the three weights gamma_k / (s_k + eps)^2 are formed as gamma_k
+// prod_{j != k} (s_j + eps)^2 (the same normalised weights, one division instead of four).
+__device__ __forceinline__ void weno5_candidates(float v1, float v2, float v3, float v4, float v5, float d[3]) {
   const float r3 = 1.f / 3.f, r6 = 1.f / 6.f;
-  const float d1 = v1 * r3 - 7.f * r6 * v2 + 11.f * r6 * v3;
-  const float d2 = -v2 * r6 + 5.f * r6 * v3 + v4 * r3;
-  const float d3 = v3 * r3 + 5.f * r6 * v4 - v5 * r6;
+  d[0] = v1 * r3 - 7.f * r6 * v2 + 11.f * r6 * v3;
+  d[1] = -v2 * r6 + 5.f * r6 * v3 + v4 * r3;
+  d[2] = v3 * r3 + 5.f * r6 * v4 - v5 * r6;
+}
+__device__ __forceinline__ float weno5_mean(float v1, float v2, float v3, float v4, float v5, const float d[3]) {
+  const float eps = 1e-6f;
   const float b1 = v1 - 2.f * v2 + v3, c1 = v1 - 4.f * v2 + 3.f * v3;
   const float b2 = v2 - 2.f * v3 + v4, c2 = v2 - v4;
   const float b3 = v3 - 2.f * v4 + v5, c3 = 3.f * v3 - 4.f * v4 + v5;
@@ -726,7 +787,32 @@ __device__ __forceinline__ float weno5(float v1, float v2, float v3, float v4, f
   const float t3 = 13.f / 12.f * b3 * b3 + 0.25f * c3 * c3 + eps;
   const float q1 = t1 * t1, q2 = t2 * t2, q3 = t3 * t3;
   const float a1 = 0.1f * q2 * q3, a2 = 0.6f * q1 * q3, a3 = 0.3f * q1 * q2;
-  return (a1 * d1 + a2 * d2 + a3 * d3) / (a1 + a2 + a3);
+  return (a1 * d[0] + a2 * d[1] + a3 * d[2]) / (a1 + a2 + a3);
+}
+
+// Godunov's |grad phi|^2 along one axis from the seven values v at offsets -3..+3, for the
+// sign of s0: max(max(d-, 0)^2, min(d+, 0)^2) for s0 > 0, the other signs otherwise, with the
+// left- and right-biased derivatives d-, d+.  A derivative is a weighted mean of its
+// candidates: where all three have the sign that Godunov's choice drops, the side's square
+// is exactly zero and its weights are not formed (one side always in smooth regions).
+__device__ __forceinline__ float godunov_axis(const float v[7], float s0) {
+  const float D0 = v[1] - v[0], D1 = v[2] - v[1], D2 = v[3] - v[2], D3 = v[4] - v[3], D4 = v[5] - v[4], D5 = v[6] - v[5];
+  float m[3], p[3];
+  weno5_candidates(D0, D1, D2, D3, D4, m);
+  weno5_candidates(D5, D4, D3, D2, D1, p);
+  const bool pos = s0 > 0.f;
+  const bool um = pos ? fmaxf(fmaxf(m[0], m[1]), m[2]) > 0.f : fminf(fminf(m[0], m[1]), m[2]) < 0.f;
+  const bool up = pos ? fminf(fminf(p[0], p[1]), p[2]) < 0.f : fmaxf(fmaxf(p[0], p[1]), p[2]) > 0.f;
+  float gm = 0.f, gp = 0.f;
+  if (um) {
+    const float dm = weno5_mean(D0, D1, D2, D3, D4, m), d = pos ? fmaxf(dm, 0.f) : fminf(dm, 0.f);
+    gm = d * d;
+  }
+  if (up) {
+    const float dp = weno5_mean(D5, D4, D3, D2, D1, p), d = pos ? fminf(dp, 0.f) : fmaxf(dp, 0.f);
+    gp = d * d;
+  }
+  return fmaxf(gm, gp);
 }
 
 // TVD-RK3 stage of phi_tau = -S(phi0)(|grad phi|_G - 1) on band cells that are not frozen.
@@ -749,12 +835,7 @@ __device__ __forceinline__ void d_reinit_stage(const Ctx &C, BlockShape S, int g
     for (int a = 0; a < D; ++a) {
       float v[7];
       gather7f<D>(C, L, S, gb, pin, true, x, y, z, cl, a, v);
-      const float dm = weno5(v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3], v[5] - v[4]);
-      const float dp = weno5(v[6] - v[5], v[5] - v[4], v[4] - v[3], v[3] - v[2], v[2] - v[1]);
-      float ga;
-      if (s0 > 0.f) ga = fmaxf(fmaxf(dm, 0.f) * fmaxf(dm, 0.f), fminf(dp, 0.f) * fminf(dp, 0.f));
-      else ga = fmaxf(fminf(dm, 0.f) * fminf(dm, 0.f), fmaxf(dp, 0.f) * fmaxf(dp, 0.f));
-      g2 += ga;
+      g2 += godunov_axis(v, s0);
     }
     const float rhs = L.dtau_reinit * (-s0 * (sqrtf(g2) - 1.0f));
     const float p0 = C.phi[fc];
@@ -770,31 +851,15 @@ __global__ void k_reinit_stage(Ctx C, BlockShape S, int glevel, int stage) {
 }
 
 // ------------------------------------------------------------------ forward passes on mirrored stage arrays
-// The forward step keeps the stage arrays equal to the committed fields at every
-// finest cell outside the band when a level-set update starts: p1 = p2 = phi and
-// ut1 = ut2 = ut0.  Band cells restore this at the end of each update (u~ in the
-// first transport stage, which also commits the extension; phi in the phase pass
-// of the classification), and the host copies the arrays in full after creation
-// and after every restore of phi or u~.  A stencil point then reads the stage
-// array wherever it lies, so the passes below need no band or frozen-cell lookups;
-// frozen cells of the reinitialisation write phi into the stage arrays their
-// neighbours read.  The arithmetic and its order are those of the passes above,
-// so the results are the same bit for bit.
-
-// Resident CTAs of 512 threads per SM the mirrored stage kernels are compiled for (their
-// registers capped to fit): the passes are latency-bound, so more warps in flight pay.
-#ifndef LSB_LS_MINB
-#define LSB_LS_MINB 3
-#endif
-#ifndef LSB_EF_MINB
-#define LSB_EF_MINB LSB_LS_MINB  // the first extension sweep
-#endif
-#ifndef LSB_ADV_MINB
-#define LSB_ADV_MINB LSB_LS_MINB  // the transport stages
-#endif
-#ifndef LSB_RE_MINB
-#define LSB_RE_MINB LSB_LS_MINB  // the reinitialisation stages
-#endif
+// The forward step keeps the stage arrays equal to the committed fields at every finest
+// cell outside the band when a level-set update starts: p1 = p2 = phi, and both sweep
+// buffers = ut0.  Band cells restore this during each update (u~ in the first transport
+// stage, which also commits the extension; phi in the phase pass of the classification),
+// and the host fills the arrays in full after creation and after every restore of phi or
+// u~.  A stencil point then reads the stage array wherever it lies, so the passes below
+// need no band or frozen-cell lookups; frozen cells of the reinitialisation write phi into
+// the stage arrays their neighbours read.  The arithmetic and its order are those of the
+// passes above, so the results are the same bit for bit.
 
 // seven values of the stage array along axis a at offsets -3..+3 (clamped or
 // wrapped at the box faces like gather7)
@@ -815,206 +880,745 @@ __device__ __forceinline__ void gather7m(const LevelDev &L, const float *__restr
   }
 }
 
-// First extension sweep of a step (mode 2 of d_ext_iter): sweep from uin = ut0 and
-// store the plan (S(phi) n, upwind sides, interface and box-boundary bits).
+// The forward step's sweep buffers hold u~ interleaved (a vector per cell, so that a
+// neighbour is one load): two floats in 2D, four in 3D.
+template <int D> struct UVec;
+template <> struct UVec<2> { using T = float2; };
+template <> struct UVec<3> { using T = float4; };
+__device__ __forceinline__ void u_get(const float2 &v, float u[3]) { u[0] = v.x; u[1] = v.y; }
+__device__ __forceinline__ void u_get(const float4 &v, float u[3]) { u[0] = v.x; u[1] = v.y; u[2] = v.z; }
+__device__ __forceinline__ void u_put(float2 &v, const float u[3], float) { v = make_float2(u[0], u[1]); }
+__device__ __forceinline__ void u_put(float4 &v, const float u[3], float w) { v = make_float4(u[0], u[1], u[2], w); }
+
+// First extension sweep at one band cell (mode 2 of d_ext_iter): sweep from ut0 into the
+// buffer uout and store the plan (S(phi) n, upwind sides, interface and box-boundary bits).
 template <int D>
-// turn: also start the classification's counters (the band count into the previous-band
-// slot, the other slots but the band count to zero; no pass between here and the
-// classification reads them).
-__global__ void __launch_bounds__(512, LSB_EF_MINB) k_ext_first(Ctx C, BlockShape S, int glevel, const float *__restrict__ uin,
-                            float *__restrict__ uout, int turn) {
-  LSB_GRID_WAIT();
-  const int nl = min(C.counters[glevel * NCOUNT + 3], C.band_cap);
-  if (turn && blockIdx.x == 0 && threadIdx.x == 0) {
-    int *cnt = C.counters + glevel * NCOUNT;
-    cnt[5] = cnt[3];
-    cnt[0] = cnt[1] = cnt[2] = cnt[4] = 0;
+__device__ __forceinline__ void ext_first_cell(const Ctx &C, const LevelDev &L, int x, int y, int z,
+                                               typename UVec<D>::T *uout) {
+  const long long fo = L.fine_off, NF = C.nfine;
+  const long long c = cidx(L, x, y, z);
+  float u0[3];
+  for (int b = 0; b < D; ++b) u0[b] = C.ut0[b * NF + fo + c];
+  if (C.tag[L.cell_off + c] & TAG_IFACE) {
+    u_put(uout[fo + c], u0, 0.f);
+    C.plan_f[fo + c] = 64;
+    return;
   }
-  const long long NF = C.nfine;
-  // the next entry of the band list is loaded while this one is processed
-  const int4 *info = C.band_info + (long long)glevel * C.band_cap;
-  int4 next = blockIdx.x < nl ? __ldg(info + blockIdx.x) : make_int4(0, 0, 0, 0);
-  for (int w = blockIdx.x; w < nl; w += gridDim.x) {
-    const int4 bi = next;
-    if (w + gridDim.x < nl) next = __ldg(info + w + gridDim.x);
-    int x, y, z;
-    const LevelDev &L = band_cell_at(C, S, bi, threadIdx.x, x, y, z);
-    if (!L.ls_active) continue;
-    if (x >= L.n[0] || y >= L.n[1] || z >= L.n[2]) continue;
-    const long long fo = L.fine_off;
-    const long long c = cidx(L, x, y, z);
-    if (C.tag[L.cell_off + c] & TAG_IFACE) {
-      for (int a = 0; a < D; ++a) uout[a * NF + fo + c] = uin[a * NF + fo + c];
-      C.plan_f[fo + c] = 64;
-      continue;
+  const int crd[3] = {x, y, z};
+  const int str[3] = {1, L.p[0], L.p[0] * L.p[1]};
+  bool inner = true;
+  for (int a = 0; a < D; ++a) inner = inner && crd[a] >= 1 && crd[a] + 1 < L.n[a];
+  const float *phiL = C.phi + fo;
+  float nvec[3], gm = 0.f;
+  uint8_t pf = inner ? 0 : 128;
+  for (int a = 0; a < D; ++a) {
+    if (inner) {
+      nvec[a] = 0.5f * (phiL[(unsigned)c + str[a]] - phiL[(unsigned)c - str[a]]);
+    } else {
+      int p[3] = {x, y, z}, m[3] = {x, y, z};
+      p[a] = clampwrap(L, a, crd[a] + 1);
+      m[a] = clampwrap(L, a, crd[a] - 1);
+      nvec[a] = 0.5f * (phiL[cidx(L, p[0], p[1], p[2])] - phiL[cidx(L, m[0], m[1], m[2])]);
     }
-    const int crd[3] = {x, y, z};
-    const int str[3] = {1, L.p[0], L.p[0] * L.p[1]};
-    bool inner = true;
-    for (int a = 0; a < D; ++a) inner = inner && crd[a] >= 1 && crd[a] + 1 < L.n[a];
-    const float *phiL = C.phi + fo;
-    float nvec[3], gm = 0.f;
-    uint8_t pf = inner ? 0 : 128;
-    for (int a = 0; a < D; ++a) {
-      if (inner) {
-        nvec[a] = 0.5f * (phiL[(unsigned)c + str[a]] - phiL[(unsigned)c - str[a]]);
-      } else {
-        int p[3] = {x, y, z}, m[3] = {x, y, z};
-        p[a] = clampwrap(L, a, crd[a] + 1);
-        m[a] = clampwrap(L, a, crd[a] - 1);
-        nvec[a] = 0.5f * (phiL[cidx(L, p[0], p[1], p[2])] - phiL[cidx(L, m[0], m[1], m[2])]);
-      }
-      gm += nvec[a] * nvec[a];
+    gm += nvec[a] * nvec[a];
+  }
+  gm = sqrtf(gm);
+  const float ph = phiL[c];
+  const float sg = ph / sqrtf(ph * ph + 1.0f);
+  float acc[3] = {0.f, 0.f, 0.f};
+  for (int a = 0; a < D; ++a) {
+    const float va = gm > 0.f ? sg * nvec[a] / gm : 0.f;
+    const int dir = va > 0.f ? -1 : 1;
+    long long cn;
+    if (inner) {
+      cn = c + dir * str[a];
+    } else {
+      int nb[3] = {x, y, z};
+      nb[a] = clampwrap(L, a, crd[a] + dir);
+      cn = cidx(L, nb[0], nb[1], nb[2]);
     }
-    gm = sqrtf(gm);
-    const float ph = phiL[c];
-    const float sg = ph / sqrtf(ph * ph + 1.0f);
-    float u0[3];
-    for (int b = 0; b < D; ++b) u0[b] = uin[b * NF + fo + c];
+    for (int b = 0; b < D; ++b) {
+      const float un = C.ut0[b * NF + fo + cn];
+      acc[b] += va * (va > 0.f ? (u0[b] - un) : (un - u0[b]));
+    }
+    C.plan_v[a * NF + fo + c] = va;
+    pf |= (dir < 0 ? 1 : 0) << a;
+  }
+  for (int b = 0; b < D; ++b) u0[b] = u0[b] - L.dtau_ext * acc[b];
+  u_put(uout[fo + c], u0, 0.f);
+  C.plan_f[fo + c] = pf;
+}
+
+// A later extension sweep at one band cell, from the stored plan.
+template <int D>
+__device__ __forceinline__ void ext_sweep_cell(const Ctx &C, const LevelDev &L, int x, int y, int z,
+                                               const typename UVec<D>::T *uin, typename UVec<D>::T *uout) {
+  const long long NF = C.nfine, c = cidx(L, x, y, z);
+  const typename UVec<D>::T *ui = uin + L.fine_off;
+  const uint8_t pf = C.plan_f[L.fine_off + c];
+  float u0[3];
+  u_get(ui[c], u0);
+  if (!(pf & 64)) {
     float acc[3] = {0.f, 0.f, 0.f};
     for (int a = 0; a < D; ++a) {
-      const float va = gm > 0.f ? sg * nvec[a] / gm : 0.f;
-      const int dir = va > 0.f ? -1 : 1;
+      const float va = C.plan_v[a * NF + L.fine_off + c];
+      const int dir = (pf >> a) & 1 ? -1 : 1;
       long long cn;
-      if (inner) {
-        cn = c + dir * str[a];
-      } else {
+      if (pf & 128) {  // box-boundary cell: the neighbour clamped or wrapped
         int nb[3] = {x, y, z};
-        nb[a] = clampwrap(L, a, crd[a] + dir);
+        nb[a] = clampwrap(L, a, nb[a] + dir);
         cn = cidx(L, nb[0], nb[1], nb[2]);
+      } else {
+        cn = c + dir * (a == 0 ? 1LL : (a == 1 ? (long long)L.p[0] : (long long)L.p[0] * L.p[1]));
       }
-      for (int b = 0; b < D; ++b) {
-        const float un = uin[b * NF + fo + cn];
-        acc[b] += va * (va > 0.f ? (u0[b] - un) : (un - u0[b]));
-      }
-      C.plan_v[a * NF + fo + c] = va;
-      pf |= (dir < 0 ? 1 : 0) << a;
+      float un[3];
+      u_get(ui[cn], un);
+      for (int b = 0; b < D; ++b) acc[b] += va * (va > 0.f ? (u0[b] - un[b]) : (un[b] - u0[b]));
     }
-    for (int b = 0; b < D; ++b) uout[b * NF + fo + c] = u0[b] - L.dtau_ext * acc[b];
-    C.plan_f[fo + c] = pf;
+    for (int b = 0; b < D; ++b) u0[b] = u0[b] - L.dtau_ext * acc[b];
   }
+  u_put(uout[L.fine_off + c], u0, 0.f);
 }
 
-// TVD-RK3 transport stage (as d_adv_stage).  Stage 1 takes u~ from the last
-// extension sweep (ufin) and commits it to ut0, ut1 and ut2 at the cell.
+// TVD-RK3 transport stage at one band cell (as d_adv_stage).  Stage 1 takes u~ from the
+// last extension sweep (ufin; nullptr: ut0, no sweeps) and commits it to ut0 and both
+// sweep buffers at the cell.
 template <int D>
-__global__ void __launch_bounds__(512, LSB_ADV_MINB) k_adv_mirror(Ctx C, BlockShape S, int glevel, int stage,
-                                                                 const float *__restrict__ ufin) {
-  LSB_GRID_WAIT();
-  const int nl = min(C.counters[glevel * NCOUNT + 3], C.band_cap);
+__device__ __forceinline__ void adv_cell(const Ctx &C, const LevelDev &L, int x, int y, int z, int stage,
+                                         const typename UVec<D>::T *ufin, typename UVec<D>::T *ub1,
+                                         typename UVec<D>::T *ub2) {
   const float *pin = stage == 1 ? C.phi : (stage == 2 ? C.p1 : C.p2);
   const long long NF = C.nfine;
-  // the next entry of the band list is loaded while this one is processed
-  const int4 *info = C.band_info + (long long)glevel * C.band_cap;
-  int4 next = blockIdx.x < nl ? __ldg(info + blockIdx.x) : make_int4(0, 0, 0, 0);
-  for (int w = blockIdx.x; w < nl; w += gridDim.x) {
-    const int4 bi = next;
-    if (w + gridDim.x < nl) next = __ldg(info + w + gridDim.x);
-    int x, y, z;
-    const LevelDev &L = band_cell_at(C, S, bi, threadIdx.x, x, y, z);
-    if (!L.ls_active) continue;
-    if (x >= L.n[0] || y >= L.n[1] || z >= L.n[2]) continue;
-    const unsigned c = (unsigned)cidx(L, x, y, z);
-    const long long fc = L.fine_off + c;
-    float ua[3];
-    if (stage == 1) {
-      for (int a = 0; a < D; ++a) {
-        const float u = ufin[a * NF + fc];
-        ua[a] = u;
-        C.ut0[a * NF + fc] = u;
-        C.ut1[a * NF + fc] = u;
-        C.ut2[a * NF + fc] = u;
-      }
-    } else {
-      for (int a = 0; a < D; ++a) ua[a] = C.ut0[a * NF + fc];
-    }
-    const float *pinL = pin + L.fine_off;
-    float rhs = 0.f;
-    for (int a = 0; a < D; ++a) {
-      float v[7];
-      gather7m(L, pinL, x, y, z, c, a, v);
-      rhs -= ua[a] * (ua[a] >= 0.f ? d5m(v) : d5p(v));
-    }
-    const float p0 = C.phi[fc];
-    if (stage == 1) C.p1[fc] = p0 + rhs;
-    else if (stage == 2) C.p2[fc] = 0.75f * p0 + 0.25f * (C.p1[fc] + rhs);
-    else C.phi[fc] = p0 / 3.0f + (2.0f / 3.0f) * (C.p2[fc] + rhs);
+  const unsigned c = (unsigned)cidx(L, x, y, z);
+  const long long fc = L.fine_off + c;
+  float ua[3];
+  if (stage == 1 && ufin) u_get(ufin[fc], ua);
+  else
+    for (int a = 0; a < D; ++a) ua[a] = C.ut0[a * NF + fc];
+  if (stage == 1) {
+    for (int a = 0; a < D; ++a) C.ut0[a * NF + fc] = ua[a];
+    u_put(ub1[fc], ua, 0.f);
+    u_put(ub2[fc], ua, 0.f);
   }
+  const float *pinL = pin + L.fine_off;
+  float rhs = 0.f;
+  for (int a = 0; a < D; ++a) {
+    float v[7];
+    gather7m(L, pinL, x, y, z, c, a, v);
+    rhs -= ua[a] * (ua[a] >= 0.f ? d5m(v) : d5p(v));
+  }
+  const float p0 = C.phi[fc];
+  if (stage == 1) C.p1[fc] = p0 + rhs;
+  else if (stage == 2) C.p2[fc] = 0.75f * p0 + 0.25f * (C.p1[fc] + rhs);
+  else C.phi[fc] = p0 / 3.0f + (2.0f / 3.0f) * (C.p2[fc] + rhs);
 }
 
-// Reinitialisation stage (as d_reinit_stage); with prep set (first stage of the first
-// pseudo step) it also finds the frozen cells and S(phi0) as d_reinit_prep does.
-// Frozen cells leave phi as it is and write it into the stage array of stages 1, 2.
+// Whether the level set changes sign between a cell (value p0, at phi) and a lattice neighbour.
 template <int Q>
-__global__ void __launch_bounds__(512, LSB_RE_MINB) k_reinit_mirror(Ctx C, BlockShape S, int glevel, int stage,
-                                                                    int prep) {
-  LSB_GRID_WAIT();
+__device__ __forceinline__ bool sign_change(const float *phi, float p0, const NearOff &o) {
   using LT = Lat<Q>;
-  constexpr int D = LT::D;
-  const int nl = min(C.counters[glevel * NCOUNT + 3], C.band_cap);
-  const float *pin = stage == 1 ? C.phi : (stage == 2 ? C.p1 : C.p2);
-  // the next entry of the band list is loaded while this one is processed
-  const int4 *info = C.band_info + (long long)glevel * C.band_cap;
-  int4 next = blockIdx.x < nl ? __ldg(info + blockIdx.x) : make_int4(0, 0, 0, 0);
-  for (int w = blockIdx.x; w < nl; w += gridDim.x) {
-    const int4 bi = next;
-    if (w + gridDim.x < nl) next = __ldg(info + w + gridDim.x);
-    int x, y, z;
-    const LevelDev &L = band_cell_at(C, S, bi, threadIdx.x, x, y, z);
-    if (!L.ls_active) continue;
-    if (x >= L.n[0] || y >= L.n[1] || z >= L.n[2]) continue;
-    const unsigned cl = (unsigned)cidx(L, x, y, z);
-    const long long fc = L.fine_off + cl;
-    const float p0 = C.phi[fc];
-    bool fr;
-    float s0;
-    if (prep) {
-      const bool g = p0 >= 0.f;
-      fr = false;
-      const bool inner = x >= 1 && x + 1 < L.n[0] && y >= 1 && y + 1 < L.n[1] && (D == 2 || (z >= 1 && z + 1 < L.n[2]));
-      if (inner) {
-        const int q0 = L.p[0], q01 = L.p[0] * L.p[1];
+  const bool g = p0 >= 0.f;
+  bool fr = false;
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-          if (i == LT::REST) continue;
-          if ((C.phi[fc + LT::cx(i) + LT::cy(i) * q0 + LT::cz(i) * q01] >= 0.f) != g) fr = true;
+  for (int i = 0; i < Q; ++i) {
+    if (i == LT::REST) continue;
+    bool out;
+    const int off = off_to(o, LT::cx(i), LT::cy(i), LT::cz(i), out);
+    if ((phi[out ? 0 : off] >= 0.f) != g) fr = true;
+  }
+  return fr;
+}
+
+// The same for a cell with every neighbour in the box.
+template <int Q>
+__device__ __forceinline__ bool sign_change_inner(const float *phi, float p0, long long q0, long long q01) {
+  using LT = Lat<Q>;
+  const bool g = p0 >= 0.f;
+  bool fr = false;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    if (i == LT::REST) continue;
+    if ((phi[LT::cx(i) + LT::cy(i) * q0 + LT::cz(i) * q01] >= 0.f) != g) fr = true;
+  }
+  return fr;
+}
+
+// Reinitialisation stage at one band cell (as d_reinit_stage); with prep set (first stage
+// of the first pseudo step) it also finds the frozen cells and S(phi0) as d_reinit_prep
+// does.  Frozen cells leave phi as it is and write it into the stage array of stages 1, 2.
+template <int Q>
+__device__ __forceinline__ void reinit_cell(const Ctx &C, const LevelDev &L, int x, int y, int z, int stage, int prep) {
+  constexpr int D = Lat<Q>::D;
+  const float *pin = stage == 1 ? C.phi : (stage == 2 ? C.p1 : C.p2);
+  const unsigned cl = (unsigned)cidx(L, x, y, z);
+  const long long fc = L.fine_off + cl;
+  const float p0 = C.phi[fc];
+  bool fr;
+  float s0;
+  if (prep) {
+    const int crd[3] = {x, y, z};
+    fr = sign_change<Q>(C.phi + fc, p0, near_off<D>(crd, L.n, per_mask(L), (unsigned)L.p[0], (unsigned)(L.p[0] * L.p[1])));
+    s0 = p0 / sqrtf(p0 * p0 + 1.0f);
+    C.frozen[fc] = fr ? 1 : 0;
+    C.s0[fc] = s0;
+  } else {
+    fr = C.frozen[fc] != 0;
+    s0 = C.s0[fc];
+  }
+  if (fr) {
+    if (stage == 1) C.p1[fc] = p0;
+    else if (stage == 2) C.p2[fc] = p0;
+    return;
+  }
+  const float *pinL = pin + L.fine_off;
+  float g2 = 0.f;
+  for (int a = 0; a < D; ++a) {
+    float v[7];
+    gather7m(L, pinL, x, y, z, cl, a, v);
+    g2 += godunov_axis(v, s0);
+  }
+  const float rhs = L.dtau_reinit * (-s0 * (sqrtf(g2) - 1.0f));
+  if (stage == 1) C.p1[fc] = p0 + rhs;
+  else if (stage == 2) C.p2[fc] = 0.75f * p0 + 0.25f * (C.p1[fc] + rhs);
+  else C.phi[fc] = p0 / 3.0f + (2.0f / 3.0f) * (C.p2[fc] + rhs);
+}
+
+// ------------------------------------------------------------------ the level-set update in one launch
+// Everything the level set does in a finest sub-step after the interface pass, in one
+// launch: n_ext extension sweeps, three transport stages, the reinitialisation, and the
+// phase and cut-link passes of the classification (16 passes by default), with a barrier
+// between passes.  As launches of their own the passes are bound by their chains: ~1 us
+// for the launch, then band count, band entry, level descriptor, plan, neighbours, one L2
+// round trip each.  Here a CTA's cells stay its own for all passes: each thread sets up
+// its band cells once (slots) and keeps their offsets, flags, extension velocity and
+// current values in shared memory, so a pass is one round of neighbour loads and stores.
+//
+// MODE 0: the grid is one thread-block cluster and the barrier is the cluster's.
+// MODE 1: a cooperative launch; the barrier counts arrivals in bar[0] (one release-add per
+// CTA, polled with an iteration limit; a barrier that gives up sets ERR_TIMEOUT and ends
+// the CTA).  bar[1] counts CTAs that left: the last one clears both words for the next launch.
+// Measured per pass, one store and two neighbour loads per thread: a launch of its own in a
+// captured graph 3.8 us, grid barrier 1.4 us (152 CTAs), cluster barrier 0.6 - 1.0 us
+// (16 CTAs of 256 - 1024 threads).
+//
+// Slots: a sweep of the grid covers gridDim.x * blockDim.x cells = GB whole band blocks
+// (blockDim.x is a multiple of the block's cells); slot k of a thread is its cell in the
+// k-th such group.  The first kcap slots live in shared memory; cells beyond (the band grew
+// since the launch was sized) take the passes' per-cell functions above, with the plan in
+// global memory.  The arithmetic and its order are those functions', so the results are
+// the same bit for bit.  No load here may go through the read-only path: every array
+// changes during the launch.
+struct __align__(16) LsfGeo {  // what the passes need of a level descriptor
+  int p0, p01;          // strides
+  float dte, dtr;
+  int n[3];
+  unsigned per;         // periodic axes; bit 3: the case's level set moves
+  long long tag_delta;  // tag index of a cell - its finest-level index
+  unsigned fo;          // offset in the finest-level arrays
+};
+__device__ __forceinline__ LsfGeo lsf_geo(const LevelDev &L) {
+  LsfGeo g;
+  g.p0 = L.p[0];
+  g.p01 = L.p[0] * L.p[1];
+  g.fo = (unsigned)L.fine_off;
+  for (int a = 0; a < 3; ++a) g.n[a] = L.n[a];
+  g.per = per_mask(L) | (L.ls_active ? 8u : 0u);
+  g.dte = L.dtau_ext;
+  g.dtr = L.dtau_reinit;
+  g.tag_delta = L.cell_off - L.fine_off;
+  return g;
+}
+constexpr int kLsfGeo = 192;              // level descriptors with an entry in shared memory
+constexpr unsigned kLsfLimit = 1u << 23;  // polls of a grid barrier before it gives up (seconds)
+enum : unsigned {  // slot flags
+  SL_NEAR = 1,      // << axis: a stencil point three cells along the axis lies outside the box
+  SL_IFACE = 8,     // interface cell: keeps its u~
+  SL_EDGE = 16,     // a lattice neighbour lies outside the box
+  SL_CELL = 32,     // a cell of the box
+  SL_LIVE = 64,     // ... of a case whose level set moves
+  SL_FROZEN = 128,  // reinitialisation: frozen
+  SL_DIST = 8,      // 12 bits from here: lsf_dist
+  SL_LD = 20        // the bits above: the cell's level descriptor
+};
+constexpr int kLsfMaxLd = 1 << (32 - SL_LD);  // more level descriptors: no slots (kcap 0)
+// How far a cell lies from the box faces, up to three cells: per axis 2 bits towards the low
+// face, 2 towards the high one.
+template <int D>
+__device__ __forceinline__ unsigned lsf_dist(const int crd[3], const int n[3]) {
+  unsigned d = 0;
+#pragma unroll
+  for (int a = 0; a < D; ++a) d |= (unsigned)(min(crd[a], 3) | (min(n[a] - 1 - crd[a], 3) << 2)) << (4 * a);
+  return d;
+}
+// The step d along axis a kept in the box: clamped at walls, wrapped on periodic axes.
+__device__ __forceinline__ int lsf_step(const LsfGeo &g, unsigned dist, int a, int d) {
+  const int lo = (int)((dist >> (4 * a)) & 3u), hi = (int)((dist >> (4 * a + 2)) & 3u);
+  if ((g.per >> a) & 1u) {
+    // lo, hi are exact where d reaches past them (|d| <= 3)
+    if (d < -lo) {
+      do d += g.n[a]; while (d < -lo);
+    } else if (d > hi) {
+      do d -= g.n[a]; while (d > hi);
+    }
+    return d;
+  }
+  return min(max(d, -lo), hi);
+}
+// The offsets of near_off from the distances.
+template <int D>
+__device__ __forceinline__ NearOff lsf_near(const LsfGeo &g, unsigned dist) {
+  int crd[3] = {0, 0, 0}, n[3] = {1, 1, 1};
+  // stands in for the coordinate: only its being 0 or n - 1 counts, beside n itself
+#pragma unroll
+  for (int a = 0; a < D; ++a) {
+    const unsigned lo = (dist >> (4 * a)) & 3u, hi = (dist >> (4 * a + 2)) & 3u;
+    n[a] = g.n[a];
+    crd[a] = lo == 0 ? 0 : (hi == 0 ? n[a] - 1 : 1);
+  }
+  return near_off<D>(crd, n, g.per, (unsigned)g.p0, (unsigned)g.p01);
+}
+
+template <int MODE>
+__device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err) {
+  if (MODE == 0) {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+    return true;
+  }
+  __shared__ int gave_up;
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    gave_up = 0;
+    unsigned v, spins = 0;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (++spins > kLsfLimit) {
+        gave_up = 1;
+        atomicOr(err, ERR_TIMEOUT);
+        break;
+      }
+    } while ((int)(v - target) < 0);
+  }
+  __syncthreads();
+  return gave_up == 0;
+}
+
+// A slot in shared memory: kcap planes of 1024 threads of each field (constant strides, so
+// a slot's fields sit at constant offsets).  v: S(phi) n during the sweeps, then phi and the
+// last stage value in its first two words; u: u~, then S(phi0) of the reinitialisation in
+// its first word.
+template <int D> struct LsfSlot {
+  using V = typename UVec<D>::T;
+  V v[1024], u[1024];
+  unsigned fc[1024], fl[1024];  // finest-level index, flags
+};
+template <int Q, int MODE>
+__global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
+                                                            int kcap, unsigned *bar) {
+  constexpr int D = Lat<Q>::D;
+  using V = typename UVec<D>::T;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  extern __shared__ __align__(16) unsigned char lsf_sm[];
+  __shared__ LsfGeo geo[kLsfGeo];
+  __shared__ int hot[32];  // link pass: a cut link in each of the CTA's blocks
+  LsfSlot<D> *const SM = reinterpret_cast<LsfSlot<D> *>(lsf_sm);
+  const int T = blockDim.x, tid = threadIdx.x;
+  const int lgnt = S.lg[0] + S.lg[1] + S.lg[2];
+  const int t = tid & ((1 << lgnt) - 1);
+  const int GB = (int)((gridDim.x * (unsigned)T) >> lgnt);         // band blocks per sweep of the grid
+  const int w0 = (int)((blockIdx.x * (unsigned)T + tid) >> lgnt);  // this thread's block in the first
+  const long long NF = C.nfine;
+  V *const ub1 = reinterpret_cast<V *>(C.ut1), *const ub2 = reinterpret_cast<V *>(C.ut2);
+  int *cnt = C.counters + glevel * NCOUNT;
+  const int4 *info = C.band_info + (long long)glevel * C.band_cap;
+  // the first band entry is fetched beside the band count, not after it
+  int4 bi = info[min(w0, C.band_cap - 1)];
+  const int nl = min(cnt[3], C.band_cap);
+  const int kn = (nl + GB - 1) / GB, ks = min(kn, kcap);
+  unsigned target = 0;
+  for (int i = tid; i < min(nld, kLsfGeo); i += T) geo[i] = lsf_geo(C.lds[i]);
+  auto geo_of = [&](unsigned ld) { return ld < (unsigned)kLsfGeo ? geo[ld] : lsf_geo(C.lds[ld]); };
+  // a cell beyond the slots: its level descriptor and coordinates (ok: a live cell of the box)
+  auto beyond = [&](int k, int &x, int &y, int &z, bool &ok) -> const LevelDev & {
+    const int w = w0 + k * GB;
+    ok = w < nl;
+    const LevelDev &L = band_cell_at(C, S, ok ? info[w] : info[0], t, x, y, z);
+    ok = ok && L.ls_active && x < L.n[0] && y < L.n[1] && z < L.n[2];
+    return L;
+  };
+  auto leave = [&]() {
+    if (MODE == 1 && tid == 0 && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+      bar[0] = 0;
+      bar[1] = 0;
+    }
+  };
+  __syncthreads();
+  // ---- slots, and the first extension sweep with the plan
+  for (int k = 0; k < ks; ++k) {
+    const int w = w0 + k * GB;
+    const int4 b = bi;
+    if (w + GB < nl) bi = info[w + GB];
+    unsigned fl = 0;
+    if (w < nl) {
+      const LsfGeo g = geo_of((unsigned)b.x);
+      const int crd[3] = {(b.y << S.lg[0]) + (t & (S.bs[0] - 1)), (b.z << S.lg[1]) + ((t >> S.lg[0]) & (S.bs[1] - 1)),
+                          (b.w << S.lg[2]) + (t >> (S.lg[0] + S.lg[1]))};
+      if (crd[0] < g.n[0] && crd[1] < g.n[1] && crd[2] < g.n[2]) {
+        const unsigned fc = g.fo + (unsigned)crd[0] + (unsigned)(g.p0 * crd[1] + g.p01 * crd[2]);
+        const unsigned dist = lsf_dist<D>(crd, g.n);
+        fl = SL_CELL | ((g.per & 8u) ? SL_LIVE : 0u) | (dist << SL_DIST) | ((unsigned)b.x << SL_LD);
+        bool edge = false;
+#pragma unroll
+        for (int a = 0; a < D; ++a) {
+          edge = edge || crd[a] < 1 || crd[a] + 1 >= g.n[a];
+          if (crd[a] < 3 || crd[a] + 3 >= g.n[a]) fl |= SL_NEAR << a;
         }
-      } else {
-        for (int i = 0; i < Q; ++i) {
-          if (i == LT::REST) continue;
-          int tx = x + LT::cx(i), ty = y + LT::cy(i), tz = z + LT::cz(i);
-          if (!(wrap(L, 0, tx) && wrap(L, 1, ty) && (D == 2 || wrap(L, 2, tz)))) continue;
-          if ((C.phi[L.fine_off + cidx(L, tx, ty, tz)] >= 0.f) != g) fr = true;
+        if (edge) fl |= SL_EDGE;
+        SM[k].fc[tid] = fc;
+        if (fl & SL_LIVE) {
+          // one round of loads: the cell's tag, phi around it, its u~
+          const uint8_t tg = C.tag[(long long)fc + g.tag_delta];
+          int om[3], op[3];
+          float u0[3] = {0.f, 0.f, 0.f}, pm[3], pp[3], va[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+          for (int a = 0; a < D; ++a) {
+            const int str = a == 0 ? 1 : (a == 1 ? g.p0 : g.p01);
+            om[a] = -str;
+            op[a] = str;
+            if (edge) {
+              om[a] = lsf_step(g, dist, a, -1) * str;
+              op[a] = lsf_step(g, dist, a, 1) * str;
+            }
+            pm[a] = C.phi[fc + (unsigned)om[a]];
+            pp[a] = C.phi[fc + (unsigned)op[a]];
+            u0[a] = C.ut0[a * NF + fc];
+          }
+          const float ph = C.phi[fc];
+          if (tg & TAG_IFACE) {
+            fl |= SL_IFACE;
+            if (n_ext > 0) u_put(ub1[fc], u0, 0.f);
+          } else if (n_ext > 0) {
+            float nvec[3], gm = 0.f, un[D][3];
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+              nvec[a] = 0.5f * (pp[a] - pm[a]);
+              gm += nvec[a] * nvec[a];
+            }
+            gm = sqrtf(gm);
+            const float sg = ph / sqrtf(ph * ph + 1.0f);
+#pragma unroll
+            for (int a = 0; a < D; ++a) {
+              va[a] = gm > 0.f ? sg * nvec[a] / gm : 0.f;
+              const unsigned cn = fc + (unsigned)(va[a] > 0.f ? om[a] : op[a]);
+#pragma unroll
+              for (int b = 0; b < D; ++b) un[a][b] = C.ut0[b * NF + cn];
+            }
+            float acc[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+            for (int a = 0; a < D; ++a)
+#pragma unroll
+              for (int b = 0; b < D; ++b) acc[b] += va[a] * (va[a] > 0.f ? (u0[b] - un[a][b]) : (un[a][b] - u0[b]));
+#pragma unroll
+            for (int b = 0; b < D; ++b) u0[b] = u0[b] - g.dte * acc[b];
+            u_put(ub1[fc], u0, 0.f);
+          }
+          u_put(SM[k].v[tid], va, 0.f);
+          u_put(SM[k].u[tid], u0, 0.f);
         }
       }
-      s0 = p0 / sqrtf(p0 * p0 + 1.0f);
-      C.frozen[fc] = fr ? 1 : 0;
-      C.s0[fc] = s0;
+    }
+    SM[k].fl[tid] = fl;
+  }
+  for (int k = ks; k < kn; ++k) {
+    int x, y, z;
+    bool ok;
+    const LevelDev &L = beyond(k, x, y, z, ok);
+    if (ok && n_ext > 0) ext_first_cell<D>(C, L, x, y, z, ub1);
+  }
+  const V *uin = n_ext > 0 ? ub1 : nullptr;
+  if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  // start the classification's counters (every CTA has read the band count; the lists are
+  // filled after the next barriers): the band count into the previous-band slot
+  if (blockIdx.x == 0 && tid == 0) {
+    cnt[5] = nl;
+    cnt[0] = cnt[1] = cnt[2] = cnt[3] = cnt[4] = 0;
+  }
+  // ---- the other sweeps
+  for (int it = 1; it < n_ext; ++it) {
+    V *const uout = (it & 1) ? ub2 : ub1;
+    for (int k = 0; k < ks; ++k) {
+      const unsigned fl = SM[k].fl[tid];
+      if (!(fl & SL_LIVE)) continue;
+      const unsigned fc = SM[k].fc[tid];
+      if (fl & SL_IFACE) {  // after two sweeps both buffers hold the value
+        if (it == 1) uout[fc] = SM[k].u[tid];
+        continue;
+      }
+      const LsfGeo g = geo_of(fl >> SL_LD);
+      float va[3], u0[3], un[D][3], acc[3] = {0.f, 0.f, 0.f};
+      u_get(SM[k].v[tid], va);
+      int dn[3];
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const int str = a == 0 ? 1 : (a == 1 ? g.p0 : g.p01);
+        dn[a] = va[a] > 0.f ? -str : str;
+      }
+      if (fl & SL_EDGE) {
+        const unsigned dist = fl >> SL_DIST;
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+          dn[a] = lsf_step(g, dist, a, va[a] > 0.f ? -1 : 1) * (a == 0 ? 1 : (a == 1 ? g.p0 : g.p01));
+      }
+#pragma unroll
+      for (int a = 0; a < D; ++a) u_get(uin[fc + (unsigned)dn[a]], un[a]);
+      u_get(SM[k].u[tid], u0);
+      // va (u0 - un) upwind, -va (u0 - un) downwind: |va| (u0 - un) on both sides
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int b = 0; b < D; ++b) acc[b] += fabsf(va[a]) * (u0[b] - un[a][b]);
+#pragma unroll
+      for (int b = 0; b < D; ++b) u0[b] = u0[b] - g.dte * acc[b];
+      V r;
+      u_put(r, u0, 0.f);
+      uout[fc] = r;
+      SM[k].u[tid] = r;
+    }
+    for (int k = ks; k < kn; ++k) {
+      int x, y, z;
+      bool ok;
+      const LevelDev &L = beyond(k, x, y, z, ok);
+      if (ok) ext_sweep_cell<D>(C, L, x, y, z, uin, uout);
+    }
+    uin = uout;
+    if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  }
+  // values around a cell (at pc) along axis a at offsets -3..+3, or mirrored; last: the
+  // highest index wanted
+  auto gather = [&](const float *pc, const LsfGeo &g, unsigned fl, int a, bool back, float v[7], int last) {
+    const int str = a == 0 ? 1 : (a == 1 ? g.p0 : g.p01);
+    if (!(fl & (SL_NEAR << a))) {
+      const long long s = back ? -str : str;
+      const float *q = pc - 3 * s;
+#pragma unroll
+      for (int m = 0; m < 7; ++m)
+        if (m <= last) v[m] = q[m * s];
     } else {
-      fr = C.frozen[fc] != 0;
-      s0 = C.s0[fc];
+      const unsigned dist = fl >> SL_DIST;
+#pragma unroll
+      for (int m = 0; m < 7; ++m)
+        if (m <= last) v[m] = pc[(long long)lsf_step(g, dist, a, back ? 3 - m : m - 3) * str];
     }
-    if (fr) {
-      if (stage == 1) C.p1[fc] = p0;
-      else if (stage == 2) C.p2[fc] = p0;
-      continue;
+  };
+  // ---- transport
+  for (int stage = 1; stage <= 3; ++stage) {
+    const float *pin = stage == 1 ? C.phi : (stage == 2 ? C.p1 : C.p2);
+    for (int k = 0; k < ks; ++k) {
+      const unsigned fl = SM[k].fl[tid];
+      if (!(fl & SL_LIVE)) continue;
+      const unsigned fc = SM[k].fc[tid];
+      const LsfGeo g = geo_of(fl >> SL_LD);
+      float ua[3], v[D][7];
+      u_get(SM[k].u[tid], ua);
+      const float p0 = stage == 1 ? C.phi[fc] : SM[k].v[tid].x;
+#pragma unroll
+      for (int a = 0; a < D; ++a)  // upwind side by the sign of u~: the mirrored stencil is the same sum negated
+        gather(pin + fc, g, fl, a, !(ua[a] >= 0.f), v[a], 5);
+      if (stage == 1) {  // commit u~ (the buffer of the last sweep holds it)
+#pragma unroll
+        for (int a = 0; a < D; ++a) C.ut0[a * NF + fc] = ua[a];
+        if (uin != ub1) u_put(ub1[fc], ua, 0.f);
+        if (uin != ub2) u_put(ub2[fc], ua, 0.f);
+      }
+      float rhs = 0.f;
+#pragma unroll
+      for (int a = 0; a < D; ++a) {
+        const float d = d5m(v[a]);
+        rhs -= ua[a] * (ua[a] >= 0.f ? d : -d);
+      }
+      float r;
+      if (stage == 1) {
+        r = p0 + rhs;
+        C.p1[fc] = r;
+        SM[k].v[tid].x = p0;
+        SM[k].v[tid].y = r;
+      } else if (stage == 2) {
+        r = 0.75f * p0 + 0.25f * (SM[k].v[tid].y + rhs);
+        C.p2[fc] = r;
+        SM[k].v[tid].y = r;
+      } else {
+        r = p0 / 3.0f + (2.0f / 3.0f) * (SM[k].v[tid].y + rhs);
+        C.phi[fc] = r;
+        SM[k].v[tid].x = r;
+      }
     }
-    const float *pinL = pin + L.fine_off;
-    float g2 = 0.f;
-    for (int a = 0; a < D; ++a) {
-      float v[7];
-      gather7m(L, pinL, x, y, z, cl, a, v);
-      const float dm = weno5(v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3], v[5] - v[4]);
-      const float dp = weno5(v[6] - v[5], v[5] - v[4], v[4] - v[3], v[3] - v[2], v[2] - v[1]);
-      float ga;
-      if (s0 > 0.f) ga = fmaxf(fmaxf(dm, 0.f) * fmaxf(dm, 0.f), fminf(dp, 0.f) * fminf(dp, 0.f));
-      else ga = fmaxf(fminf(dm, 0.f) * fminf(dm, 0.f), fmaxf(dp, 0.f) * fmaxf(dp, 0.f));
-      g2 += ga;
+    for (int k = ks; k < kn; ++k) {
+      int x, y, z;
+      bool ok;
+      const LevelDev &L = beyond(k, x, y, z, ok);
+      if (ok) adv_cell<D>(C, L, x, y, z, stage, uin, ub1, ub2);
     }
-    const float rhs = L.dtau_reinit * (-s0 * (sqrtf(g2) - 1.0f));
-    if (stage == 1) C.p1[fc] = p0 + rhs;
-    else if (stage == 2) C.p2[fc] = 0.75f * p0 + 0.25f * (C.p1[fc] + rhs);
-    else C.phi[fc] = p0 / 3.0f + (2.0f / 3.0f) * (C.p2[fc] + rhs);
+    if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  }
+  // ---- reinitialisation
+  for (int r = 0; r < n_re; ++r)
+    for (int stage = 1; stage <= 3; ++stage) {
+      const float *pin = stage == 1 ? C.phi : (stage == 2 ? C.p1 : C.p2);
+      const bool prep = r == 0 && stage == 1;
+      for (int k = 0; k < ks; ++k) {
+        unsigned fl = SM[k].fl[tid];
+        if (!(fl & SL_LIVE)) continue;
+        const unsigned fc = SM[k].fc[tid];
+        const LsfGeo g = geo_of(fl >> SL_LD);
+        const float p0 = SM[k].v[tid].x;
+        if (prep) {
+          if ((fl & SL_EDGE) ? sign_change<Q>(C.phi + fc, p0, lsf_near<D>(g, fl >> SL_DIST))
+                             : sign_change_inner<Q>(C.phi + fc, p0, g.p0, g.p01))
+            fl |= SL_FROZEN;
+          SM[k].fl[tid] = fl;
+          SM[k].u[tid].x = p0 / sqrtf(p0 * p0 + 1.0f);
+        }
+        if (fl & SL_FROZEN) {
+          if (stage == 1) C.p1[fc] = p0;
+          else if (stage == 2) C.p2[fc] = p0;
+          continue;
+        }
+        const float s0 = SM[k].u[tid].x;
+        float g2 = 0.f, v[D][7];
+#pragma unroll
+        for (int a = 0; a < D; ++a) gather(pin + fc, g, fl, a, false, v[a], 6);
+#pragma unroll
+        for (int a = 0; a < D; ++a) g2 += godunov_axis(v[a], s0);
+        const float rhs = g.dtr * (-s0 * (sqrtf(g2) - 1.0f));
+        float q;
+        if (stage == 1) {
+          q = p0 + rhs;
+          C.p1[fc] = q;
+          SM[k].v[tid].y = q;
+        } else if (stage == 2) {
+          q = 0.75f * p0 + 0.25f * (SM[k].v[tid].y + rhs);
+          C.p2[fc] = q;
+          SM[k].v[tid].y = q;
+        } else {
+          q = p0 / 3.0f + (2.0f / 3.0f) * (SM[k].v[tid].y + rhs);
+          C.phi[fc] = q;
+          SM[k].v[tid].x = q;
+        }
+      }
+      for (int k = ks; k < kn; ++k) {
+        int x, y, z;
+        bool ok;
+        const LevelDev &L = beyond(k, x, y, z, ok);
+        if (ok) reinit_cell<Q>(C, L, x, y, z, stage, prep);
+      }
+      if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+    }
+  // ---- phases (k_classify_phase without init): p1, p2 back to phi, tags, flips
+  for (int k = 0; k < kn; ++k) {
+    const int w = w0 + k * GB;
+    unsigned fc;
+    long long tc;
+    float ph;
+    int ld;
+    if (k < ks) {
+      const unsigned fl = SM[k].fl[tid];
+      if (!(fl & SL_CELL)) continue;
+      fc = SM[k].fc[tid];
+      ld = (int)(fl >> SL_LD);
+      tc = (long long)fc + geo_of((unsigned)ld).tag_delta;
+      ph = (fl & SL_LIVE) ? SM[k].v[tid].x : C.phi[fc];
+    } else {
+      if (w >= nl) continue;
+      int x, y, z;
+      const int4 b = info[w];
+      const LevelDev &L = band_cell_at(C, S, b, t, x, y, z);
+      if (x >= L.n[0] || y >= L.n[1] || z >= L.n[2]) continue;
+      fc = (unsigned)(L.fine_off + cidx(L, x, y, z));
+      ld = b.x;
+      tc = (long long)fc + L.cell_off - L.fine_off;
+      ph = C.phi[fc];
+    }
+    const uint8_t tg = C.tag[tc];
+    if (!(tg & TAG_LEAF)) continue;
+    C.p1[fc] = ph;
+    C.p2[fc] = ph;
+    const int gas = ph >= 0.0f ? 1 : 0, prev = tg & TAG_GAS;
+    C.tag[tc] = (tg & (TAG_LEAF | TAG_RLAYER | TAG_GHOST)) | (gas ? TAG_GAS : 0) | (prev ? TAG_PREVGAS : 0) |
+                (gas != prev ? TAG_FLIP : 0);
+    if (gas != prev) {
+      const LevelDev &L = C.lds[ld];
+      int x, y, z;
+      cell_xyz(L, fc - L.fine_off, x, y, z);
+      list_flip<Q>(C, L, S, glevel, ld, fc - L.fine_off, x, y, z);
+    }
+  }
+  if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  // ---- cut links (k_classify_links without full): the previous band, then the check list
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int *lst = C.band_list + (long long)glevel * C.band_cap, *chk = C.check_list + (long long)glevel * C.band_cap;
+  const int nb2 = nl + min(cnt[4], C.band_cap);
+  const int hb = tid >> lgnt;
+  for (int k = 0; k * GB < nb2; ++k) {
+    const int w = w0 + k * GB;
+    if (t == 0) hot[hb] = 0;
+    __syncthreads();
+    int gb = 0;
+    if (w < nb2) {
+      uint32_t m = 0;
+      unsigned fc = 0, dist = 0;
+      uint8_t tg = 0;
+      int ld = 0;
+      bool cell, edge;
+      gb = w < nl ? lst[w] : chk[w - nl];
+      if (k < ks && w < nl) {
+        const unsigned fl = SM[k].fl[tid];
+        ld = (int)(fl >> SL_LD);
+        cell = (fl & SL_CELL) != 0;
+        edge = (fl & SL_EDGE) != 0;
+        dist = fl >> SL_DIST;
+        if (cell) fc = SM[k].fc[tid];
+      } else {
+        const int4 b = C.blk_info[gb];
+        ld = b.x;
+        const int crd[3] = {(b.y << S.lg[0]) + (t & (S.bs[0] - 1)), (b.z << S.lg[1]) + ((t >> S.lg[0]) & (S.bs[1] - 1)),
+                            (b.w << S.lg[2]) + (t >> (S.lg[0] + S.lg[1]))};
+        const LsfGeo g = geo_of((unsigned)ld);
+        cell = crd[0] < g.n[0] && crd[1] < g.n[1] && crd[2] < g.n[2];
+        edge = true;
+        if (cell) {
+          fc = g.fo + (unsigned)crd[0] + (unsigned)(g.p0 * crd[1] + g.p01 * crd[2]);
+          dist = lsf_dist<D>(crd, g.n);
+        }
+      }
+      const LsfGeo g = geo_of((unsigned)ld);
+      const long long tc = (long long)fc + g.tag_delta;
+      if (cell) {
+        tg = C.tag[tc];
+        if (tg & TAG_LEAF) {
+          m = edge ? cut_mask<Q>(C.tag + tc, tg, lsf_near<D>(g, dist)) : cut_mask_inner<Q>(C.tag + tc, tg, g.p0, g.p01);
+          C.cmask[fc] = m;
+        }
+      }
+      list_links(C, glevel, m, ld, (int)(fc - g.fo), fc, tc, tg);
+      if (m) hot[hb] = 1;
+    }
+    __syncthreads();
+    if (t == 0 && w < nb2) C.bflag[gb] = hot[hb] ? BF_IFACE : 0;
+  }
+  leave();
+}
+
+// Both sweep buffers from ut0 at every finest cell (their state between updates).
+template <int D>
+__global__ void k_ut_pack(const float *__restrict__ ut0, typename UVec<D>::T *ub1, typename UVec<D>::T *ub2,
+                          long long n) {
+  LSB_GRID_WAIT();
+  for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
+    float u[3];
+    for (int a = 0; a < D; ++a) u[a] = ut0[a * n + c];
+    u_put(ub1[c], u, 0.f);
+    u_put(ub2[c], u, 0.f);
   }
 }
 
@@ -1332,24 +1936,92 @@ cudaError_t run_ext_iter(int D, Launch L, Ctx C, BlockShape S, int glevel, const
 cudaError_t run_adv_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage) {
   LDP(k_adv_stage, C, S, glevel, stage);
 }
-cudaError_t run_ext_first(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *uin, float *uout,
-                          int turn) {
-  LDP(k_ext_first, C, S, glevel, uin, uout, turn);
-}
-cudaError_t run_ext_sweep_mirror(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *uin, float *uout) {
-  if (D == 2)
-    launcher(k_ext_plan<2, true>, with_grid(L, resident_grid(k_ext_plan<2, true>, L.block, L.grid)))(C, S, glevel, uin,
-                                                                                                      uout);
-  else
-    launcher(k_ext_plan<3, true>, with_grid(L, resident_grid(k_ext_plan<3, true>, L.block, L.grid)))(C, S, glevel, uin,
-                                                                                                      uout);
+// Shared memory of the one-launch level-set update.
+size_t lsf_smem(int D, int kcap) { return (D == 2 ? sizeof(LsfSlot<2>) : sizeof(LsfSlot<3>)) * (size_t)kcap; }
+cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n) {
+  if (D == 2) launcher(k_ut_pack<2>, L, 0)(ut0, (float2 *)ut1, (float2 *)ut2, n);
+  else launcher(k_ut_pack<3>, L, 0)(ut0, (float4 *)ut1, (float4 *)ut2, n);
   return cudaGetLastError();
 }
-cudaError_t run_adv_mirror(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage, const float *ufin) {
-  LDP(k_adv_mirror, C, S, glevel, stage, ufin);
+template <int Q>
+cudaError_t lsf_prepare(LsfLimits *out) {
+  constexpr int D = Lat<Q>::D;
+  int dev = 0, sms = 0, optin = 0, coop = 0, nb = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+  cudaFuncAttributes fa;
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, k_levelset_fused<Q, 1>);
+  if (e != cudaSuccess) return e;
+  out->kmax = (int)(((size_t)optin - fa.sharedSizeBytes - 1024) / lsf_smem(D, 1));
+  const int smem = (int)lsf_smem(D, out->kmax);
+  e = cudaFuncSetAttribute(k_levelset_fused<Q, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_levelset_fused<Q, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(k_levelset_fused<Q, 0>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_levelset_fused<Q, 1>, 1024, smem);
+  if (e != cudaSuccess) return e;
+  out->grid = coop && nb > 0 ? sms : 0;
+  out->cluster = 8;
+  out->max_ld = kLsfMaxLd;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 16;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(16);
+  cfg.blockDim = dim3(1024);
+  cfg.dynamicSmemBytes = lsf_smem(D, 2);
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int nc = 0;
+  if (cudaOccupancyMaxActiveClusters(&nc, k_levelset_fused<Q, 0>, &cfg) == cudaSuccess && nc > 0) out->cluster = 16;
+  else cudaGetLastError();
+  return cudaSuccess;
 }
-cudaError_t run_reinit_mirror(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, int prep) {
-  LQP(k_reinit_mirror, C, S, glevel, stage, prep);
+cudaError_t prepare_levelset_fused(int Q, LsfLimits *out) {
+  return Q == 9 ? lsf_prepare<9>(out) : (Q == 19 ? lsf_prepare<19>(out) : lsf_prepare<27>(out));
+}
+template <int Q>
+cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
+                       unsigned *bar) {
+  cudaLaunchAttribute at[3];
+  unsigned na = 0;
+  if (P.coop) {
+    at[na].id = cudaLaunchAttributeCooperative;
+    at[na++].val.cooperative = 1;
+  } else {
+    at[na].id = cudaLaunchAttributeClusterDimension;
+    at[na].val.clusterDim.x = (unsigned)P.grid;
+    at[na].val.clusterDim.y = at[na].val.clusterDim.z = 1;
+    ++na;
+  }
+  // a cooperative launch is no programmatic dependent: launched early it loses the guarantee
+  // that its CTAs become resident together (steps of 1 to 80 ms seen beside a side stream's
+  // collide, 0.77 without)
+  if (L.pdl && !P.coop) {
+    at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[na++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (L.prio) {
+    at[na].id = cudaLaunchAttributePriority;
+    at[na++].val.priority = L.prio;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)P.grid);
+  cfg.blockDim = dim3((unsigned)P.threads);
+  cfg.dynamicSmemBytes = lsf_smem(Lat<Q>::D, P.kcap);
+  cfg.stream = L.stream;
+  cfg.attrs = at;
+  cfg.numAttrs = na;
+  if (P.coop) return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 1>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar);
+  return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 0>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar);
+}
+cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
+                               unsigned *bar) {
+  if (Q == 9) return lsf_launch<9>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
+  if (Q == 19) return lsf_launch<19>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
+  return lsf_launch<27>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
 }
 cudaError_t run_reinit_prep(int Q, Launch L, Ctx C, BlockShape S, int glevel) { LQP(k_reinit_prep, C, S, glevel); }
 cudaError_t run_reinit_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage) {
