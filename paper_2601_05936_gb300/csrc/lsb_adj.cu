@@ -380,10 +380,6 @@ __global__ void k_adj_links(Ctx C, int glevel, const float *__restrict__ F, floa
       if (sg[k] != 0.0) atomicAdd(grad + (long long)(k / 5) * NG_ADJ + (k % 5), sg[k]);
 }
 
-#ifndef LSB_ADJ_MINB
-#define LSB_ADJ_MINB 2  // CTAs of 512 threads per SM the adjoint collision is built for (64 registers,
-                        // some spills: 0.354 -> 0.371 of measured HBM against one CTA at 128)
-#endif
 // ------------------------------------------------------------------ streaming + collision
 // One thread per leaf cell.  lambda_c (adjoint of the post-collision values) is
 // the transpose of the forward push: population i of x went to x + c_i, to
@@ -393,7 +389,18 @@ __global__ void k_adj_links(Ctx C, int glevel, const float *__restrict__ F, floa
 // the strain rate S = k Pi, k = -omega / (2 rho c_s^2),
 // Pi_ab = sum c_a c_b (f - feq), with dPi_ab / df_j = c_ja c_jb - c_s^2 d_ab
 // + u_a u_b - c_ja u_b - u_a c_jb.
-template <int Q>
+//
+// Bound by HBM (3 Q floats per cell) as far as its loads keep up: 38 loads per thread in
+// flight, two CTAs of 512 threads per SM (64 registers).  With the transposed collision
+// written per population (~570 flops a cell) and a grid of one CTA per SM it took 383 us on
+// 4.19 M cells (D3Q19, 2.50 TB/s); two CTAs per SM 298 us; through lambda's weighted moments
+// (MOMENTS, ~150 flops) 221 us, 4.32 TB/s (0.64 of the measured copy).  One CTA per SM at
+// 128 registers 316 us, three at 40 (spills) 386 us, shorter-lived CTAs (a grid of 1216) 234 us.
+// MOMENTS serves the frozen level set, where its error against the float64 oracle is the
+// smaller one (dJ/df_0 2.2 - 4.7e-7 against 3.0 - 6.9e-7).  The sweep over a moving level set
+// keeps the sums per population: its parameter gradients cancel down to a part in 10^4 - 10^5
+// of their terms, so that a change of rounding here shows there.
+template <int Q, bool MOMENTS>
 __global__ void __launch_bounds__(512, LSB_ADJ_MINB) k_adj_collide(Ctx C, BlockShape S, const int *__restrict__ list, int nlist,
                                                       const float *__restrict__ F, const float *__restrict__ lamN,
                                                       float *__restrict__ lamO, const float *__restrict__ LA,
@@ -462,9 +469,7 @@ __global__ void __launch_bounds__(512, LSB_ADJ_MINB) k_adj_collide(Ctx C, BlockS
       cb = C.cbase[L.fine_off + c];
     }
     const bool ccut = !fine && (tg & TAG_CCUT);
-    // lc: adjoint of the post-collision populations.  Held in registers with up to
-    // 128 of them per thread (one CTA of 512 per SM): more loads in flight per
-    // thread measured faster than two CTAs per SM with lc in shared memory.
+    // lc: adjoint of the post-collision populations, in registers
     float lc[Q];
 #define LC(i) lc[(i)]
 #pragma unroll
@@ -532,29 +537,66 @@ __global__ void __launch_bounds__(512, LSB_ADJ_MINB) k_adj_collide(Ctx C, BlockS
     const int ph = tg & TAG_GAS;
     const float om = L.omega[ph];
     const float ac[3] = {L.acc[ph][0], L.acc[ph][1], L.acc[ph][2]};
-    float As = 0.f, Bv[3] = {0.f, 0.f, 0.f}, slfe = 0.f, lac[3] = {0.f, 0.f, 0.f};
+    float lom, base, g0[3], lac[3] = {0.f, 0.f, 0.f};
+    if constexpr (MOMENTS) {
+      // Everything the transposed collision needs of lambda are its weighted moments M0 = sum w l,
+      // M1_a = sum w l c_a, M2_ab = sum w l c_a c_b, formed per pair (i, opp(i)): with e_i = 1 +
+      // 3 c_i.u + 9/2 (c_i.u)^2 - 3/2 u^2 (feq_i = w_i rho e_i), sum w l (e_i - 1) = 3 u.M1 +
+      // 9/2 u.M2.u - 3/2 u^2 M0 =: e1, sum l d feq_i / d rho = M0 + e1, sum l d feq_i / d u_a =
+      // rho (3 M1_a + 9 (M2 u)_a - 3 u_a M0) and sum l f~eq_i = drho M0 + rho e1.
+      float M0 = LT::w(LT::REST) * LC(LT::REST), M1[3] = {0.f, 0.f, 0.f}, Mxx = 0.f, Mxy = 0.f, Mxz = 0.f, Myy = 0.f,
+            Myz = 0.f, Mzz = 0.f;
 #pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const float cx = LT::cx(i), cy = LT::cy(i), cz = LT::cz(i);
-      const float cu = cx * u[0] + cy * u[1] + cz * u[2];
-      const float fe = feq_dev<Q>(i, drho, u, usq);
-      const float l = LC(i);
-      const float wl = LT::w(i) * l;
-      // d feq_i / d rho = feq_i / rho (full feq = w + f~eq), d feq_i / d u_a = w rho (3 c_a + 9 cu c_a - 3 u_a)
-      As += l * (om * (fe + LT::w(i)) * irho + 3.0f * LT::w(i) * (cx * ac[0] + cy * ac[1] + cz * ac[2]));
-      const float g = om * wl * rho;
-      Bv[0] += g * (3.0f * cx + 9.0f * cu * cx - 3.0f * u[0]);
-      Bv[1] += g * (3.0f * cy + 9.0f * cu * cy - 3.0f * u[1]);
-      if (D == 3) Bv[2] += g * (3.0f * cz + 9.0f * cu * cz - 3.0f * u[2]);
-      slfe += l * fe;
-      lac[0] += 3.0f * wl * rho * cx;
-      lac[1] += 3.0f * wl * rho * cy;
-      if (D == 3) lac[2] += 3.0f * wl * rho * cz;
+      for (int i = 0; i < Q; ++i) {
+        if (i == LT::REST || LT::opp(i) < i) continue;
+        const float cx = LT::cx(i), cy = LT::cy(i), cz = LT::cz(i);
+        const float wp = LT::w(i) * (LC(i) + LC(LT::opp(i))), wm = LT::w(i) * (LC(i) - LC(LT::opp(i)));
+        M0 += wp;
+        M1[0] += cx * wm;
+        M1[1] += cy * wm;
+        M1[2] += cz * wm;
+        Mxx += cx * cx * wp;
+        Mxy += cx * cy * wp;
+        Myy += cy * cy * wp;
+        Mxz += cx * cz * wp;
+        Myz += cy * cz * wp;
+        Mzz += cz * cz * wp;
+      }
+      const float Mu[3] = {Mxx * u[0] + Mxy * u[1] + Mxz * u[2], Mxy * u[0] + Myy * u[1] + Myz * u[2],
+                           Mxz * u[0] + Myz * u[1] + Mzz * u[2]};
+      const float e1 = 3.0f * (u[0] * M1[0] + u[1] * M1[1] + u[2] * M1[2]) +
+                       4.5f * (u[0] * Mu[0] + u[1] * Mu[1] + u[2] * Mu[2]) - 1.5f * usq * M0;
+      lom = drho * M0 + rho * e1 - slf;  // sum lc_i (feq_i - f_i)
+      for (int a = 0; a < 3; ++a) {
+        g0[a] = om * (3.0f * M1[a] + 9.0f * Mu[a] - 3.0f * u[a] * M0);
+        lac[a] = 3.0f * rho * M1[a];
+      }
+      base = om * (M0 + e1) + 3.0f * (M1[0] * ac[0] + M1[1] * ac[1] + M1[2] * ac[2]) -
+                         (g0[0] * u[0] + g0[1] * u[1] + g0[2] * u[2]);
+    } else {
+      float As = 0.f, Bv[3] = {0.f, 0.f, 0.f}, slfe = 0.f;
+#pragma unroll
+      for (int i = 0; i < Q; ++i) {
+        const float cx = LT::cx(i), cy = LT::cy(i), cz = LT::cz(i);
+        const float cu = cx * u[0] + cy * u[1] + cz * u[2];
+        const float fe = feq_dev<Q>(i, drho, u, usq);
+        const float l = LC(i);
+        const float wl = LT::w(i) * l;
+        // d feq_i / d rho = feq_i / rho (full feq = w + f~eq), d feq_i / d u_a = w rho (3 c_a + 9 cu c_a - 3 u_a)
+        As += l * (om * (fe + LT::w(i)) * irho + 3.0f * LT::w(i) * (cx * ac[0] + cy * ac[1] + cz * ac[2]));
+        const float g = om * wl * rho;
+        Bv[0] += g * (3.0f * cx + 9.0f * cu * cx - 3.0f * u[0]);
+        Bv[1] += g * (3.0f * cy + 9.0f * cu * cy - 3.0f * u[1]);
+        if (D == 3) Bv[2] += g * (3.0f * cz + 9.0f * cu * cz - 3.0f * u[2]);
+        slfe += l * fe;
+        lac[0] += 3.0f * wl * rho * cx;
+        lac[1] += 3.0f * wl * rho * cy;
+        if (D == 3) lac[2] += 3.0f * wl * rho * cz;
+      }
+      lom = slfe - slf;  // sum lc_i (feq_i - f_i)
+      for (int a = 0; a < 3; ++a) g0[a] = Bv[a] * irho;
+      base = As - (g0[0] * u[0] + g0[1] * u[1] + g0[2] * u[2]);
     }
-    const float lom = slfe - slf;  // sum lc_i (feq_i - f_i)
-    float g0[3];
-    for (int a = 0; a < 3; ++a) g0[a] = Bv[a] * irho;
-    const float base = As - (g0[0] * u[0] + g0[1] * u[1] + g0[2] * u[2]);
 #pragma unroll
     for (int j = 0; j < Q; ++j)
       lO[j * N + c] = (1.0f - om) * LC(j) + base + g0[0] * LT::cx(j) + g0[1] * LT::cy(j) + g0[2] * LT::cz(j);
@@ -1183,8 +1225,15 @@ cudaError_t run_adj_geometry(int D, Launch L, Ctx C, int glevel, GeoAdj G) {
 }
 
 cudaError_t run_adj_collide(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *F,
-                            const float *lamN, float *lamO, const float *LA, double *grad) {
-  LSB_ADJ_Q(Q, k_adj_collide, L, C, S, list, n, F, lamN, lamO, LA, grad);
+                            const float *lamN, float *lamO, const float *LA, double *grad, int moments) {
+  if (Q == 9) {
+    if (moments) k_adj_collide<9, true><<<L.grid, L.block, 0, L.stream>>>(C, S, list, n, F, lamN, lamO, LA, grad);
+    else k_adj_collide<9, false><<<L.grid, L.block, 0, L.stream>>>(C, S, list, n, F, lamN, lamO, LA, grad);
+  } else {
+    if (moments) k_adj_collide<19, true><<<L.grid, L.block, 0, L.stream>>>(C, S, list, n, F, lamN, lamO, LA, grad);
+    else k_adj_collide<19, false><<<L.grid, L.block, 0, L.stream>>>(C, S, list, n, F, lamN, lamO, LA, grad);
+  }
+  return cudaGetLastError();
 }
 
 cudaError_t run_adj_macro(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamO, float *MA, double *grad,

@@ -1183,10 +1183,10 @@ lsb_status adj_lb(lsb_grid *g, int l, const float *F, float *lamN, float *lamO, 
   if (fine)
     RUN(KADJ_LINKS, 0, 1, 128, run_adj_links, Q, LN(g, DYN_GRID, 128), C, l, F, lamN, g->d_linkadj, g->d_madj,
         g->d_grad, g->ncase, G);
-  const int grid = std::min(g->cs[l].n, 152);
+  const int grid = std::min(g->cs[l].n, 152 * LSB_ADJ_MINB);  // the resident CTAs
   RUN(KADJ_COLLIDE, 3.0 * Q * sizeof(float) * g->leaf_cells[l], g->cs[l].n, g->nthreads, run_adj_collide, Q,
       LN(g, grid, g->nthreads), C, S, (const int *)g->cs[l].d, g->cs[l].n, F, (const float *)lamN, lamO,
-      (const float *)g->d_linkadj, g->d_grad);
+      (const float *)g->d_linkadj, g->d_grad, g->rec_moving ? 0 : 1);
   if (fine)
     RUN(KADJ_MACRO, 0, 1, 128, run_adj_macro, Q, LN(g, DYN_GRID, 128), C, l, F, lamO, g->d_madj, g->d_grad,
         g->ncase);

@@ -127,6 +127,9 @@ cudaError_t run_levelset_persistent(int Q, Launch L, Ctx C, BlockShape S, int gl
 cudaError_t run_sensor(Launch L, Ctx C, BlockShape S, const int *list, int n, int mode, float *out);
 
 // lsb_adj.cu: adjoint of the frozen-interface step
+#ifndef LSB_ADJ_MINB
+#define LSB_ADJ_MINB 2  // CTAs of 512 threads per SM the adjoint collision is built for (its grid)
+#endif
 constexpr int NG_ADJ = 13;  // parameter partials per case accumulated on the device
 // Adjoints of the frozen geometry, finest-level arrays (nullptr: not computed):
 // phi (nfine), interface cells' normal (D planes of nfine) and curvature (nfine).
@@ -138,8 +141,9 @@ cudaError_t run_adj_seed(int Q, Launch L, Ctx C, BlockShape S, const int *list, 
 cudaError_t run_adj_links(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamN, float *LA, float *MA,
                           double *grad, int ncase, GeoAdj G);
 cudaError_t run_adj_geometry(int D, Launch L, Ctx C, int glevel, GeoAdj G);
+// moments: the transposed collision through lambda's weighted moments (see k_adj_collide)
 cudaError_t run_adj_collide(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *F,
-                            const float *lamN, float *lamO, const float *LA, double *grad);
+                            const float *lamN, float *lamO, const float *LA, double *grad, int moments);
 cudaError_t run_adj_macro(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamO, float *MA, double *grad,
                           int ncase);
 // Multi-level grids: transposes of the ghost-ring transfer (per ghost cell of a
