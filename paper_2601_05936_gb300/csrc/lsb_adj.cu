@@ -710,7 +710,8 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
 }
 
 // ------------------------------------------------------------------ level-set adjoint
-// One thread per interface cell, once after the sweep: the adjoints of the cell's
+// One thread per interface cell, once after the sweep (moving level set: after every
+// sub-step; the adjoints are cleared as they are read): the adjoints of the cell's
 // normal n = g / |g| and curvature kappa = (|g|^2 tr H - g.H.g) / |g|^3 (summed over
 // the window by k_adj_links) go back through the closed-form least-squares
 // quadratic of k_geometry (Sec. 2.2): gradient g and Hessian H are linear in the
@@ -727,8 +728,12 @@ __global__ void k_adj_geometry(Ctx C, int glevel, GeoAdj G) {
     const LevelDev &L = C.lds[it.x];
     const long long c = it.y, fc = L.fine_off + c;
     double ln[3] = {0, 0, 0};
-    for (int a = 0; a < D; ++a) ln[a] = G.n[a * NF + fc];
+    for (int a = 0; a < D; ++a) {
+      ln[a] = G.n[a * NF + fc];
+      G.n[a * NF + fc] = 0.f;
+    }
     const double lk = G.kappa[fc];
+    G.kappa[fc] = 0.f;
     if (lk == 0.0 && ln[0] == 0.0 && ln[1] == 0.0 && ln[2] == 0.0) continue;
     int x, y, z;
     cell_xyz(L, c, x, y, z);

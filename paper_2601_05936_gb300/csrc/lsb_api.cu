@@ -102,6 +102,7 @@ struct lsb_grid {
   unsigned *d_bar = nullptr;  // grid barriers: of the persistent level-set kernel, of the one-launch update
   LsfLimits lsf_lim;
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
+  int band_est[MAXL] = {0, 0, 0, 0};  // band blocks when it was planned
   long long wait_limit = 1LL << 22;  // sleeps of ~64 ns before a device-side wait gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
@@ -149,7 +150,6 @@ struct lsb_grid {
   cudaEvent_t ev_free[MAXL] = {}, ev_fill[MAXL] = {}, ev_ring0[MAXL] = {}, ev_ring0_done[MAXL] = {};
   int early_fill = -1;  // level whose next ghost ring fills right after its collide
   bool classified[MAXL] = {};  // the level's phases and cut links came with the level-set update
-  bool init_done[MAXL] = {};        // the level's interface u~ came with the interface pass
   uint64_t gnodes[2][2] = {};
   // adjoint of the frozen-interface step: recording and reverse sweep
   int rec_on = 0, rec_every = 0;
@@ -170,7 +170,6 @@ struct lsb_grid {
   int tape_on = 0, tape_call = 0;
   std::vector<float *> tape_old, tape_new;  // state at the call's start (after restriction), after its sub-step
   std::vector<float *> tape_ls;             // moving level set: phi and u~ at each finest call's start
-  int lspar = 0;                            // moving level set: its adjoints are in LP[lspar], LU[lspar]
   float *d_adjx = nullptr;                  // coarse adjoint shares of the ghost rings (kept zero)
   float *d_fsave = nullptr, *d_madj = nullptr, *d_linkadj = nullptr;
   float *d_gphi = nullptr, *d_gn = nullptr, *d_gk = nullptr;  // level-set adjoint (finest level)
@@ -577,8 +576,6 @@ lsb_status levelset(lsb_grid *g, int l) {
         g->n_reinit, g->d_bar, g->wait_limit);
     return LSB_OK;
   }
-  if (!g->init_done[l]) RUN(12, 0, 1, 128, run_ext_init, Q, LN(g, DYN_GRID, 128), C, l);
-  g->init_done[l] = false;
   const bool due = g->reinit_every > 0 && ((g->fine_steps[l] + 1) % g->reinit_every == 0);
   RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
       (int)g->lds.size(), g->d_bar + 2);
@@ -596,6 +593,7 @@ lsb_status plan_levelset(lsb_grid *g, int l) {
   CU(cudaMemcpyAsync(&nb, g->d_counters + l * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   CU(cudaStreamSynchronize(g->stream));
   nb = std::max(1, std::min(nb, g->band_cap));
+  g->band_est[l] = nb;
   nb += nb / 16;  // room for the band to grow until the next regrid
   const int nt = g->nthreads, per = 1024 / nt;  // blocks of a full CTA
   const LsfLimits &M = g->lsf_lim;
@@ -756,7 +754,6 @@ lsb_status advance(lsb_grid *g, int l) {
       // the interface pass and the level set's first pass (u~ at the interface cells) share
       // a launch; the level-set update then starts from its first extension sweep
       RUN(1, 0, 1, 128, run_iface_init, Q, st, LN(g, LSB_INIT_CTAS + LSB_IFACE_CTAS, 128), C, l, LSB_INIT_CTAS);
-      g->init_done[l] = true;
     } else {
       RUN(1, 0, 1, 128, run_interface_bc, Q, st, LN(g, DYN_GRID, 128), C, l);
     }
@@ -1059,23 +1056,18 @@ lsb_status rec_checkpoint(lsb_grid *g) {
   return LSB_OK;
 }
 
-// Scratch of the moving level-set adjoint, carved from one allocation (finest-level
-// arrays of nfine floats; "vector" arrays hold D planes).
+// Scratch of the moving level-set adjoint, carved from one allocation (finest-level arrays of
+// nfine floats; "vector" arrays hold D planes).  The arrays from LP on start a reverse sweep
+// at zero (lsa_zero_from planes precede them).
 struct LsaPtrs {
-  float *S;                       // S_0 .. S_n_ext: u~ after the interface pass and each sweep
-  float *U1;                      // committed u~ of the step
-  float *PHI0, *PS, *A1, *A2, *R1, *R2, *SS, *KP;
-  float *NV;                      // normals of phi_n (D planes)
-  float *L0r, *L1, *L2, *LS0;     // RK3 adjoints and d/dS0
-  float *LA, *LK[2], *LOFF, *LV;  // adjoints of the extension (D planes each)
-  float *LP[2];                   // adjoint of phi (ping-pong)
-  float *LU[2];                   // adjoint of u~ (ping-pong, D planes)
-  uint8_t *FR;                    // frozen cells of the reinitialisation
+  LsaScratch A;   // (S0 is the step's own u~)
+  float *KP, *NV; // curvature and normals (D planes) of phi_n
 };
 
+size_t lsa_zero_from(const lsb_grid *g) { return (size_t)g->D * std::max(g->n_ext, 1) + 8 + g->D; }
 size_t lsa_floats_needed(const lsb_grid *g) {
   const size_t NF = g->nfine, D = g->D;
-  return NF * (D * (g->n_ext + 1) + D + 8 + D + 4 + 5 * D + 2 + 2 * D) + NF / 4 + 64;
+  return NF * (lsa_zero_from(g) + 1 + D + 2 + 3 * D) + NF / 4 + 64;
 }
 
 LsaPtrs lsa_ptrs(const lsb_grid *g) {
@@ -1087,16 +1079,16 @@ LsaPtrs lsa_ptrs(const lsb_grid *g) {
     return r;
   };
   LsaPtrs P;
-  P.S = take(D * (g->n_ext + 1));
-  P.U1 = take(D);
-  P.PHI0 = take(1); P.PS = take(1); P.A1 = take(1); P.A2 = take(1);
-  P.R1 = take(1); P.R2 = take(1); P.SS = take(1); P.KP = take(1);
+  P.A.S0 = nullptr;
+  P.A.S = take(D * std::max(g->n_ext, 1));
+  P.A.A1 = take(1); P.A.A2 = take(1); P.A.R1 = take(1); P.A.R2 = take(1);
+  P.A.PB = take(1); P.A.SS = take(1); P.A.LS0 = take(1);
+  P.KP = take(1);
   P.NV = take(D);
-  P.L0r = take(1); P.L1 = take(1); P.L2 = take(1); P.LS0 = take(1);
-  P.LA = take(D); P.LK[0] = take(D); P.LK[1] = take(D); P.LOFF = take(D); P.LV = take(D);
-  P.LP[0] = take(1); P.LP[1] = take(1);
-  P.LU[0] = take(D); P.LU[1] = take(D);
-  P.FR = reinterpret_cast<uint8_t *>(p);
+  P.A.LP = take(1); P.A.LU = take(D);
+  P.A.L1 = take(1); P.A.L2 = take(1);
+  P.A.LK0 = take(D); P.A.LK1 = take(D); P.A.LV = take(D);
+  P.A.FR = reinterpret_cast<uint8_t *>(p);
   return P;
 }
 
@@ -1159,7 +1151,8 @@ lsb_status adj_buffers(lsb_grid *g, int seg_len) {
       if (e != cudaSuccess) return fail(g, LSB_ENOMEM, "level-set adjoint scratch cudaMalloc: %s", cudaGetErrorString(e));
       g->lsa_floats = need;
     }
-    CU(cudaMemsetAsync(g->d_lsa, 0, sizeof(float) * g->lsa_floats, g->stream));
+    const size_t z = lsa_zero_from(g) * g->nfine;
+    CU(cudaMemsetAsync(g->d_lsa + z, 0, sizeof(float) * (lsa_floats_needed(g) - z), g->stream));
     if (!g->d_phisave) {
       TRY(dalloc(g, &g->d_phisave, sizeof(float) * g->nfine));
       TRY(dalloc(g, &g->d_utsave, sizeof(float) * g->D * g->nfine));
@@ -1202,109 +1195,29 @@ lsb_status adj_step(lsb_grid *g, const float *F, int cur, GeoAdj G) {
 // from (f_n, phi_n, u~_n), then the transposes in reverse order (reinitialisation,
 // transport, extension, interface velocity), then the lattice Boltzmann part with
 // the geometry of phi_n.  l is the finest level; population adjoints lamN -> lamO, the
-// level set's LP[cur], LU[cur] -> LP[1 - cur], LU[1 - cur].
-lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, const float *ut_n, float *lamN, float *lamO,
-                      int cur) {
-  const LsaPtrs P = lsa_ptrs(g);
+// level set's LP, LU in place.  phi_n and ut_n are the step's stored copies: phi_n is
+// overwritten and written back on the way, u~ takes the interface cells' new values.
+lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *ut_n, float *lamN, float *lamO) {
+  LsaPtrs P = lsa_ptrs(g);
+  P.A.S0 = ut_n;
   const int Q = g->Q, D = g->D, nt = g->nthreads;
-  const long long NF = g->nfine;
-  const size_t b1 = sizeof(float) * NF, bD = sizeof(float) * D * NF;
-  const Ctx base = make_ctx(g);
   const BlockShape S = shape(g);
-  const int nb = std::max(1, std::min(g->band_cap, 152 * 16));
-  auto Sk = [&](int k) { return P.S + (size_t)k * D * NF; };
-  // ---- replay of the level-set passes of step n
-  CU(cudaMemcpyAsync(Sk(0), ut_n, bD, cudaMemcpyDeviceToDevice, g->stream));
-  Ctx R = base;
+  Ctx R = make_ctx(g);
   R.phi = phi_n;
-  RUN(KLSA, 0, 1, 128, run_lsa_init, Q, LN(g, DYN_GRID, 128), R, l, F, Sk(0));
-  Ctx E = base;
-  E.phi = phi_n;
-  E.ut0 = Sk(0);
-  for (int k = 0; k < g->n_ext; ++k)
-    RUN(KLSA, 0, nb, nt, run_ext_iter, D, LN(g, nb, nt), E, S, l, Sk(k), Sk(k + 1), k == 0 ? 2 : 3);
-  CU(cudaMemcpyAsync(P.U1, Sk(0), bD, cudaMemcpyDeviceToDevice, g->stream));
-  if (g->n_ext > 0) {
-    Ctx Cm = base;
-    Cm.ut0 = P.U1;
-    RUN(KLSA, 0, nb, nt, run_ext_iter, D, LN(g, nb, nt), Cm, S, l, Sk(g->n_ext), (float *)nullptr, 1);
-  }
-  CU(cudaMemcpyAsync(P.PHI0, phi_n, b1, cudaMemcpyDeviceToDevice, g->stream));
-  Ctx A = base;
-  A.phi = P.PHI0;
-  A.p1 = P.A1;
-  A.p2 = P.A2;
-  A.ut0 = P.U1;
-  for (int st = 1; st <= 3; ++st) RUN(KLSA, 0, nb, nt, run_adv_stage, D, LN(g, nb, nt), A, S, l, st);
-  const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
-  Ctx Rt = base;
-  Rt.phi = P.PS;
-  Rt.p1 = P.R1;
-  Rt.p2 = P.R2;
-  Rt.frozen = P.FR;
-  Rt.s0 = P.SS;
-  if (rein) {
-    CU(cudaMemcpyAsync(P.PS, P.PHI0, b1, cudaMemcpyDeviceToDevice, g->stream));
-    RUN(KLSA, 0, nb, nt, run_reinit_prep, Q, LN(g, nb, nt), Rt, S, l);
-    Ctx Rs = Rt;
-    Rs.phi = P.PHI0;
-    for (int st = 1; st <= 3; ++st) RUN(KLSA, 0, nb, nt, run_reinit_stage, D, LN(g, nb, nt), Rs, S, l, st);
-  }
-  Ctx Gm = base;
-  Gm.phi = phi_n;
+  RUN(KLSA, 0, 1, 128, run_lsa_init, Q, LN(g, DYN_GRID, 128), R, l, F, ut_n);
+  Ctx Gm = R;
   Gm.nvec = P.NV;
   Gm.kappa = P.KP;
   RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l, 0);
-  // ---- transposes
-  float *LPin = P.LP[cur], *LPout = P.LP[1 - cur], *LUin = P.LU[cur], *LUout = P.LU[1 - cur];
-  const float *lps = LPin;
-  if (rein) {
-    CU(cudaMemcpyAsync(P.L0r, LPin, b1, cudaMemcpyDeviceToDevice, g->stream));
-    CU(cudaMemsetAsync(P.LS0, 0, b1, g->stream));
-    RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), Rt, S, l, 0, 1, LPin, P.L0r, P.L1, P.L2, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_reinit_rt, D, LN(g, nb, nt), Rt, S, l, P.R2, LPin, 2.0f / 3.0f, P.L2, P.L0r, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), Rt, S, l, 1, 1, LPin, P.L0r, P.L1, P.L2, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_reinit_rt, D, LN(g, nb, nt), Rt, S, l, P.R1, P.L2, 0.25f, P.L1, P.L0r, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), Rt, S, l, 2, 1, LPin, P.L0r, P.L1, P.L2, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_reinit_rt, D, LN(g, nb, nt), Rt, S, l, P.PS, P.L1, 1.0f, P.L0r, P.L0r, P.LS0);
-    RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), Rt, S, l, 3, 1, LPin, P.L0r, P.L1, P.L2, P.LS0);
-    lps = P.L0r;
-  }
-  Ctx At = base;
-  At.phi = phi_n;
-  At.p1 = P.A1;
-  At.p2 = P.A2;
-  At.ut0 = P.U1;
-  CU(cudaMemcpyAsync(LPout, lps, b1, cudaMemcpyDeviceToDevice, g->stream));
-  CU(cudaMemcpyAsync(P.LA, LUin, bD, cudaMemcpyDeviceToDevice, g->stream));
-  RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), At, S, l, 0, 0, lps, LPout, P.L1, P.L2, P.LS0);
-  RUN(KLSA, 0, nb, nt, run_lsa_adv_rt, D, LN(g, nb, nt), At, S, l, P.A2, lps, 2.0f / 3.0f, P.L2, LPout, P.LA);
-  RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), At, S, l, 1, 0, lps, LPout, P.L1, P.L2, P.LS0);
-  RUN(KLSA, 0, nb, nt, run_lsa_adv_rt, D, LN(g, nb, nt), At, S, l, P.A1, P.L2, 0.25f, P.L1, LPout, P.LA);
-  RUN(KLSA, 0, nb, nt, run_lsa_mix, D, LN(g, nb, nt), At, S, l, 2, 0, lps, LPout, P.L1, P.L2, P.LS0);
-  RUN(KLSA, 0, nb, nt, run_lsa_adv_rt, D, LN(g, nb, nt), At, S, l, (const float *)phi_n, P.L1, 1.0f, LPout, LPout,
-      P.LA);
-  float *Lc = P.LA;
-  if (g->n_ext > 0) {
-    CU(cudaMemsetAsync(P.LOFF, 0, bD, g->stream));
-    for (int k = g->n_ext - 1; k >= 0; --k) {
-      float *out = Lc == P.LK[0] ? P.LK[1] : P.LK[0];
-      CU(cudaMemcpyAsync(out, Lc, bD, cudaMemcpyDeviceToDevice, g->stream));
-      RUN(KLSA, 0, nb, nt, run_lsa_ext_T, D, LN(g, nb, nt), E, S, l, (const float *)Sk(k), (const float *)Sk(0),
-          (const float *)Lc, out, P.LOFF, P.LV);
-      Lc = out;
-    }
-    RUN(KLSA, 0, nb, nt, run_lsa_ext_v, D, LN(g, nb, nt), E, S, l, P.LV, LPout);
-    RUN(KLSA, 0, 1, 256, run_lsa_axpy, LN(g, 152 * 8, 256), (long long)D * NF, (const float *)P.LOFF, Lc);
-  }
-  RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, Lc, g->d_madj, LPout);
-  CU(cudaMemcpyAsync(LUout, Lc, bD, cudaMemcpyDeviceToDevice, g->stream));
-  // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LPout
-  const GeoAdj G{LPout, g->d_gn, g->d_gk};
+  const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
+  RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, g->band_est[l]), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
+      g->d_bar + 2);
+  RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, P.A.LU, g->d_madj, P.A.LP);
+  // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LP
+  const GeoAdj G{P.A.LP, g->d_gn, g->d_gk};
   TRY(adj_lb(g, l, F, lamN, lamO, G, phi_n, P.NV, P.KP));
+  // (clears the normals' and curvatures' adjoints as it reads them)
   RUN(KADJ_GEOM, 0, 1, 128, run_adj_geometry, D, LN(g, DYN_GRID, 128), R, l, G);
-  CU(cudaMemsetAsync(g->d_gn, 0, bD, g->stream));
-  CU(cudaMemsetAsync(g->d_gk, 0, b1, g->stream));
   return LSB_OK;
 }
 
@@ -1384,8 +1297,7 @@ lsb_status adj_amr(lsb_grid *g, int l, int call, GeoAdj G) {
   }
   if (last && g->rec_moving) {  // finest sub-step with the level set transported
     float *t = g->tape_ls[call];
-    TRY(adj_moving(g, l, Fold, t, t + g->nfine, lamN, lamO, g->lspar));
-    g->lspar ^= 1;
+    TRY(adj_moving(g, l, Fold, t, t + g->nfine, lamN, lamO));
   } else {
     TRY(adj_lb(g, l, Fold, lamN, lamO, G));
   }
@@ -1416,7 +1328,6 @@ lsb_status backward_amr(lsb_grid *g, GeoAdj G) {
   const size_t sl = slot_floats(g), sf = state_floats(g), NF = g->nfine;
   TRY(amr_buffers(g));
   for (int l = 0; l < MAXL; ++l) g->apar[l] = 0;
-  g->lspar = 0;
   // a stored state: every level's populations, and with a moving level set phi and u~ after
   // them; a loaded one is reclassified (interface geometry and lists of its phi)
   auto save = [&](float *dst) -> lsb_status {
@@ -1892,7 +1803,7 @@ lsb_status lsb_get_fields(lsb_grid *g, int case_idx, int field, int level, void 
     case LSB_FIELD_ADJ_UEXT:
       if (g->adj_cur < 0 || !g->rec_moving)
         return fail(g, LSB_ESTATE, "no u~ adjoint: lsb_backward over a moving level set first");
-      src = lsa_ptrs(g).LU[g->adj_cur] + L.fine_off;
+      src = lsa_ptrs(g).A.LU + L.fine_off;
       planes = g->D;
       plane_stride = g->nfine;
       break;
@@ -2162,7 +2073,7 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
   TRY(observables_pass(g, C, S, stride));
   // the objective's direct dependence on phi (smoothed indicator): into the level set's
   // adjoint at the end of the window (moving), or into dJ/dphi (frozen)
-  float *lphi = g->obj_eps > 0.f ? (mv ? lsa_ptrs(g).LP[0] : (dJ_dphi0 ? g->d_gphi : nullptr)) : nullptr;
+  float *lphi = g->obj_eps > 0.f ? (mv ? lsa_ptrs(g).A.LP : (dJ_dphi0 ? g->d_gphi : nullptr)) : nullptr;
   RUN(KADJ_SEED, 0, g->leaf.n, g->nthreads, run_adj_seed, Q, LN(g, std::min(g->leaf.n, 152 * 8), g->nthreads), C,
       S, (const int *)g->leaf.d, g->leaf.n, (const float *)g->d_fsave, g->d_adj[0], g->d_wobs, g->d_obs, stride,
       g->obj_eps, lphi);
@@ -2208,7 +2119,7 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
     g->d_buf[1] = bufs[1];
     for (int j = len - 1; j >= 0 && st == LSB_OK; --j) {
       float *slot = g->d_seg + sl * j;
-      st = mv ? adj_moving(g, 0, slot, slot + sf, slot + sf + NF, g->d_adj[cur], g->d_adj[1 - cur], cur)
+      st = mv ? adj_moving(g, 0, slot, slot + sf, slot + sf + NF, g->d_adj[cur], g->d_adj[1 - cur])
               : adj_step(g, slot, cur, G);
       cur ^= 1;
     }
@@ -2236,7 +2147,7 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
   if (dJ_dphi0) {
     const float *src = g->d_gphi;
     if (mv) {
-      src = lsa_ptrs(g).LP[amr ? g->lspar : cur];  // the adjoint of phi_0 through every pass
+      src = lsa_ptrs(g).A.LP;  // the adjoint of phi_0 through every pass
     } else {
       // normal and curvature adjoints through the least-squares fit, then the dense boxes
       Ctx C2 = make_ctx(g);
@@ -2258,7 +2169,7 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
   std::vector<double> h((size_t)NG_ADJ * g->ncase);
   CU(cudaMemcpyAsync(h.data(), g->d_grad, sizeof(double) * h.size(), cudaMemcpyDeviceToHost, g->stream));
   TRY(lsb_sync(g));
-  g->adj_cur = amr ? g->lspar : cur;  // with a moving level set on several levels: LU[lspar]
+  g->adj_cur = amr ? 0 : cur;
   if (!amr) g->apar[0] = cur;
   if (dJ_dparams) {
     for (int c = 0; c < g->ncase; ++c) {

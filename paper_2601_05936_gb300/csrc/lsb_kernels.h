@@ -98,11 +98,6 @@ cudaError_t run_export_noalloc(int Q, int st, Launch L, Ctx C, int ld, int field
 cudaError_t run_classify_phase(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, int glevel, int init);
 cudaError_t run_classify_links(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, int glevel, int full);
 cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel, int which);
-cudaError_t run_ext_init(int Q, Launch L, Ctx C, int glevel);
-cudaError_t run_ext_iter(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *uin, float *uout, int mode);
-cudaError_t run_adv_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage);
-cudaError_t run_reinit_prep(int Q, Launch L, Ctx C, BlockShape S, int glevel);
-cudaError_t run_reinit_stage(int D, Launch L, Ctx C, BlockShape S, int glevel, int stage);
 // The level-set update and the classification's phase and link passes of a finest sub-step
 // in one launch (see k_levelset_fused).  LsfLimits: what the device allows (kmax slots of
 // 1024 threads in shared memory, CTAs of a cooperative launch or 0, largest cluster);
@@ -161,16 +156,18 @@ cudaError_t run_adj_restrict(int Q, Launch L, Ctx C, const int2 *cells, int n, c
 // lsb_adj_ls.cu: adjoint of the level-set passes of a step with a moving interface
 cudaError_t run_lsa_init(int Q, Launch L, Ctx C, int glevel, const float *F, float *U0);
 cudaError_t run_lsa_init_T(int Q, Launch L, Ctx C, int glevel, const float *F, float *LS0, float *MA, float *LPHI);
-cudaError_t run_lsa_mix(int D, Launch L, Ctx C, BlockShape S, int glevel, int mode, int use_frozen, const float *L3,
-                        float *L0, float *L1, float *L2, const float *Ls0);
-cudaError_t run_lsa_reinit_rt(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *pin, const float *MU,
-                              float scale, float *Lt, float *L0, float *Ls0);
-cudaError_t run_lsa_adv_rt(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *pin, const float *MU,
-                           float scale, float *Lt, float *L0, float *LU);
-cudaError_t run_lsa_ext_T(int D, Launch L, Ctx C, BlockShape S, int glevel, const float *Sk, const float *S0,
-                          const float *Lin, float *Lout, float *LOFF, float *LV);
-cudaError_t run_lsa_ext_v(int D, Launch L, Ctx C, BlockShape S, int glevel, float *LV, float *LPHI);
-cudaError_t run_lsa_axpy(Launch L, long long n, const float *x, float *y);
+// Arrays of the level-set part of the reverse sweep (finest-level planes; u~ holds D of them):
+// S0 the step's starting u~ with the interface cells' new values, S the sweeps' results 1 ..
+// n_ext, A1, A2 / R1, R2 the transport's and reinitialisation's stages, PB phi_n of the band, SS
+// and FR S(phi*) and the frozen cells; LP, LU the adjoints of phi and u~ (in place), LS0 d/dS;
+// L1, L2, LK0, LK1, LV collect adjoints within a sub-step and are zero between sub-steps.
+struct LsaScratch {
+  float *S0, *S, *A1, *A2, *R1, *R2, *PB, *SS;
+  uint8_t *FR;
+  float *LP, *LU, *L1, *L2, *LS0, *LK0, *LK1, *LV;
+};
+cudaError_t run_lsa_levelset(int Q, Launch L, Ctx C, BlockShape S, int glevel, int n_ext, int rein, LsaScratch A,
+                             unsigned *bar);
 cudaError_t run_lsa_flipflag(Launch L, const int *counters, int glevel, int *flag);
 
 }  // namespace lsb
