@@ -1208,7 +1208,7 @@ lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *u
   Ctx Gm = R;
   Gm.nvec = P.NV;
   Gm.kappa = P.KP;
-  RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l, 0);
+  RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l);
   const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
   RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, g->band_est[l]), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
       g->d_bar + 2);

@@ -97,7 +97,7 @@ cudaError_t run_export_noalloc(int Q, int st, Launch L, Ctx C, int ld, int field
 // lsb_ls.cu: level set, classification, geometry, refill, sensor
 cudaError_t run_classify_phase(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, int glevel, int init);
 cudaError_t run_classify_links(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, int glevel, int full);
-cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel, int which);
+cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel);
 // The level-set update and the classification's phase and link passes of a finest sub-step
 // in one launch (see k_levelset_fused).  LsfLimits: what the device allows (kmax slots of
 // 1024 threads in shared memory, CTAs of a cooperative launch or 0, largest cluster);
@@ -113,8 +113,8 @@ cudaError_t prepare_levelset_fused(int Q, LsfLimits *out);
 cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n);
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
                                unsigned *bar);
-// the curvature fit of the interface and flipped cells on CTAs [0, gg) (each flipped cell
-// then refilled when refill is set) and the band pass on the rest, one launch
+// the flipped cells (fit, and refill when refill is set), the curvature fit of the interface
+// cells on gg CTAs and the band pass on the other CTAs of L.grid, one launch
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,
                               int refill);
 cudaError_t run_levelset_persistent(int Q, Launch L, Ctx C, BlockShape S, int glevel, int n_ext, int reinit,

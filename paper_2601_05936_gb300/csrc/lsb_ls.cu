@@ -300,26 +300,60 @@ __device__ __forceinline__ void d_band(const Ctx &C, const int *list, int nlist,
 // H_ab = sum(o_a o_b phi)/sum(o_a^2 o_b^2) (a != b); the constant and pure
 // quadratic coefficients solve the 1 + D even normal equations in closed form.
 // n = g/|g|, kappa = (|g|^2 tr H - g.H.g)/|g|^3.
-// which: 0 the interface list, 1 the flip list, 2 both (one index space, interface
-// cells first; a cell on both lists gets the same values twice).
-// On the CTAs [b0, b0 + nb) of the launch; post(it) runs after the fit of each flipped cell.
-template <int D, typename Post>
-__device__ __forceinline__ void d_geometry(const Ctx &C, int glevel, int which, int b0, int nb, Post post) {
-  const int ni = which == 1 ? 0 : min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
-  const int nf = which == 0 ? 0 : min(C.counters[glevel * NCOUNT + 2], (int)C.list_cap);
+// The fit from the stencil sums (exact integers in units of 2^-30): n and kappa.
+// The fit's coefficients are fixed rational combinations of the stencil sums.  In 2D
+// (9 points: sum o^2 = 6, sum o_x^2 o_y^2 = 4, sum o^4 = 6) g_a = S_a / 6, H_aa =
+// (3 S_aa - 2 P) / 3, H_xy = S_xy / 4; in 3D (27 points: 18, 12, 18) g_a = S_a / 18,
+// H_aa = (3 S_aa - 2 P) / 9, H_ab = S_ab / 12.  In the unit 1 / (12 * 2^30) (2D) or
+// 1 / (36 * 2^30) (3D) both read g = 2 G and H = K with the integers G_a = S_a,
+// K_aa = 4 (3 S_aa - 2 P), K_ab = 3 S_ab, and kappa, homogeneous of degree zero in
+// (g, H), is (|G|^2 tr K - G.K.G) / (2 |G|^3): float64 from exact integers, one
+// square root and two divisions.
+template <int D>
+__device__ __forceinline__ void fit_from_sums(long long iP, const long long isx[3], const long long isxx[3],
+                                              const long long isxy[3], float n[3], float &kappa) {
+  double G[3] = {0, 0, 0}, K[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
+  for (int a = 0; a < D; ++a) {
+    G[a] = (double)isx[a];
+    K[a][a] = (double)(4 * (3 * isxx[a] - 2 * iP));
+  }
+  K[0][1] = K[1][0] = (double)(3 * isxy[0]);
+  if (D == 3) {
+    K[0][2] = K[2][0] = (double)(3 * isxy[1]);
+    K[1][2] = K[2][1] = (double)(3 * isxy[2]);
+  }
+  double g2 = 0, tr = 0, gKg = 0;
+  for (int a = 0; a < D; ++a) {
+    g2 += G[a] * G[a];
+    tr += K[a][a];
+    for (int b = 0; b < D; ++b) gKg += G[a] * K[a][b] * G[b];
+  }
+  const double mag = sqrt(g2);
+  n[0] = n[1] = n[2] = 0.f;
+  kappa = 0.f;
+  // |grad phi| = |G| / (6 or 18) / 2^30
+  if (mag > 1e-12 * (D == 2 ? 6.0 : 18.0) * 1073741824.0) {
+    const double inv = 1.0 / mag;
+    for (int a = 0; a < D; ++a) n[a] = (float)(G[a] * inv);
+    kappa = (float)((g2 * tr - gKg) / (2.0 * g2 * mag));
+  }
+}
+// phi in fixed point with 30 fraction bits (exact for |phi| >= 2^-6, within 2^-31 below): the
+// stencil sums are exact in 64-bit integers, so the float64 work of the fit is its closed form
+// only (GB300 runs float64 at a small fraction of its integer rate).
+__device__ __forceinline__ long long phi_fixed(float p) { return __float2ll_rn(p * 1073741824.0f); }
+
+// The interface cells, one thread each, on the CTAs [b0, b0 + nb) of the launch.
+template <int D>
+__device__ __forceinline__ void d_geometry(const Ctx &C, int glevel, int b0, int nb) {
+  const int ni = min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
   const int2 *li = C.iface_list + (long long)glevel * C.list_cap;
-  const int2 *lf = C.flip_list + (long long)glevel * C.list_cap;
-  for (int e = ((int)blockIdx.x - b0) * blockDim.x + threadIdx.x; e < ni + nf; e += nb * blockDim.x) {
-    const int2 it = e < ni ? li[e] : lf[e - ni];
+  for (int e = ((int)blockIdx.x - b0) * blockDim.x + threadIdx.x; e < ni; e += nb * blockDim.x) {
+    const int2 it = li[e];
     const LevelDev &L = C.lds[it.x];
     const long long c = it.y;
     int x, y, z;
     cell_xyz(L, c, x, y, z);
-    // Stencil sums exactly: phi (float) in fixed point with 30 fraction bits (exact
-    // for |phi| >= 2^-6, within 2^-31 below), summed in 64-bit integers, then
-    // converted to float64 (exact below 2^53).  This keeps the float64 work of the
-    // fit to the closed-form solve; GB300 runs float64 at a small fraction of its
-    // integer rate.
     long long iP = 0, isx[3] = {0, 0, 0}, isxx[3] = {0, 0, 0}, isxy[3] = {0, 0, 0};
     // cells whose 3^D stencil lies inside the box read it at direct offsets
     const bool inner = x >= 1 && x + 1 < L.n[0] && y >= 1 && y + 1 < L.n[1] && (D == 2 || (z >= 1 && z + 1 < L.n[2]));
@@ -338,7 +372,7 @@ __device__ __forceinline__ void d_geometry(const Ctx &C, int glevel, int which, 
             const int zz = D == 3 ? clampwrap(L, 2, z + oz) : 0;
             cc = cidx(L, xx, yy, zz);
           }
-          const long long v = __float2ll_rn(C.phi[L.fine_off + cc] * 1073741824.0f);
+          const long long v = phi_fixed(C.phi[L.fine_off + cc]);
           const int o[3] = {ox, oy, oz};
           iP += v;
           for (int a = 0; a < D; ++a) {
@@ -351,48 +385,17 @@ __device__ __forceinline__ void d_geometry(const Ctx &C, int glevel, int which, 
             isxy[2] += oy * oz > 0 ? v : (oy * oz < 0 ? -v : 0);
           }
         }
-    // The fit's coefficients are fixed rational combinations of the stencil sums.  In 2D
-    // (9 points: sum o^2 = 6, sum o_x^2 o_y^2 = 4, sum o^4 = 6) g_a = S_a / 6, H_aa =
-    // (3 S_aa - 2 P) / 3, H_xy = S_xy / 4; in 3D (27 points: 18, 12, 18) g_a = S_a / 18,
-    // H_aa = (3 S_aa - 2 P) / 9, H_ab = S_ab / 12.  In the unit 1 / (12 * 2^30) (2D) or
-    // 1 / (36 * 2^30) (3D) both read g = 2 G and H = K with the integers G_a = S_a,
-    // K_aa = 4 (3 S_aa - 2 P), K_ab = 3 S_ab, and kappa, homogeneous of degree zero in
-    // (g, H), is (|G|^2 tr K - G.K.G) / (2 |G|^3): float64 from exact integers, one
-    // square root and two divisions.
-    double G[3] = {0, 0, 0}, K[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int a = 0; a < D; ++a) {
-      G[a] = (double)isx[a];
-      K[a][a] = (double)(4 * (3 * isxx[a] - 2 * iP));
-    }
-    K[0][1] = K[1][0] = (double)(3 * isxy[0]);
-    if (D == 3) {
-      K[0][2] = K[2][0] = (double)(3 * isxy[1]);
-      K[1][2] = K[2][1] = (double)(3 * isxy[2]);
-    }
-    double g2 = 0, tr = 0, gKg = 0;
-    for (int a = 0; a < D; ++a) {
-      g2 += G[a] * G[a];
-      tr += K[a][a];
-      for (int b = 0; b < D; ++b) gKg += G[a] * K[a][b] * G[b];
-    }
-    const double mag = sqrt(g2);
+    float n[3], kap;
+    fit_from_sums<D>(iP, isx, isxx, isxy, n, kap);
     const long long fc = L.fine_off + c;
-    // |grad phi| = |G| / (6 or 18) / 2^30
-    if (mag > 1e-12 * (D == 2 ? 6.0 : 18.0) * 1073741824.0) {
-      const double inv = 1.0 / mag;
-      for (int a = 0; a < D; ++a) C.nvec[a * C.nfine + fc] = (float)(G[a] * inv);
-      C.kappa[fc] = (float)((g2 * tr - gKg) / (2.0 * g2 * mag));
-    } else {
-      for (int a = 0; a < D; ++a) C.nvec[a * C.nfine + fc] = 0.f;
-      C.kappa[fc] = 0.f;
-    }
-    if (e >= ni) post(it);
+    for (int a = 0; a < D; ++a) C.nvec[a * C.nfine + fc] = n[a];
+    C.kappa[fc] = kap;
   }
 }
 template <int D>
-__global__ void k_geometry(Ctx C, int glevel, int which) {
+__global__ void k_geometry(Ctx C, int glevel) {
   LSB_GRID_WAIT();
-  d_geometry<D>(C, glevel, which, 0, gridDim.x, [](int2) {});
+  d_geometry<D>(C, glevel, 0, gridDim.x);
 }
 
 // ------------------------------------------------------------------ forward passes on mirrored stage arrays
@@ -1212,21 +1215,6 @@ __global__ void k_levelset_persistent(Ctx C, BlockShape S, int glevel, int n_ext
 
 // ------------------------------------------------------------------ refill (Sec. 2.4)
 template <int Q>
-__device__ __forceinline__ void moments_q(const float *f, float &drho, float u[3]) {
-  using LT = Lat<Q>;
-  float d = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
-  for (int i = 0; i < Q; ++i) {
-    d += f[i];
-    jx += LT::cx(i) * f[i];
-    jy += LT::cy(i) * f[i];
-    jz += LT::cz(i) * f[i];
-  }
-  drho = d;
-  const float inv = 1.0f / (1.0f + d);
-  u[0] = jx * inv; u[1] = jy * inv; u[2] = jz * inv;
-}
-
-template <int Q>
 __device__ __forceinline__ float feq_q(int i, float drho, const float u[3]) {
   using LT = Lat<Q>;
   const float cu = LT::cx(i) * u[0] + LT::cy(i) * u[1] + LT::cz(i) * u[2];
@@ -1234,61 +1222,100 @@ __device__ __forceinline__ float feq_q(int i, float drho, const float u[3]) {
   return LT::w(i) * (drho + (1.0f + drho) * (3.0f * cu + 4.5f * cu * cu - 1.5f * usq));
 }
 
-// Refill of one flipped cell (its normal and curvature already fitted).
+// The flipped cells, one warp each, on the CTAs [b0, b0 + nb) of the launch: the curvature fit
+// (lane k takes stencil point k; integer sums, so the order does not matter) and, with refill
+// set, the refill (lane i takes direction i).  A launch that flips a cell waits for that cell's
+// whole chain, so it is spread over lanes and kept short: as one thread per cell after its fit
+// it was ~25 us of loops over the directions (3D bubble, ~5 flips per sub-step; unrolled to
+// issue its loads together it took longer still, all of it instruction fetch).
 template <int Q, typename T>
-__device__ __forceinline__ void refill_cell(const Ctx &C, int2 it) {
+__device__ __forceinline__ void d_flipped(const Ctx &C, int glevel, int refill, int b0, int nb) {
   using LT = Lat<Q>;
-  constexpr int D = LT::D;
-  {
+  constexpr int D = LT::D, NS = D == 3 ? 27 : 9;
+  const unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5;
+  const int nf = min(C.counters[glevel * NCOUNT + 2], (int)C.list_cap);
+  const int2 *lf = C.flip_list + (long long)glevel * C.list_cap;
+  for (int e = ((int)blockIdx.x - b0) * wpb + (threadIdx.x >> 5); e < nf; e += nb * wpb) {
+    const int2 it = lf[e];
     const LevelDev &L = C.lds[it.x];
-    const long long c = it.y;
+    const long long c = it.y, fo = L.fine_off;
     int x, y, z;
     cell_xyz(L, c, x, y, z);
-    const long long fo = L.fine_off, NF = C.nfine, N = L.ncell;
+    // ---- fit
+    const int ox = lane % 3 - 1, oy = (lane / 3) % 3 - 1, oz = D == 3 ? lane / 9 - 1 : 0;
+    long long v = 0;
+    if (lane < NS)
+      v = phi_fixed(C.phi[fo + cidx(L, clampwrap(L, 0, x + ox), clampwrap(L, 1, y + oy),
+                                    D == 3 ? clampwrap(L, 2, z + oz) : 0)]);
+    auto sum = [&](int s) {  // sum of s v over the stencil, s = -1, 0, 1
+      long long r = s > 0 ? v : (s < 0 ? -v : 0);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) r += __shfl_xor_sync(all, r, o);
+      return r;
+    };
+    const long long iP = sum(1), isx[3] = {sum(ox), sum(oy), sum(oz)}, isxx[3] = {sum(ox * ox), sum(oy * oy), sum(oz * oz)},
+                    isxy[3] = {sum(ox * oy), sum(ox * oz), sum(oy * oz)};
+    float n[3], kap;
+    fit_from_sums<D>(iP, isx, isxx, isxy, n, kap);
+    if (lane < D) C.nvec[lane * C.nfine + fo + c] = lane == 0 ? n[0] : (lane == 1 ? n[1] : n[2]);
+    if (lane == 0) C.kappa[fo + c] = kap;
+    if (!refill) continue;
+    // ---- refill
+    const long long N = L.ncell;
     T *Bf = fB<T, Q>(C, L);
-    const uint8_t tg = C.tag[L.cell_off + c];
+    const uint8_t *tagL = C.tag + L.cell_off;
+    const uint8_t tg = tagL[c];
     const int Pn = tg & TAG_GAS;
     const int Po = (tg & TAG_PREVGAS) ? 1 : 0;
     const float sg = Pn == 0 ? 1.0f : -1.0f;
-    float mvec[3] = {0.f, 0.f, 0.f};
-    for (int a = 0; a < D; ++a) mvec[a] = -sg * C.nvec[a * NF + fo + c];  // into the new phase
     auto valid_new = [&](int tx, int ty, int tz, long long &ct) -> bool {
       if (!(wrap(L, 0, tx) && wrap(L, 1, ty) && (D == 2 || wrap(L, 2, tz)))) return false;
       ct = cidx(L, tx, ty, tz);
-      const uint8_t tt = C.tag[L.cell_off + ct];
-      const int g = tt & TAG_GAS, pg = (tt & TAG_PREVGAS) ? 1 : 0;
-      return (tt & TAG_LEAF) && g == Pn && pg == Pn;
+      const uint8_t tt = tagL[ct];
+      return (tt & TAG_LEAF) && (tt & TAG_GAS) == Pn && ((tt & TAG_PREVGAS) ? 1 : 0) == Pn;
     };
-    int best = -1;
-    float bestv = -1e30f;
-    for (int i = 0; i < Q; ++i) {
-      if (i == LT::REST) continue;
-      long long ct;
-      if (!valid_new(x + LT::cx(i), y + LT::cy(i), z + LT::cz(i), ct)) continue;
-      const float nrm = sqrtf((float)(LT::cx(i) * LT::cx(i) + LT::cy(i) * LT::cy(i) + LT::cz(i) * LT::cz(i)));
-      const float v = (LT::cx(i) * mvec[0] + LT::cy(i) * mvec[1] + LT::cz(i) * mvec[2]) / nrm;
-      if (v > bestv) {
-        bestv = v;
+    // e_min: the largest e.m / |e|, m = the normal into the new phase; ties to the lowest index
+    const int i = lane < Q ? lane : LT::REST;
+    const int ci = LT::cx(i), cj = LT::cy(i), ck = LT::cz(i);
+    long long ct = c;
+    float bv = -1e30f;
+    int best = Q;
+    if (i != LT::REST && valid_new(x + ci, y + cj, z + ck, ct)) {
+      const float mvec[3] = {-sg * n[0], -sg * n[1], D == 3 ? -sg * n[2] : 0.f};
+      const float nrm = sqrtf((float)(ci * ci + cj * cj + ck * ck));
+      const float w = (ci * mvec[0] + cj * mvec[1] + ck * mvec[2]) / nrm;
+      if (w > bv) {
+        bv = w;
         best = i;
       }
     }
-    if (best < 0) {
-      for (int i = 0; i < Q; ++i) Store<T>::st(Bf + i * N + c, 0.0f, C.fp16_scale);
-      return;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float ov = __shfl_xor_sync(all, bv, o);
+      const int ob = __shfl_xor_sync(all, best, o);
+      if (ov > bv || (ov == bv && ob < best)) {
+        bv = ov;
+        best = ob;
+      }
+    }
+    if (best >= Q) {
+      if (lane < Q) Store<T>::st(Bf + i * N + c, 0.0f, C.fp16_scale);
+      continue;
     }
     const int ex = LT::cx(best), ey = LT::cy(best), ez = LT::cz(best);
+    const long long c1 = __shfl_sync(all, ct, best);
+    long long c2 = c;
+    const bool quad = valid_new(x + 2 * ex, y + 2 * ey, z + 2 * ez, c2);
     const float phr = C.phi[fo + c];
     float q = 0.5f;
     {
       int bx = x - ex, by = y - ey, bz = z - ez;
       if (wrap(L, 0, bx) && wrap(L, 1, by) && (D == 2 || wrap(L, 2, bz))) {
         const long long cb = cidx(L, bx, by, bz);
-        if ((C.tag[L.cell_off + cb] & TAG_GAS) != Pn) q = phr / (phr - C.phi[fo + cb]);
+        if ((tagL[cb] & TAG_GAS) != Pn) q = phr / (phr - C.phi[fo + cb]);
       }
     }
-    long long c1 = 0, c2 = 0;
-    valid_new(x + ex, y + ey, z + ez, c1);
-    const bool quad = valid_new(x + 2 * ex, y + 2 * ey, z + 2 * ez, c2);
     float w0, w1, w2;
     if (quad) {
       w0 = 2.0f / ((q + 1.0f) * (q + 2.0f));
@@ -1299,49 +1326,58 @@ __device__ __forceinline__ void refill_cell(const Ctx &C, int2 it) {
       w1 = q / (1.0f + q);
       w2 = 0.0f;
     }
-    float fo_[Q], f1[Q];
-    for (int i = 0; i < Q; ++i) {
-      fo_[i] = Store<T>::ld(Bf + i * N + c, C.fp16_inv);
-      f1[i] = Store<T>::ld(Bf + i * N + c1, C.fp16_inv);
+    const float f_old = Store<T>::ld(Bf + i * N + c, C.fp16_inv), f_1 = Store<T>::ld(Bf + i * N + c1, C.fp16_inv);
+    const float f_2 = Store<T>::ld(Bf + i * N + c2, C.fp16_inv);
+    // moments of the three cells, summed in the order of the populations
+    float d[3] = {0.f, 0.f, 0.f}, jx[3] = {0.f, 0.f, 0.f}, jy[3] = {0.f, 0.f, 0.f}, jz[3] = {0.f, 0.f, 0.f};
+#pragma unroll 1
+    for (int k = 0; k < Q; ++k) {
+      const float a = (float)LT::cx(k), b = (float)LT::cy(k), g = (float)LT::cz(k);
+      const float fk[3] = {__shfl_sync(all, f_old, k), __shfl_sync(all, f_1, k), __shfl_sync(all, f_2, k)};
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        d[m] += fk[m];
+        jx[m] += a * fk[m];
+        jy[m] += b * fk[m];
+        jz[m] += g * fk[m];
+      }
     }
-    float r_old, u_old[3], r1, u1[3];
-    moments_q<Q>(fo_, r_old, u_old);
-    moments_q<Q>(f1, r1, u1);
-    const float p_gamma = L.rho_phys[Po] * CS2 * r_old + L.sigma * sg * C.kappa[fo + c];
+    float u_old[3], u1[3], u2[3];
+    auto velocity = [&](int m, float u[3]) {
+      const float inv = 1.0f / (1.0f + d[m]);
+      u[0] = jx[m] * inv; u[1] = jy[m] * inv; u[2] = jz[m] * inv;
+    };
+    velocity(0, u_old);
+    velocity(1, u1);
+    const float p_gamma = L.rho_phys[Po] * CS2 * d[0] + L.sigma * sg * kap;
     const float r_g = p_gamma / (L.rho_phys[Pn] * CS2);
-    float rr = w0 * r_g + w1 * r1;
+    float rr = w0 * r_g + w1 * d[1];
     float ur[3];
     for (int a = 0; a < 3; ++a) ur[a] = w0 * u_old[a] + w1 * u1[a];
     if (quad) {
-      float f2[Q], r2, u2[3];
-      for (int i = 0; i < Q; ++i) f2[i] = Store<T>::ld(Bf + i * N + c2, C.fp16_inv);
-      moments_q<Q>(f2, r2, u2);
-      rr += w2 * r2;
+      velocity(2, u2);
+      rr += w2 * d[2];
       for (int a = 0; a < 3; ++a) ur[a] += w2 * u2[a];
     }
-    for (int i = 0; i < Q; ++i) {
-      const float v = feq_q<Q>(i, rr, ur) + (f1[i] - feq_q<Q>(i, r1, u1));
-      Store<T>::st(Bf + i * N + c, v, C.fp16_scale);
-    }
+    if (lane < Q)
+      Store<T>::st(Bf + i * N + c, feq_q<Q>(i, rr, ur) + (f_1 - feq_q<Q>(i, d[1], u1)), C.fp16_scale);
   }
 }
 
-// The classification's last passes in one launch: the curvature fit of the interface and
-// flipped cells (CTAs [0, gg): the longer chain per thread, scheduled first) and the band
-// (the rest, a warp per finest block), which read nothing of each other's; with refill
-// set, each flipped cell is refilled by the thread that fitted it (the refill reads the
-// fit at its own cell only, and neighbours of the new phase that did not flip).
+// The classification's last passes in one launch, which read nothing of each other's: the
+// flipped cells (CTAs [0, kFlipCtas), a warp per cell: the longest chain, scheduled first), the
+// curvature fit of the interface cells (the next gg) and the band (the rest, a warp per finest
+// block).  The refill reads the fit at its own cell, and neighbours of the new phase that did
+// not flip; a cell on both lists gets the same fit twice.
+constexpr int kFlipCtas = 16;
 template <int Q, typename T>
 __global__ void k_post_classify(Ctx C, const int *list, int nlist, int glevel, int gg, int refill) {
   LSB_GRID_WAIT();
   constexpr int D = Lat<Q>::D;
-  if ((int)blockIdx.x >= gg) {
-    d_band<Q>(C, list, nlist, glevel, gg, (int)gridDim.x - gg);
-  } else if (refill) {
-    d_geometry<D>(C, glevel, 2, 0, gg, [&](int2 it) { refill_cell<Q, T>(C, it); });
-  } else {
-    d_geometry<D>(C, glevel, 2, 0, gg, [](int2) {});
-  }
+  const int b = (int)blockIdx.x;
+  if (b < kFlipCtas) d_flipped<Q, T>(C, glevel, refill, 0, kFlipCtas);
+  else if (b < kFlipCtas + gg) d_geometry<D>(C, glevel, kFlipCtas, gg);
+  else d_band<Q>(C, list, nlist, glevel, kFlipCtas + gg, (int)gridDim.x - gg - kFlipCtas);
 }
 
 // ------------------------------------------------------------------ refinement sensor
@@ -1426,7 +1462,7 @@ cudaError_t run_classify_phase(int Q, Launch L, Ctx C, BlockShape S, const int *
 cudaError_t run_classify_links(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, int glevel, int full) {
   LQ(k_classify_links, C, S, list, n, glevel, full);
 }
-cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel, int which) { LD(k_geometry, C, glevel, which); }
+cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel) { LD(k_geometry, C, glevel); }
 // Shared memory of the one-launch level-set update.
 size_t lsf_smem(int D, int kcap) { return (D == 2 ? sizeof(LsfSlot<2>) : sizeof(LsfSlot<3>)) * (size_t)kcap; }
 cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n) {
@@ -1516,6 +1552,7 @@ cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, 
 }
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,
                               int refill) {
+  L.grid += kFlipCtas;
   if (Q == 9) {
     if (st == 0) launcher(k_post_classify<9, float>, L, 0)(C, list, n, glevel, gg, refill);
     else launcher(k_post_classify<9, __half>, L, 0)(C, list, n, glevel, gg, refill);
