@@ -672,7 +672,8 @@ lsb_status coarse_side(lsb_grid *g, int l) {
   CU(cudaEventRecord(g->ev_fork[l], g->stream));
   CU(cudaStreamWaitEvent(g->side[l], g->ev_fork[l], 0));
   const CellList &rc = g->rl_cells[l];
-  RUN(2, 0, rc.n, 128, run_restrict_cells, Q, st, (Launch{(rc.n + 127) / 128, 128, g->side[l]}), C,
+  // (at the step's own priority: it is short and the collide behind it waits for it)
+  RUN(2, 0, rc.n, 128, run_restrict_cells, Q, st, (Launch{1, 32, g->side[l], 0, LSB_PRIO ? g->prio_hi : 0}), C,
       (const int2 *)rc.d, rc.n);
   const double cs_bytes = 2.0 * g->Q * (g->storage == LSB_FP32 ? 4 : 2) * g->leaf_cells[l];
   const int grid = std::min(g->cs[l].n, std::max(1, g->tma_grid / LSB_SIDE_DIV));
@@ -683,12 +684,6 @@ lsb_status coarse_side(lsb_grid *g, int l) {
   return LSB_OK;
 }
 
-// The first sub-step's ghost ring of the deepest level on its side stream beside that
-// sub-step's collide (which takes its blocks dynamically, so the ring's CTAs cost it only
-// their share): 0.803 -> 0.799 ms per step.
-#ifndef LSB_RING0_SIDE
-#define LSB_RING0_SIDE 1
-#endif
 // One advance of global level l (recursive over finer levels).
 lsb_status advance(lsb_grid *g, int l) {
   BlockShape S = shape(g);
@@ -708,7 +703,7 @@ lsb_status advance(lsb_grid *g, int l) {
   if (fork) {
     TRY(coarse_side(g, l));
   } else {
-    RUN(2, 0, rc.n, 128, run_restrict_cells, Q, st, LN(g, (rc.n + 127) / 128, 128), C, (const int2 *)rc.d, rc.n);
+    RUN(2, 0, rc.n, 128, run_restrict_cells, Q, st, LN(g, 1, 32), C, (const int2 *)rc.d, rc.n);
   }
   const int call = g->tape_on ? g->tape_call++ : -1;
   if (call >= 0) TRY(copy_level(g, g->tape_old[call], (const float *)g->d_buf[g->par[l]], l));
@@ -739,7 +734,7 @@ lsb_status advance(lsb_grid *g, int l) {
     // for that level's collide on side[l - 1]
     g->early_fill = -1;  // (the side stream and its events are made by the coarser level)
     CU(cudaEventRecord(g->ev_free[l], g->stream));
-    if (LSB_RING0_SIDE) CU(cudaStreamWaitEvent(g->stream, g->ev_ring0_done[l], 0));  // this sub-step's ring
+    CU(cudaStreamWaitEvent(g->stream, g->ev_ring0_done[l], 0));  // this sub-step's ring
     CU(cudaStreamWaitEvent(g->side2[l], g->ev_free[l], 0));
     CU(cudaStreamWaitEvent(g->side2[l], g->ev_join[l - 1], 0));
     Ctx C2 = make_ctx(g);
@@ -775,10 +770,12 @@ lsb_status advance(lsb_grid *g, int l) {
         CU(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     }
     for (int sub = 0; sub < 2; ++sub) {
-      if (sub == 0 && early && LSB_RING0_SIDE) {
+      if (sub == 0 && early) {
         // the first sub-step's ring (theta = 0) reads only the coarser level's A buffer at
         // leaf cells and writes pushes into the finer B buffer that no leaf pushes to: it
-        // runs beside that sub-step's collide-and-stream, joined before its interface pass
+        // runs beside that sub-step's collide-and-stream, joined before its interface pass.
+        // (The second beside the second sub-step's collide, instead of the first's interface and
+        // level-set passes: 746 -> 751 us per step of the 3D bubble, 472 -> 479 with FP16.)
         CU(cudaEventRecord(g->ev_ring0[l + 1], g->stream));
         CU(cudaStreamWaitEvent(g->side2[l + 1], g->ev_ring0[l + 1], 0));
         C = make_ctx(g);

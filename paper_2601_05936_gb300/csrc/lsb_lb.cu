@@ -1169,41 +1169,6 @@ __global__ void k_collect(Ctx C, BlockShape S, const int *list, int nlist, int b
   }
 }
 
-// Restriction layer from a cell list (one thread per covered cell).
-template <int Q, typename T>
-__global__ void k_restrict_cells(Ctx C, const int2 *cells, int n) {
-  LSB_GRID_WAIT();
-  constexpr int D = Lat<Q>::D;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int2 it = cells[e];
-    const LevelDev &L = C.lds[it.x];
-    const long long c = it.y;
-    int x, y, z;
-    cell_xyz(L, c, x, y, z);
-    const LevelDev &F = C.lds[L.child_ld];
-    const T *Af = fA<T, Q>(C, F);
-    float f[Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) f[i] = 0.f;
-    const int nz = (D == 3) ? 2 : 1;
-    for (int sz = 0; sz < nz; ++sz)
-      for (int sy = 0; sy < 2; ++sy)
-        for (int sx = 0; sx < 2; ++sx) {
-          const long long cf = cidx(F, 2 * x + sx, 2 * y + sy, D == 3 ? 2 * z + sz : 0);
-#pragma unroll
-          for (int i = 0; i < Q; ++i) f[i] += Store<T>::ld(Af + i * F.ncell + cf, C.fp16_inv);
-        }
-    const float inv = 1.0f / (float)(4 * nz);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) f[i] *= inv;
-    const int ph = C.tag[L.cell_off + c] & TAG_GAS;
-    rescale_neq<Q>(f, 2.0f * L.tau[ph] / F.tau[ph]);
-    T *Ac = fA<T, Q>(C, L);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) Store<T>::st(Ac + i * L.ncell + c, f[i], C.fp16_scale);
-  }
-}
-
 // Ghost ring of level F (TAG_GHOST cells), one thread per listed cell: coarse
 // interpolation at time weight theta, f^neq scaled by tau_f / (2 tau_c), a
 // fine-level collision, pushed into the fine leaves that stream from it.
@@ -1266,35 +1231,53 @@ __global__ void LSB_GHOST_LB k_ghost_cells(Ctx C, const int2 *cells, int n, floa
   }
 }
 
-// ------------------------------------------------------------------ restriction, one warp per cell
-// The restriction update with the populations of one covered cell spread over the
-// lanes of a group (population i on lane i; 16 lanes per cell on D2Q9, 32 on
-// D3Q19): the 2^D children's loads of every lane are independent and in flight
-// together instead of one thread walking Q x 2^D loads; the moments are summed
-// over the group with shuffles.  (The ghost ring keeps one thread per cell: there
-// neighbouring cells share their coarse sources, and loads coalesced over cells
-// measured 2.4x faster than this layout.)
+// ------------------------------------------------------------------ restriction, one warp per population
+// The restriction update of 32 listed cells per CTA, warp i holding population i of all of
+// them (lane = cell): the list is sorted, so a warp's cells run along x and its loads of the
+// children (two neighbours in x at once) fill whole sectors; as one warp per cell with a
+// population per lane every 32-byte sector carried two values.  3D bubble, 23.8 k cells: 32 ->
+// 22 us (its shells of cells lie scattered over Q planes of 134 MB), with FP16 storage on the
+// 96 x 96 x 192 box 20 -> 8 us; the step 746 -> 742 and 472 -> 462 us.  The moments are summed in the order of a butterfly over the populations, each by one
+// warp, and go through shared memory.  (D3Q27 has 27 warps of 32; D2Q9 9.)
 template <int Q>
-struct GroupLanes {
-  static constexpr int LPC = Q <= 16 ? 16 : 32;  // lanes per cell
-  static constexpr int GPW = 32 / LPC;           // cells per warp
-};
+constexpr int kRestrictThreads = 32 * Q;
+// Sum of c_a f over the populations of a cell (comp 0: of f), in butterfly order (D3Q27: in
+// their own order).
 template <int Q>
-__device__ __forceinline__ float group_sum(float v) {
+__device__ __forceinline__ float tree_moment(const float (*f)[32], int lane, int comp) {
+  using LT = Lat<Q>;
+  if constexpr (Q == 27) {
+    float r = 0.f;
 #pragma unroll
-  for (int o = GroupLanes<Q>::LPC / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
+    for (int i = 0; i < Q; ++i) {
+      const float x = f[i][lane];
+      r += comp == 0 ? x : (comp == 1 ? LT::cx(i) * x : (comp == 2 ? LT::cy(i) * x : LT::cz(i) * x));
+    }
+    return r;
+  }
+  constexpr int W = Q <= 16 ? 16 : 32;
+  float v[W];
+#pragma unroll
+  for (int i = 0; i < W; ++i) {
+    const float x = i < Q ? f[i < Q ? i : 0][lane] : 0.f;
+    v[i] = i < Q ? (comp == 0 ? x : (comp == 1 ? LT::cx(i) * x : (comp == 2 ? LT::cy(i) * x : LT::cz(i) * x))) : 0.f;
+  }
+#pragma unroll
+  for (int o = W / 2; o > 0; o >>= 1)
+#pragma unroll
+    for (int i = 0; i < o; ++i) v[i] += v[i + o];
+  return v[0];
 }
-// drho and u of the group's populations (lanes past Q hold zero).
-template <int Q>
-__device__ __forceinline__ void group_moments(float f, int cxi, int cyi, int czi, float &drho, float u[3]) {
-  const float d = group_sum<Q>(f), jx = group_sum<Q>(cxi * f), jy = group_sum<Q>(cyi * f);
-  const float jz = Lat<Q>::D == 3 ? group_sum<Q>(czi * f) : 0.f;
-  const float inv = 1.0f / (1.0f + d);
-  drho = d;
-  u[0] = jx * inv;
-  u[1] = jy * inv;
-  u[2] = jz * inv;
+// Two neighbouring stored values in x (the first at an even index).
+__device__ __forceinline__ void ld_pair(const float *p, float, float &a, float &b) {
+  const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+  a = v.x;
+  b = v.y;
+}
+__device__ __forceinline__ void ld_pair(const __half *p, float inv, float &a, float &b) {
+  const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2 *>(p)));
+  a = v.x * inv;
+  b = v.y * inv;
 }
 // Eq. feq deviation of one population, given its velocity and weight.
 __device__ __forceinline__ float feq_lane(float wi, int cxi, int cyi, int czi, float drho, const float u[3]) {
@@ -1304,38 +1287,45 @@ __device__ __forceinline__ float feq_lane(float wi, int cxi, int cyi, int czi, f
 }
 
 template <int Q, typename T>
-__global__ void k_restrict_cells_w(Ctx C, const int2 *cells, int n) {
+__global__ void __launch_bounds__(kRestrictThreads<Q>) k_restrict_cells(Ctx C, const int2 *cells, int n) {
   LSB_GRID_WAIT();
   using LT = Lat<Q>;
-  constexpr int D = LT::D, LPC = GroupLanes<Q>::LPC, GPW = GroupLanes<Q>::GPW;
-  const int lane = threadIdx.x & 31, sub = lane & (LPC - 1);
-  const bool act = sub < Q;
-  const int i = act ? sub : LT::REST;
+  constexpr int D = LT::D;
+  __shared__ float fs[Q][32], mom[4][32];
+  const int lane = threadIdx.x & 31, i = threadIdx.x >> 5;
   const int cxi = LT::cx(i), cyi = LT::cy(i), czi = LT::cz(i);
   const float wi = LT::w(i);
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * blockDim.x) >> 5;
-  for (int e0 = warp * GPW; e0 < n; e0 += nwarps * GPW) {
-    const int e = min(e0 + lane / LPC, n - 1);  // a group past the end repeats the last cell and stores nothing
-    const bool store = act && e0 + lane / LPC < n;
-    const int2 it = cells[e];
+  for (int e0 = blockIdx.x * 32; e0 < n; e0 += gridDim.x * 32) {
+    const bool act = e0 + lane < n;
+    const int2 it = cells[act ? e0 + lane : n - 1];  // a lane past the end repeats the last cell
     const LevelDev &L = C.lds[it.x];
     const unsigned c = (unsigned)it.y, p0 = (unsigned)L.p[0], p1 = (unsigned)L.p[1];
-    const int x = (int)(c % p0), y = (int)((c / p0) % p1), z = (int)(c / (p0 * p1));
+    const unsigned q = c / p0, x = c - q * p0, z = q / p1, y = q - z * p1;
     const LevelDev &F = C.lds[L.child_ld];
     const T *Af = fA<T, Q>(C, F) + (size_t)i * F.ncell;
     const unsigned fp0 = (unsigned)F.p[0], fp01 = (unsigned)(F.p[0] * F.p[1]);
     const unsigned cf0 = 2u * x + fp0 * (2u * y) + (D == 3 ? fp01 * (2u * z) : 0u);
-    float f = 0.f;
-#pragma unroll
-    for (int k = 0; k < (D == 3 ? 8 : 4); ++k)
-      f += Store<T>::ld(Af + (cf0 + (k & 1) + ((k >> 1) & 1) * fp0 + ((k >> 2) & 1) * fp01), C.fp16_inv);
-    f = act ? f * (1.0f / (float)(D == 3 ? 8 : 4)) : 0.f;
     const int ph = C.tag[L.cell_off + c] & TAG_GAS;
-    float drho, u[3];
-    group_moments<Q>(f, cxi, cyi, czi, drho, u);
+    float v[D == 3 ? 8 : 4], f = 0.f;
+#pragma unroll
+    for (int k = 0; k < (D == 3 ? 4 : 2); ++k)
+      ld_pair(Af + (cf0 + (k & 1) * fp0 + (k >> 1) * fp01), C.fp16_inv, v[2 * k], v[2 * k + 1]);
+#pragma unroll
+    for (int k = 0; k < (D == 3 ? 8 : 4); ++k) f += v[k];
+    f *= 1.0f / (float)(D == 3 ? 8 : 4);
+    fs[i][lane] = f;
+    __syncthreads();
+    if (i == 0) mom[0][lane] = tree_moment<Q>(fs, lane, 0);
+    else if (i == 1) mom[1][lane] = tree_moment<Q>(fs, lane, 1);
+    else if (i == 2) mom[2][lane] = tree_moment<Q>(fs, lane, 2);
+    else if (i == 3) mom[3][lane] = D == 3 ? tree_moment<Q>(fs, lane, 3) : 0.f;
+    __syncthreads();
+    const float drho = mom[0][lane], inv = 1.0f / (1.0f + drho);
+    const float u[3] = {mom[1][lane] * inv, mom[2][lane] * inv, mom[3][lane] * inv};
     const float fe = feq_lane(wi, cxi, cyi, czi, drho, u);
     f = fe + (2.0f * L.tau[ph] / F.tau[ph]) * (f - fe);
-    if (store) Store<T>::st(fA<T, Q>(C, L) + (size_t)i * L.ncell + c, f, C.fp16_scale);
+    if (act) Store<T>::st(fA<T, Q>(C, L) + (size_t)i * L.ncell + c, f, C.fp16_scale);
+    __syncthreads();  // the moments are read before the next cells overwrite them
   }
 }
 
@@ -1471,30 +1461,10 @@ cudaError_t run_collect(Launch L, Ctx C, BlockShape S, const int *list, int n, i
   launcher(k_collect, L, 0)(C, S, list, n, bits, out, count, cap);
   return cudaGetLastError();
 }
-// One warp per GPW cells for the lattices with a group kernel (D2Q9, D3Q19); D3Q27 keeps
-// one thread per cell on the grid it was given.
-Launch group_launch(Launch L, int Q, int n) {
-  const int gpw = Q <= 16 ? 2 : 1;
-  const long long threads = (long long)((n + gpw - 1) / gpw) * 32;
-  L.block = 128;
-  L.grid = (int)std::max(1LL, (threads + 127) / 128);
-  return L;
-}
-#define LSB_GROUP_Q(Q, st, KERN, ...)                                                              \
-  do {                                                                                             \
-    L = group_launch(L, Q, n);                                                                     \
-    if (Q == 9) {                                                                                  \
-      if (st == 0) launcher(KERN<9, float>, L, 0)(__VA_ARGS__);                \
-      else launcher(KERN<9, __half>, L, 0)(__VA_ARGS__);                       \
-    } else {                                                                                       \
-      if (st == 0) launcher(KERN<19, float>, L, 0)(__VA_ARGS__);               \
-      else launcher(KERN<19, __half>, L, 0)(__VA_ARGS__);                      \
-    }                                                                                              \
-    return cudaGetLastError();                                                                     \
-  } while (0)
 cudaError_t run_restrict_cells(int Q, int st, Launch L, Ctx C, const int2 *cells, int n) {
-  if (Q == 27) LSB_QT(Q, st, (LK(k_restrict_cells)(C, cells, n)));
-  LSB_GROUP_Q(Q, st, k_restrict_cells_w, C, cells, n);
+  L.grid = std::max(1, (n + 31) / 32);
+  L.block = 32 * Q;
+  LSB_QT(Q, st, (LK(k_restrict_cells)(C, cells, n)));
 }
 cudaError_t run_ghost_cells(int Q, int st, Launch L, Ctx C, const int2 *cells, int n, float theta) {
   LSB_QT(Q, st, (LK(k_ghost_cells)(C, cells, n, theta)));
