@@ -138,8 +138,8 @@ __global__ void k_adj_seed(Ctx C, BlockShape S, const int *list, int nlist, cons
 }
 
 // ------------------------------------------------------------------ cut links
-// One thread per interface cell x (phase A); for each cut link (x, k), i = opp(k)
-// points to y = x + c_i (phase B).  The forward value was
+// One thread per cut link (x, k) of an interface cell x (phase A); i = opp(k) points to y =
+// x + c_i (phase B).  The forward value was
 //   q >= 1/2:          fi / 2q + (2q - 1)/2q fk + df / 2q
 //   q < 1/2, back ok:  2q fi + (1 - 2q) fb + df
 //   otherwise:         fi + df
@@ -155,9 +155,46 @@ __global__ void k_adj_seed(Ctx C, BlockShape S, const int *list, int nlist, cons
 // rates and times of every level (d omega_l / d nu = -3 omega_l^2 / r_l with
 // r_l = 2^(L-1-l)), [7 .. 12] the finest level's lattice acceleration per phase
 // (level l uses r_l times it).
+//
+// Frozen level set (LINK): one thread per cut link, with drho, u and S of both cells from
+// k_adj_moments (both are interface cells).  One thread per interface cell that walks its links
+// and forms the partner's moments from Q populations per link took 115 us on 147 k links of 33 k
+// cells (3D bubble, 128 x 128 x 256): a serial chain of loads per link at 159 registers.  The
+// two launches take 29 us.  Moving level set: one thread per interface cell, whose sums have the order of
+// its links.  Per link their order varies from run to run, and reinitialisation's transpose
+// turns that round-off into 2e-5 of dJ/dphi (41 x 92, 8 steps) where it was 1e-8.
+
+// Moments and strain rate of every interface cell's populations in F, into the macro planes
+// (drho, u[D], S): scratch during a reverse sweep, every forward step writes them before it
+// reads them.
 template <int Q>
-__global__ void k_adj_links(Ctx C, int glevel, const float *__restrict__ F, float *lamN, float *LA, float *MA,
-                            double *grad, int ncase, GeoAdj G) {
+__global__ void k_adj_moments(Ctx C, int glevel, const float *__restrict__ F) {
+  using LT = Lat<Q>;
+  constexpr int D = LT::D, NS = D * (D + 1) / 2;
+  const int n = min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
+  const int2 *lst = C.iface_list + (long long)glevel * C.list_cap;
+  const long long NF = C.nfine;
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
+    const int2 it = lst[e];
+    const LevelDev &L = C.lds[it.x];
+    const long long c = it.y, N = L.ncell, fc = L.fine_off + c;
+    const float *Fl = F + L.cell_off * Q;
+    const int A = C.tag[L.cell_off + c] & TAG_GAS;
+    float f[Q], r, u[3], S[6];
+#pragma unroll
+    for (int j = 0; j < Q; ++j) f[j] = Fl[j * N + c];
+    moments_strain<Q>(f, L.omega[A], r, u, S);
+    C.macro[fc] = r;
+#pragma unroll
+    for (int a = 0; a < D; ++a) C.macro[(1 + a) * NF + fc] = u[a];
+#pragma unroll
+    for (int k = 0; k < NS; ++k) C.macro[(1 + D + k) * NF + fc] = S[k];
+  }
+}
+
+template <int Q, bool LINK>
+__global__ void __launch_bounds__(128) k_adj_links(Ctx C, int glevel, const float *__restrict__ F, float *lamN, float *LA,
+                                                   float *MA, double *grad, int ncase, GeoAdj G) {
   using LT = Lat<Q>;
   constexpr int D = LT::D;
   constexpr int NS = D * (D + 1) / 2;
@@ -165,213 +202,253 @@ __global__ void k_adj_links(Ctx C, int glevel, const float *__restrict__ F, floa
   const bool shared_sum = ncase <= kShCases;
   for (int k = threadIdx.x; k < kShCases * 5; k += blockDim.x) sg[k] = 0.0;
   __syncthreads();
-  const int n = min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
-  const int2 *lst = C.iface_list + (long long)glevel * C.list_cap;
+  const long long n = LINK ? min((long long)C.counters[glevel * NCOUNT + 0], C.link_cap)
+                           : (long long)min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
+  const int2 *lst = LINK ? C.link_cell + C.link_list_off[glevel] : C.iface_list + (long long)glevel * C.list_cap;
   const long long NF = C.nfine;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) {
-    const int2 it = lst[e];
-    const LevelDev &L = C.lds[it.x];
-    const long long c = it.y;
-    int x, y, z;
-    cell_xyz(L, c, x, y, z);
-    const long long fo = L.fine_off;
-    const uint32_t cm = C.cmask[fo + c];
-    const int cb = C.cbase[fo + c];
-    const uint8_t tg = C.tag[L.cell_off + c];
-    const int A = tg & TAG_GAS;
-    const int Bp = 1 - A;
-    const long long N = L.ncell;
-    const float *Fl = F + L.cell_off * Q;
-    float *lam = lamN + L.cell_off * Q;
-    float f[Q];
-#pragma unroll
-    for (int j = 0; j < Q; ++j) f[j] = Fl[j * N + c];
-    float rA, uA[3], SA[6];
-    moments_strain<Q>(f, L.omega[A], rA, uA, SA);
-    const float phx = C.phi[fo + c];
-    float nx[3] = {0.f, 0.f, 0.f};
-    for (int a = 0; a < D; ++a) nx[a] = C.nvec[a * NF + fo + c];
-    const float kx = C.kappa[fo + c];
-    const float etaA = L.eta[A], etaB = L.eta[Bp];
-    const float eb = 0.5f * (etaA + etaB);
-    const float je = etaB - etaA;
-    const float r = je / eb;
-    const float sgn = (A == 0) ? 1.0f : -1.0f;
-    // macro adjoint of x, summed over its links: rho, u[D], S[NS]
-    float mx[1 + 3 + 6];
-    for (int m = 0; m < 1 + D + NS; ++m) mx[m] = 0.f;
+  const float *M = C.macro;
+  // (every lane of a warp makes the same rounds: the parameter partials are summed over it)
+  for (long long e0 = blockIdx.x * (long long)blockDim.x; e0 < n; e0 += (long long)gridDim.x * blockDim.x) {
+    const long long e = e0 + threadIdx.x;
     double gs = 0.0, grp[2] = {0.0, 0.0}, get[2] = {0.0, 0.0};
-    for (int k = 0; k < Q; ++k) {
-      if (!(cm & (1u << k))) continue;
-      const int i = LT::opp(k);
-      const long long li = cb + __popc(cm & ((1u << k) - 1u));
-      if (li >= C.link_cap) continue;
-      const float lml = lam[k * N + c];
-      int yx = x + LT::cx(i), yy = y + LT::cy(i), yz = z + LT::cz(i);
-      wrap(L, 0, yx); wrap(L, 1, yy); if (D == 3) wrap(L, 2, yz);
-      const long long cy_ = cidx(L, yx, yy, yz);
-      const float phy = C.phi[fo + cy_];
-      const float q = phx / (phx - phy);
-      // Bouzidi branch coefficients
-      bool hi = q >= 0.5f, ok = false;
-      if (!hi) {
-        int bx = x - LT::cx(i), by = y - LT::cy(i), bz = z - LT::cz(i);
-        ok = wrap(L, 0, bx) && wrap(L, 1, by) && (D == 2 || wrap(L, 2, bz));
-        if (ok) {
-          const uint8_t tb = C.tag[L.cell_off + cidx(L, bx, by, bz)];
-          ok = (tb & TAG_LEAF) && ((tb & TAG_GAS) == A);
-        }
-      }
-      const float c_fi = hi ? 0.5f / q : (ok ? 2.0f * q : 1.0f);
-      const float c_fk = hi ? (2.0f * q - 1.0f) / (2.0f * q) : 0.0f;
-      const float c_df = hi ? 0.5f / q : 1.0f;
-      LA[2 * li] = c_fi * lml;
-      LA[2 * li + 1] = c_fk * lml;
-      if (!hi && ok) lam[i * N + c] += (1.0f - 2.0f * q) * lml;
-      const float ldf = c_df * lml;
-      if (ldf == 0.0f) continue;
-      // forward pieces of Eq. bb_cc at this link
-      float fy[Q];
+    int cid = -1;
+    if (e < n) {
+      const int2 it = lst[e];
+      const LevelDev &L = C.lds[it.x];
+      const long long c = it.y;
+      cid = L.case_id;
+      int x, y, z;
+      cell_xyz(L, c, x, y, z);
+      const long long fo = L.fine_off;
+      const int k0 = LINK ? C.link_dir[C.link_list_off[glevel] + e] : 0, k1 = LINK ? k0 + 1 : Q;
+      const uint32_t cm = LINK ? 1u << k0 : C.cmask[fo + c];
+      const long long cb = LINK ? e : C.cbase[fo + c];
+      const uint8_t tg = C.tag[L.cell_off + c];
+      const int A = tg & TAG_GAS;
+      const int Bp = 1 - A;
+      const long long N = L.ncell;
+      const float *Fl = F + L.cell_off * Q;
+      float *lam = lamN + L.cell_off * Q;
+      float f[Q];
+      float rA, uA[3] = {0.f, 0.f, 0.f}, SA[6];
+      if (LINK) {
+        rA = M[fo + c];
 #pragma unroll
-      for (int j = 0; j < Q; ++j) fy[j] = Fl[j * N + cy_];
-      float rB, uB[3], SB[6];
-      moments_strain<Q>(fy, L.omega[Bp], rB, uB, SB);
-      float nv[3] = {0.f, 0.f, 0.f}, nn = 0.f;
-      for (int a = 0; a < D; ++a) {
-        nv[a] = (1.0f - q) * nx[a] + q * C.nvec[a * NF + fo + cy_];
-        nn += nv[a] * nv[a];
-      }
-      nn = sqrtf(nn);
-      for (int a = 0; a < D; ++a) nv[a] = nn > 0.f ? sgn * nv[a] / nn : 0.f;
-      const float kap = sgn * ((1.0f - q) * kx + q * C.kappa[fo + cy_]);
-      float Sb[6];
-      for (int s = 0; s < NS; ++s) Sb[s] = 0.5f * (SA[s] + SB[s]);
-      const float jp = CS2 * (L.rho_phys[Bp] * rB - L.rho_phys[A] * rA);
-      const float ci[3] = {(float)LT::cx(i), (float)LT::cy(i), (float)LT::cz(i)};
-      float v[3] = {0.f, 0.f, 0.f}, Snn = 0.f, cn = 0.f, cv = 0.f;
-      for (int a = 0; a < D; ++a) {
-        for (int b = 0; b < D; ++b) v[a] += Sb[sym<D>(a, b)] * nv[b];
-        Snn += nv[a] * v[a];
-        cn += ci[a] * nv[a];
-        cv += ci[a] * v[a];
-      }
-      const float cvt = cv - Snn * cn;
-      // transpose of df = -6 w_i (c_i . u_I - q (1 - q) ccS), ccS = alpha cn^2 - 2 r cn cvt,
-      // alpha = (jp + sigma kappa) / (2 eb) - r Snn, r = je / eb
-      const float w6 = 6.0f * LT::w(i);
-      const float luI = -w6 * ldf;  // times c_i
-      const float lccS = w6 * q * (1.0f - q) * ldf;
-      const float la = lccS * cn * cn;
-      const float lcvt = -2.0f * r * cn * lccS;
-      const float lr = -2.0f * cn * cvt * lccS - Snn * la;
-      const float ljp = la / (2.0f * eb);
-      const float leb = -la * (jp + L.sigma * kap) / (2.0f * eb * eb) - lr * je / (eb * eb);
-      const float lje = lr / eb;
-      gs += (double)(la * kap / (2.0f * eb));
-      grp[Bp] += (double)(ljp * CS2 * rB);
-      grp[A] -= (double)(ljp * CS2 * rA);
-      get[A] += (double)(0.5f * leb - lje);
-      get[Bp] += (double)(0.5f * leb + lje);
-      const float lSnn = -r * la - cn * lcvt;
-      if (G.phi) {
-        // adjoint of the frozen geometry: q (explicit in Eq. bb, in u_I, in q (1 - q)
-        // and in the interpolated n, kappa), the link's n_A and kappa_A
-        const float om = L.omega[A];
-        const float acA = LT::cx(i) * L.acc[A][0] + LT::cy(i) * L.acc[A][1] + LT::cz(i) * L.acc[A][2];
-        const float usA = uA[0] * uA[0] + uA[1] * uA[1] + uA[2] * uA[2];
-        // post-collision f_i, f_k of x (Eq. 1) and the forward df
-        float f_i = 0.f, f_k = 0.f;  // select without dynamic register indexing
+        for (int a = 0; a < D; ++a) uA[a] = M[(1 + a) * NF + fo + c];
 #pragma unroll
-        for (int j = 0; j < Q; ++j) {
-          f_i = j == i ? f[j] : f_i;
-          f_k = j == k ? f[j] : f_k;
-        }
-        const float fi = f_i + om * (feq_dev<Q>(i, rA, uA, usA) - f_i) + 3.0f * LT::w(i) * (1.0f + rA) * acA;
-        const float fk = f_k + om * (feq_dev<Q>(k, rA, uA, usA) - f_k) - 3.0f * LT::w(k) * (1.0f + rA) * acA;
-        const float ccS = cn * cn * ((jp + L.sigma * kap) / (2.0f * eb) - r * Snn) - 2.0f * r * cn * cvt;
-        float cuI = 0.f, cdu = 0.f;
-        for (int a = 0; a < D; ++a) {
-          cuI += ci[a] * ((1.0f - q) * uA[a] + q * uB[a]);
-          cdu += ci[a] * (uB[a] - uA[a]);
-        }
-        const float df = -w6 * (cuI - q * (1.0f - q) * ccS);
-        float lq = 0.f;
-        if (hi) {
-          lq = lml * (-fi + fk - df) / (2.0f * q * q);
-        } else if (ok) {
+        for (int s = 0; s < NS; ++s) SA[s] = M[(1 + D + s) * NF + fo + c];
+      } else {
+#pragma unroll
+        for (int j = 0; j < Q; ++j) f[j] = Fl[j * N + c];
+        moments_strain<Q>(f, L.omega[A], rA, uA, SA);
+      }
+      const float phx = C.phi[fo + c];
+      float nx[3] = {0.f, 0.f, 0.f};
+      for (int a = 0; a < D; ++a) nx[a] = C.nvec[a * NF + fo + c];
+      const float kx = C.kappa[fo + c];
+      const float etaA = L.eta[A], etaB = L.eta[Bp];
+      const float eb = 0.5f * (etaA + etaB);
+      const float je = etaB - etaA;
+      const float r = je / eb;
+      const float sgn = (A == 0) ? 1.0f : -1.0f;
+      // macro adjoint of x, summed over its links: rho, u[D], S[NS]
+      float mx[1 + 3 + 6];
+      for (int m = 0; m < 1 + D + NS; ++m) mx[m] = 0.f;
+      for (int k = k0; k < k1; ++k) {
+        if (!(cm & (1u << k))) continue;
+        const int i = LT::opp(k);
+        const long long li = cb + __popc(cm & ((1u << k) - 1u));
+        if (li >= C.link_cap) continue;
+        const float lml = lam[k * N + c];
+        int yx = x + LT::cx(i), yy = y + LT::cy(i), yz = z + LT::cz(i);
+        wrap(L, 0, yx); wrap(L, 1, yy); if (D == 3) wrap(L, 2, yz);
+        const long long cy_ = cidx(L, yx, yy, yz), my = fo + cy_;
+        const float phy = C.phi[fo + cy_];
+        const float q = phx / (phx - phy);
+        // Bouzidi branch coefficients
+        bool hi = q >= 0.5f, ok = false;
+        if (!hi) {
           int bx = x - LT::cx(i), by = y - LT::cy(i), bz = z - LT::cz(i);
-          wrap(L, 0, bx); wrap(L, 1, by); if (D == 3) wrap(L, 2, bz);
-          const long long cbk = cidx(L, bx, by, bz);
-          float fbv[Q];
+          ok = wrap(L, 0, bx) && wrap(L, 1, by) && (D == 2 || wrap(L, 2, bz));
+          if (ok) {
+            const uint8_t tb = C.tag[L.cell_off + cidx(L, bx, by, bz)];
+            ok = (tb & TAG_LEAF) && ((tb & TAG_GAS) == A);
+          }
+        }
+        const float c_fi = hi ? 0.5f / q : (ok ? 2.0f * q : 1.0f);
+        const float c_fk = hi ? (2.0f * q - 1.0f) / (2.0f * q) : 0.0f;
+        const float c_df = hi ? 0.5f / q : 1.0f;
+        LA[2 * li] = c_fi * lml;
+        LA[2 * li + 1] = c_fk * lml;
+        if (!hi && ok) lam[i * N + c] += (1.0f - 2.0f * q) * lml;
+        const float ldf = c_df * lml;
+        if (ldf == 0.0f) continue;
+        // forward pieces of Eq. bb_cc at this link
+        float rB, uB[3] = {0.f, 0.f, 0.f}, SB[6];
+        if (LINK) {
+          rB = M[my];
 #pragma unroll
-          for (int j = 0; j < Q; ++j) fbv[j] = Fl[j * N + cbk];
-          float rb, ub[3];
-          lb_moments<Q>(fbv, rb, ub);
-          const float usb = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
-          const float fb_i = Fl[(long long)i * N + cbk];
-          const float fb = fb_i + om * (feq_dev<Q>(i, rb, ub, usb) - fb_i) + 3.0f * LT::w(i) * (1.0f + rb) * acA;
-          lq = lml * (2.0f * fi - 2.0f * fb);
+          for (int a = 0; a < D; ++a) uB[a] = M[(1 + a) * NF + my];
+#pragma unroll
+          for (int s = 0; s < NS; ++s) SB[s] = M[(1 + D + s) * NF + my];
+        } else {
+          float fy[Q];
+#pragma unroll
+          for (int j = 0; j < Q; ++j) fy[j] = Fl[j * N + cy_];
+          moments_strain<Q>(fy, L.omega[Bp], rB, uB, SB);
         }
-        lq += ldf * (-w6) * cdu + ldf * w6 * (1.0f - 2.0f * q) * ccS;
-        // d ccS / d n_A = cn^2 (-2 r v) + (2 alpha cn - 2 r cvt) c - 2 r cn (Sbar c - 2 cn v - Snn c)
-        const float alpha = (jp + L.sigma * kap) / (2.0f * eb) - r * Snn;
-        float lnA[3] = {0.f, 0.f, 0.f};
+        float nv[3] = {0.f, 0.f, 0.f}, nn = 0.f;
         for (int a = 0; a < D; ++a) {
-          float Sc = 0.f;
-          for (int b = 0; b < D; ++b) Sc += Sb[sym<D>(a, b)] * ci[b];
-          lnA[a] = lccS * (-2.0f * r * cn * cn * v[a] + (2.0f * alpha * cn - 2.0f * r * cvt) * ci[a] -
-                           2.0f * r * cn * (Sc - 2.0f * cn * v[a] - Snn * ci[a]));
+          nv[a] = (1.0f - q) * nx[a] + q * C.nvec[a * NF + fo + cy_];
+          nn += nv[a] * nv[a];
         }
-        const float lkA = lccS * cn * cn * L.sigma / (2.0f * eb);
-        // n_A = sgn m / |m|, m = (1 - q) n_x + q n_y; kappa_A = sgn ((1 - q) kappa_x + q kappa_y)
-        const long long my = fo + cy_;
-        if (nn > 0.f) {
-          float nh[3], dot = 0.f;
-          for (int a = 0; a < D; ++a) {
-            nh[a] = sgn * nv[a];  // m / |m|
-            dot += nh[a] * sgn * lnA[a];
+        nn = sqrtf(nn);
+        for (int a = 0; a < D; ++a) nv[a] = nn > 0.f ? sgn * nv[a] / nn : 0.f;
+        const float kap = sgn * ((1.0f - q) * kx + q * C.kappa[fo + cy_]);
+        float Sb[6];
+        for (int s = 0; s < NS; ++s) Sb[s] = 0.5f * (SA[s] + SB[s]);
+        const float jp = CS2 * (L.rho_phys[Bp] * rB - L.rho_phys[A] * rA);
+        const float ci[3] = {(float)LT::cx(i), (float)LT::cy(i), (float)LT::cz(i)};
+        float v[3] = {0.f, 0.f, 0.f}, Snn = 0.f, cn = 0.f, cv = 0.f;
+        for (int a = 0; a < D; ++a) {
+          for (int b = 0; b < D; ++b) v[a] += Sb[sym<D>(a, b)] * nv[b];
+          Snn += nv[a] * v[a];
+          cn += ci[a] * nv[a];
+          cv += ci[a] * v[a];
+        }
+        const float cvt = cv - Snn * cn;
+        // transpose of df = -6 w_i (c_i . u_I - q (1 - q) ccS), ccS = alpha cn^2 - 2 r cn cvt,
+        // alpha = (jp + sigma kappa) / (2 eb) - r Snn, r = je / eb
+        const float w6 = 6.0f * LT::w(i);
+        const float luI = -w6 * ldf;  // times c_i
+        const float lccS = w6 * q * (1.0f - q) * ldf;
+        const float la = lccS * cn * cn;
+        const float lcvt = -2.0f * r * cn * lccS;
+        const float lr = -2.0f * cn * cvt * lccS - Snn * la;
+        const float ljp = la / (2.0f * eb);
+        const float leb = -la * (jp + L.sigma * kap) / (2.0f * eb * eb) - lr * je / (eb * eb);
+        const float lje = lr / eb;
+        gs += (double)(la * kap / (2.0f * eb));
+        const double gA = -(double)(ljp * CS2 * rA), gB = (double)(ljp * CS2 * rB);
+        const double eA = (double)(0.5f * leb - lje), eB = (double)(0.5f * leb + lje);
+        grp[0] += A ? gB : gA;
+        grp[1] += A ? gA : gB;
+        get[0] += A ? eB : eA;
+        get[1] += A ? eA : eB;
+        const float lSnn = -r * la - cn * lcvt;
+        if (G.phi) {
+          // adjoint of the frozen geometry: q (explicit in Eq. bb, in u_I, in q (1 - q)
+          // and in the interpolated n, kappa), the link's n_A and kappa_A
+          const float om = L.omega[A];
+          const float acA = LT::cx(i) * L.acc[A][0] + LT::cy(i) * L.acc[A][1] + LT::cz(i) * L.acc[A][2];
+          const float usA = uA[0] * uA[0] + uA[1] * uA[1] + uA[2] * uA[2];
+          // post-collision f_i, f_k of x (Eq. 1) and the forward df
+          float f_i = 0.f, f_k = 0.f;
+          if (LINK) {
+            f_i = Fl[i * N + c];
+            f_k = Fl[k * N + c];
+          } else {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {  // select without dynamic register indexing
+              f_i = j == i ? f[j] : f_i;
+              f_k = j == k ? f[j] : f_k;
+            }
           }
+          const float fi = f_i + om * (feq_dev<Q>(i, rA, uA, usA) - f_i) + 3.0f * LT::w(i) * (1.0f + rA) * acA;
+          const float fk = f_k + om * (feq_dev<Q>(k, rA, uA, usA) - f_k) - 3.0f * LT::w(k) * (1.0f + rA) * acA;
+          const float ccS = cn * cn * ((jp + L.sigma * kap) / (2.0f * eb) - r * Snn) - 2.0f * r * cn * cvt;
+          float cuI = 0.f, cdu = 0.f;
           for (int a = 0; a < D; ++a) {
-            const float lm = (sgn * lnA[a] - nh[a] * dot) / nn;
-            lq += lm * (C.nvec[a * NF + my] - nx[a]);
-            atomicAdd(G.n + a * NF + fo + c, (1.0f - q) * lm);
-            atomicAdd(G.n + a * NF + my, q * lm);
+            cuI += ci[a] * ((1.0f - q) * uA[a] + q * uB[a]);
+            cdu += ci[a] * (uB[a] - uA[a]);
           }
+          const float df = -w6 * (cuI - q * (1.0f - q) * ccS);
+          float lq = 0.f;
+          if (hi) {
+            lq = lml * (-fi + fk - df) / (2.0f * q * q);
+          } else if (ok) {
+            int bx = x - LT::cx(i), by = y - LT::cy(i), bz = z - LT::cz(i);
+            wrap(L, 0, bx); wrap(L, 1, by); if (D == 3) wrap(L, 2, bz);
+            const long long cbk = cidx(L, bx, by, bz);
+            float fbv[Q];
+#pragma unroll
+            for (int j = 0; j < Q; ++j) fbv[j] = Fl[j * N + cbk];
+            float rb, ub[3];
+            lb_moments<Q>(fbv, rb, ub);
+            const float usb = ub[0] * ub[0] + ub[1] * ub[1] + ub[2] * ub[2];
+            const float fb_i = Fl[(long long)i * N + cbk];
+            const float fb = fb_i + om * (feq_dev<Q>(i, rb, ub, usb) - fb_i) + 3.0f * LT::w(i) * (1.0f + rb) * acA;
+            lq = lml * (2.0f * fi - 2.0f * fb);
+          }
+          lq += ldf * (-w6) * cdu + ldf * w6 * (1.0f - 2.0f * q) * ccS;
+          // d ccS / d n_A = cn^2 (-2 r v) + (2 alpha cn - 2 r cvt) c - 2 r cn (Sbar c - 2 cn v - Snn c)
+          const float alpha = (jp + L.sigma * kap) / (2.0f * eb) - r * Snn;
+          float lnA[3] = {0.f, 0.f, 0.f};
+          for (int a = 0; a < D; ++a) {
+            float Sc = 0.f;
+            for (int b = 0; b < D; ++b) Sc += Sb[sym<D>(a, b)] * ci[b];
+            lnA[a] = lccS * (-2.0f * r * cn * cn * v[a] + (2.0f * alpha * cn - 2.0f * r * cvt) * ci[a] -
+                             2.0f * r * cn * (Sc - 2.0f * cn * v[a] - Snn * ci[a]));
+          }
+          const float lkA = lccS * cn * cn * L.sigma / (2.0f * eb);
+          // n_A = sgn m / |m|, m = (1 - q) n_x + q n_y; kappa_A = sgn ((1 - q) kappa_x + q kappa_y)
+          if (nn > 0.f) {
+            float nh[3], dot = 0.f;
+            for (int a = 0; a < D; ++a) {
+              nh[a] = sgn * nv[a];  // m / |m|
+              dot += nh[a] * sgn * lnA[a];
+            }
+            for (int a = 0; a < D; ++a) {
+              const float lm = (sgn * lnA[a] - nh[a] * dot) / nn;
+              lq += lm * (C.nvec[a * NF + my] - nx[a]);
+              atomicAdd(G.n + a * NF + fo + c, (1.0f - q) * lm);
+              atomicAdd(G.n + a * NF + my, q * lm);
+            }
+          }
+          const float ky = C.kappa[my];
+          lq += sgn * (ky - kx) * lkA;
+          atomicAdd(G.kappa + fo + c, sgn * (1.0f - q) * lkA);
+          atomicAdd(G.kappa + my, sgn * q * lkA);
+          // q = phi_x / (phi_x - phi_y)
+          const float den = (phx - phy) * (phx - phy);
+          atomicAdd(G.phi + fo + c, -lq * phy / den);
+          atomicAdd(G.phi + my, lq * phx / den);
         }
-        const float ky = C.kappa[my];
-        lq += sgn * (ky - kx) * lkA;
-        atomicAdd(G.kappa + fo + c, sgn * (1.0f - q) * lkA);
-        atomicAdd(G.kappa + my, sgn * q * lkA);
-        // q = phi_x / (phi_x - phi_y)
-        const float den = (phx - phy) * (phx - phy);
-        atomicAdd(G.phi + fo + c, -lq * phy / den);
-        atomicAdd(G.phi + my, lq * phx / den);
-      }
-      // macro adjoint: rho through [p], u through u_I, S through Sbar (half to each cell)
-      const long long my = fo + cy_;
-      mx[0] -= CS2 * L.rho_phys[A] * ljp;
-      atomicAdd(MA + my, CS2 * L.rho_phys[Bp] * ljp);
-      for (int a = 0; a < D; ++a) {
-        mx[1 + a] += (1.0f - q) * luI * ci[a];
-        atomicAdd(MA + (1 + a) * NF + my, q * luI * ci[a]);
-      }
-      for (int a = 0; a < D; ++a)
-        for (int b = a; b < D; ++b) {
-          // sum of the (a, b) and (b, a) entries of ci n^T lcvt + n n^T lSnn
-          const float t = a == b ? ci[a] * nv[a] * lcvt + nv[a] * nv[a] * lSnn
-                                 : (ci[a] * nv[b] + ci[b] * nv[a]) * lcvt + 2.0f * nv[a] * nv[b] * lSnn;
-          const int s = sym<D>(a, b);
-          mx[1 + D + s] += 0.5f * t;
-          atomicAdd(MA + (1 + D + s) * NF + my, 0.5f * t);
+        // macro adjoint: rho through [p], u through u_I, S through Sbar (half to each cell)
+        mx[0] -= CS2 * L.rho_phys[A] * ljp;
+        atomicAdd(MA + my, CS2 * L.rho_phys[Bp] * ljp);
+        for (int a = 0; a < D; ++a) {
+          mx[1 + a] += (1.0f - q) * luI * ci[a];
+          atomicAdd(MA + (1 + a) * NF + my, q * luI * ci[a]);
         }
+        for (int a = 0; a < D; ++a)
+          for (int b = a; b < D; ++b) {
+            // sum of the (a, b) and (b, a) entries of ci n^T lcvt + n n^T lSnn
+            const float t = a == b ? ci[a] * nv[a] * lcvt + nv[a] * nv[a] * lSnn
+                                   : (ci[a] * nv[b] + ci[b] * nv[a]) * lcvt + 2.0f * nv[a] * nv[b] * lSnn;
+            const int s = sym<D>(a, b);
+            mx[1 + D + s] += 0.5f * t;
+            atomicAdd(MA + (1 + D + s) * NF + my, 0.5f * t);
+          }
+      }
+      for (int m = 0; m < 1 + D + NS; ++m)
+        if (mx[m] != 0.f) atomicAdd(MA + m * NF + fo + c, mx[m]);
     }
-    for (int m = 0; m < 1 + D + NS; ++m)
-      if (mx[m] != 0.f) atomicAdd(MA + m * NF + fo + c, mx[m]);
+    // parameter partials in float64: with a thread per link, over the warp when its links are of
+    // one case
     const double vals[5] = {gs, grp[0], grp[1], get[0], get[1]};
+    const int c0 = __shfl_sync(0xffffffffu, cid, 0);
+    const bool one = LINK && __all_sync(0xffffffffu, cid == c0 || cid < 0);
+#pragma unroll
     for (int k = 0; k < 5; ++k) {
-      if (vals[k] == 0.0) continue;
-      if (shared_sum) atomicAdd(sg + L.case_id * 5 + k, vals[k]);
-      else atomicAdd(grad + (long long)L.case_id * NG_ADJ + k, vals[k]);
+      double v = vals[k];
+      if (one) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      }
+      if (v == 0.0 || cid < 0 || (one && (threadIdx.x & 31))) continue;
+      if (shared_sum) atomicAdd(sg + cid * 5 + k, v);
+      else atomicAdd(grad + (long long)cid * NG_ADJ + k, v);
     }
   }
   __syncthreads();
@@ -630,7 +707,12 @@ __global__ void __launch_bounds__(512, LSB_ADJ_MINB) k_adj_collide(Ctx C, BlockS
 // with k = -omega / (2 rho c_s^2), Pi_ab = sum c_a c_b (f - feq), and
 // dPi_ab/df_j = c_ja c_jb - c_s^2 d_ab + u_a u_b - c_ja u_b - u_a c_jb; the strain
 // rate's omega dependence (S / omega) goes to the omega partial.
-template <int Q>
+//
+// Latency-bound: lamO's values are loaded before the sums they join (loads and stores of one
+// array would wait for one another).  Frozen level set (MOM): drho, u and S come from
+// k_adj_moments' planes, Pi_ab = S_ab / k, and F is not read: 37 -> 31 us on the 33 k cells of
+// the 3D bubble.  Moving: from F as the oracle has it (round-off is amplified, see k_adj_links).
+template <int Q, bool MOM>
 __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, float *lamO, float *MA, double *grad,
                             int ncase) {
   using LT = Lat<Q>;
@@ -658,8 +740,20 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
     if (!any) continue;
     const float *Fl = F + L.cell_off * Q;
     float *lO = lamO + L.cell_off * Q;
+    float lv[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) lv[i] = lO[i * N + c];
     float d = 0.f, j[3] = {0.f, 0.f, 0.f}, m2[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    for (int i = 0; i < Q; ++i) {
+    float uM[3] = {0.f, 0.f, 0.f};
+    if (MOM) {
+      d = C.macro[fc];
+#pragma unroll
+      for (int a = 0; a < D; ++a) uM[a] = C.macro[(1 + a) * NF + fc];
+#pragma unroll
+      for (int k = 0; k < NS; ++k) m2[k] = C.macro[(1 + D + k) * NF + fc];
+    }
+#pragma unroll
+    for (int i = 0; i < (MOM ? 0 : Q); ++i) {
       const float fi = Fl[i * N + c];
       const float c3[3] = {(float)LT::cx(i), (float)LT::cy(i), (float)LT::cz(i)};
       d += fi;
@@ -669,24 +763,27 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
       }
     }
     const float rho = 1.0f + d, irho = 1.0f / rho;
-    const float u[3] = {j[0] * irho, j[1] * irho, j[2] * irho};
+    const float u[3] = {MOM ? uM[0] : j[0] * irho, MOM ? uM[1] : j[1] * irho, MOM ? uM[2] : j[2] * irho};
     const int ph = C.tag[L.cell_off + c] & TAG_GAS;
     const float om = L.omega[ph];
     const float kk = -1.5f * om * irho;
     const float *mu = m + 1, *mS = m + 1 + D;
     // j-independent parts; Pi_ab = m2_ab - drho c_s^2 d_ab - rho u_a u_b (isotropy of the weights)
     float sP = 0.f, sD = 0.f, sUU = 0.f, muu = 0.f;
+#pragma unroll
     for (int a = 0; a < D; ++a) {
       muu += mu[a] * u[a];
+#pragma unroll
       for (int b = a; b < D; ++b) {
         const float ms = mS[sym<D>(a, b)];
-        const float Pab = m2[sym<D>(a, b)] - (a == b ? CS2 * d : 0.f) - rho * u[a] * u[b];
+        const float Pab = MOM ? m2[sym<D>(a, b)] / kk : m2[sym<D>(a, b)] - (a == b ? CS2 * d : 0.f) - rho * u[a] * u[b];
         sP += ms * Pab;
         sUU += ms * u[a] * u[b];
         if (a == b) sD += ms;
       }
     }
     const float base = m[0] - muu * irho + kk * (-CS2 * sD + sUU - sP * irho);
+#pragma unroll
     for (int jj = 0; jj < Q; ++jj) {
       const float cj[3] = {(float)LT::cx(jj), (float)LT::cy(jj), (float)LT::cz(jj)};
       float v = base;
@@ -695,7 +792,7 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
         for (int b = a; b < D; ++b)  // for a < b the stored lS holds both orderings
           v += kk * mS[sym<D>(a, b)] * (cj[a] * cj[b] - cj[a] * u[b] - u[a] * cj[b]);
       }
-      lO[jj * N + c] += v;
+      lO[jj * N + c] = lv[jj] + v;
     }
     const double lom = (double)(sP * kk / om) * (double)(-3.0f * om * om / (float)L.scale);  // per nu
     if (lom != 0.0) {
@@ -717,7 +814,11 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
 // quadratic of k_geometry (Sec. 2.2): gradient g and Hessian H are linear in the
 // stencil sums P = sum v, sx_a = sum o_a v, sxx_a = sum o_a^2 v, sxy = sum o_a o_b v
 // over the 3^D points (walls clamp, periodic axes wrap), so each point's phi
-// receives l_P + o . l_sx + o^2 . l_sxx + (o_a o_b) . l_sxy.
+// receives l_P + o . l_sx + o^2 . l_sxx + (o_a o_b) . l_sxy.  Bound by the few FP64 units: the
+// sums and their transpose go by rows and planes (100 additions each in 3D instead of 400
+// multiply-adds with converted offsets), and what the cell's constants divide is multiplied by
+// their inverses: 203 -> 74 us on the interface of 96 x 96 x 128 on two levels, 61 -> 25
+// on the 33 k cells of the 3D bubble, 22 -> 12 on 64 x 96 on two levels.
 template <int D>
 __global__ void k_adj_geometry(Ctx C, int glevel, GeoAdj G) {
   const int n = min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
@@ -737,48 +838,71 @@ __global__ void k_adj_geometry(Ctx C, int glevel, GeoAdj G) {
     if (lk == 0.0 && ln[0] == 0.0 && ln[1] == 0.0 && ln[2] == 0.0) continue;
     int x, y, z;
     cell_xyz(L, c, x, y, z);
+    constexpr int NZ = D == 3 ? 3 : 1;
+    int xo[3], yo[3], zo[3] = {0, 0, 0};
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+      xo[o] = clampwrap(L, 0, x + o - 1);
+      yo[o] = clampwrap(L, 1, y + o - 1);
+      if (D == 3) zo[o] = clampwrap(L, 2, z + o - 1);
+    }
+    const float *ph = C.phi + L.fine_off;
+    float v[NZ][3][3];
+#pragma unroll
+    for (int k = 0; k < NZ; ++k)
+#pragma unroll
+      for (int j = 0; j < 3; ++j)
+#pragma unroll
+        for (int i = 0; i < 3; ++i) v[k][j][i] = ph[cidx(L, xo[i], yo[j], zo[k])];
+    // the sums by rows (r: sum, difference, squares), then planes (q), then over the planes
     double P = 0, sx[3] = {0, 0, 0}, sxx[3] = {0, 0, 0}, sxy[3] = {0, 0, 0};
-    for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz)
-      for (int oy = -1; oy <= 1; ++oy)
-        for (int ox = -1; ox <= 1; ++ox) {
-          const int xx = clampwrap(L, 0, x + ox), yy = clampwrap(L, 1, y + oy);
-          const int zz = D == 3 ? clampwrap(L, 2, z + oz) : 0;
-          const double v = (double)C.phi[L.fine_off + cidx(L, xx, yy, zz)];
-          const int o[3] = {ox, oy, oz};
-          P += v;
-          for (int a = 0; a < D; ++a) {
-            sx[a] += o[a] * v;
-            sxx[a] += o[a] * o[a] * v;
-          }
-          sxy[0] += ox * oy * v;
-          if (D == 3) {
-            sxy[1] += ox * oz * v;
-            sxy[2] += oy * oz * v;
-          }
-        }
+#pragma unroll
+    for (int k = 0; k < NZ; ++k) {
+      double r0[3], r1[3], r2[3];
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        const double vm = v[k][j][0], vp = v[k][j][2];
+        r1[j] = vp - vm;
+        r2[j] = vp + vm;
+        r0[j] = r2[j] + (double)v[k][j][1];
+      }
+      const double qyy = r0[2] + r0[0], q = qyy + r0[1], qy = r0[2] - r0[0], qx = r1[2] + r1[1] + r1[0];
+      P += q;
+      sx[0] += qx;
+      sx[1] += qy;
+      sxx[0] += r2[2] + r2[1] + r2[0];
+      sxx[1] += qyy;
+      sxy[0] += r1[2] - r1[0];
+      if (D == 3 && k != 1) {
+        sx[2] += k ? q : -q;
+        sxx[2] += q;
+        sxy[1] += k ? qx : -qx;
+        sxy[2] += k ? qy : -qy;
+      }
+    }
     // forward fit (as in k_geometry)
     double g[3] = {0, 0, 0}, H[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
     double a0, s;
     if (D == 2) {
       const double R = sxx[0] + sxx[1];
-      s = (3.0 * R - 4.0 * P) / 6.0;
-      a0 = (5.0 * P - 3.0 * R) / 9.0;
+      s = (3.0 * R - 4.0 * P) * (1.0 / 6.0);
+      a0 = (5.0 * P - 3.0 * R) * (1.0 / 9.0);
       for (int a = 0; a < 2; ++a) {
-        g[a] = sx[a] / 6.0;
+        g[a] = sx[a] * (1.0 / 6.0);
         H[a][a] = sxx[a] - 6.0 * a0 - 4.0 * s;
       }
-      H[0][1] = H[1][0] = sxy[0] / 4.0;
+      H[0][1] = H[1][0] = sxy[0] * 0.25;
     } else {
       const double R = sxx[0] + sxx[1] + sxx[2];
-      s = (R - 2.0 * P) / 6.0;
-      a0 = (7.0 * P - 3.0 * R) / 27.0;
+      s = (R - 2.0 * P) * (1.0 / 6.0);
+      a0 = (7.0 * P - 3.0 * R) * (1.0 / 27.0);
       for (int a = 0; a < 3; ++a) {
-        g[a] = sx[a] / 18.0;
-        H[a][a] = (sxx[a] - 18.0 * a0 - 12.0 * s) / 3.0;
+        g[a] = sx[a] * (1.0 / 18.0);
+        H[a][a] = (sxx[a] - 18.0 * a0 - 12.0 * s) * (1.0 / 3.0);
       }
-      H[0][1] = H[1][0] = sxy[0] / 12.0;
-      H[0][2] = H[2][0] = sxy[1] / 12.0;
-      H[1][2] = H[2][1] = sxy[2] / 12.0;
+      H[0][1] = H[1][0] = sxy[0] * (1.0 / 12.0);
+      H[0][2] = H[2][0] = sxy[1] * (1.0 / 12.0);
+      H[1][2] = H[2][1] = sxy[2] * (1.0 / 12.0);
     }
     double g2 = 0, tr = 0, gHg = 0, Hg[3] = {0, 0, 0};
     for (int a = 0; a < D; ++a) {
@@ -789,52 +913,65 @@ __global__ void k_adj_geometry(Ctx C, int glevel, GeoAdj G) {
     }
     const double mag = sqrt(g2);
     if (!(mag > 1e-12)) continue;  // n = 0, kappa = 0: no dependence
-    const double kap = (g2 * tr - gHg) / (mag * mag * mag);
+    const double im = 1.0 / mag, im3 = im * im * im;
+    const double kap = (g2 * tr - gHg) * im3;
     // l_g, l_H from l_n, l_kappa
     double nd = 0, lg[3] = {0, 0, 0}, lH[3][3] = {{0, 0, 0}, {0, 0, 0}, {0, 0, 0}};
-    for (int a = 0; a < D; ++a) nd += g[a] / mag * ln[a];
+    for (int a = 0; a < D; ++a) nd += g[a] * im * ln[a];
     for (int a = 0; a < D; ++a) {
-      lg[a] = (ln[a] - g[a] / mag * nd) / mag;
-      lg[a] += lk * ((2.0 * g[a] * tr - 2.0 * Hg[a]) / (mag * mag * mag) - 3.0 * kap * g[a] / g2);
-      for (int b = 0; b < D; ++b) lH[a][b] = lk * ((a == b ? g2 : 0.0) - g[a] * g[b]) / (mag * mag * mag);
+      lg[a] = (ln[a] - g[a] * im * nd) * im;
+      lg[a] += lk * ((2.0 * g[a] * tr - 2.0 * Hg[a]) * im3 - 3.0 * kap * g[a] * (im * im));
+      for (int b = 0; b < D; ++b) lH[a][b] = lk * ((a == b ? g2 : 0.0) - g[a] * g[b]) * im3;
     }
     // transpose of the closed-form fit
     double lP = 0, lsx[3] = {0, 0, 0}, lsxx[3] = {0, 0, 0}, lsxy[3] = {0, 0, 0}, la0 = 0, ls = 0, lR = 0;
     if (D == 2) {
       for (int a = 0; a < 2; ++a) {
-        lsx[a] = lg[a] / 6.0;
+        lsx[a] = lg[a] * (1.0 / 6.0);
         lsxx[a] += lH[a][a];
         la0 += -6.0 * lH[a][a];
         ls += -4.0 * lH[a][a];
       }
-      lsxy[0] = (lH[0][1] + lH[1][0]) / 4.0;
+      lsxy[0] = (lH[0][1] + lH[1][0]) * 0.25;
       lP += 5.0 / 9.0 * la0 - 4.0 / 6.0 * ls;
       lR += -3.0 / 9.0 * la0 + 3.0 / 6.0 * ls;
     } else {
       for (int a = 0; a < 3; ++a) {
-        lsx[a] = lg[a] / 18.0;
-        lsxx[a] += lH[a][a] / 3.0;
+        lsx[a] = lg[a] * (1.0 / 18.0);
+        lsxx[a] += lH[a][a] * (1.0 / 3.0);
         la0 += -6.0 * lH[a][a];
         ls += -4.0 * lH[a][a];
       }
-      lsxy[0] = (lH[0][1] + lH[1][0]) / 12.0;
-      lsxy[1] = (lH[0][2] + lH[2][0]) / 12.0;
-      lsxy[2] = (lH[1][2] + lH[2][1]) / 12.0;
+      lsxy[0] = (lH[0][1] + lH[1][0]) * (1.0 / 12.0);
+      lsxy[1] = (lH[0][2] + lH[2][0]) * (1.0 / 12.0);
+      lsxy[2] = (lH[1][2] + lH[2][1]) * (1.0 / 12.0);
       lP += 7.0 / 27.0 * la0 - 2.0 / 6.0 * ls;
       lR += -3.0 / 27.0 * la0 + 1.0 / 6.0 * ls;
     }
     for (int a = 0; a < D; ++a) lsxx[a] += lR;
-    for (int oz = (D == 3 ? -1 : 0); oz <= (D == 3 ? 1 : 0); ++oz)
-      for (int oy = -1; oy <= 1; ++oy)
-        for (int ox = -1; ox <= 1; ++ox) {
-          const int o[3] = {ox, oy, oz};
-          double lv = lP + ox * oy * lsxy[0];
-          if (D == 3) lv += ox * oz * lsxy[1] + oy * oz * lsxy[2];
-          for (int a = 0; a < D; ++a) lv += o[a] * lsx[a] + o[a] * o[a] * lsxx[a];
-          const int xx = clampwrap(L, 0, x + ox), yy = clampwrap(L, 1, y + oy);
-          const int zz = D == 3 ? clampwrap(L, 2, z + oz) : 0;
-          atomicAdd(G.phi + L.fine_off + cidx(L, xx, yy, zz), (float)lv);
+    float *gp = G.phi + L.fine_off;
+#pragma unroll
+    for (int k = 0; k < NZ; ++k) {
+      const int oz = D == 3 ? k - 1 : 0;
+      double pz = lP, ez = lsx[1], cz = lsx[0];  // of every point of the plane, its o_y and its o_x
+      if (oz) {
+        pz += oz > 0 ? lsxx[2] + lsx[2] : lsxx[2] - lsx[2];
+        ez += oz > 0 ? lsxy[2] : -lsxy[2];
+        cz += oz > 0 ? lsxy[1] : -lsxy[1];
+      }
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        double py = pz, cy = cz;
+        if (j != 1) {
+          py += j ? lsxx[1] + ez : lsxx[1] - ez;
+          cy += j ? lsxy[0] : -lsxy[0];
         }
+        const double px = py + lsxx[0];
+        atomicAdd(gp + cidx(L, xo[0], yo[j], zo[k]), (float)(px - cy));
+        atomicAdd(gp + cidx(L, xo[1], yo[j], zo[k]), (float)py);
+        atomicAdd(gp + cidx(L, xo[2], yo[j], zo[k]), (float)(px + cy));
+      }
+    }
   }
 }
 
@@ -1213,14 +1350,25 @@ __global__ void k_copy_blocks(Ctx C, BlockShape S, const int *list, int n, const
     return cudaGetLastError();                                                        \
   } while (0)
 
+#define LSB_ADJ_QB(Q, B, fn, L, ...)                                                  \
+  do {                                                                                \
+    if ((Q) == 9) fn<9, B><<<(L).grid, (L).block, 0, (L).stream>>>(__VA_ARGS__);      \
+    else fn<19, B><<<(L).grid, (L).block, 0, (L).stream>>>(__VA_ARGS__);              \
+    return cudaGetLastError();                                                        \
+  } while (0)
+
 cudaError_t run_adj_seed(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *F, float *lam,
                          const double *wobs, const double *obs, int stride, float eps, float *lphi) {
   LSB_ADJ_Q(Q, k_adj_seed, L, C, S, list, n, F, lam, wobs, obs, stride, eps, lphi);
 }
 
+cudaError_t run_adj_moments(int Q, Launch L, Ctx C, int glevel, const float *F) {
+  LSB_ADJ_Q(Q, k_adj_moments, L, C, glevel, F);
+}
 cudaError_t run_adj_links(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamN, float *LA, float *MA,
-                          double *grad, int ncase, GeoAdj G) {
-  LSB_ADJ_Q(Q, k_adj_links, L, C, glevel, F, lamN, LA, MA, grad, ncase, G);
+                          double *grad, int ncase, GeoAdj G, bool frozen) {
+  if (frozen) LSB_ADJ_QB(Q, true, k_adj_links, L, C, glevel, F, lamN, LA, MA, grad, ncase, G);
+  LSB_ADJ_QB(Q, false, k_adj_links, L, C, glevel, F, lamN, LA, MA, grad, ncase, G);
 }
 
 cudaError_t run_adj_geometry(int D, Launch L, Ctx C, int glevel, GeoAdj G) {
@@ -1242,8 +1390,9 @@ cudaError_t run_adj_collide(int Q, Launch L, Ctx C, BlockShape S, const int *lis
 }
 
 cudaError_t run_adj_macro(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamO, float *MA, double *grad,
-                          int ncase) {
-  LSB_ADJ_Q(Q, k_adj_macro, L, C, glevel, F, lamO, MA, grad, ncase);
+                          int ncase, bool frozen) {
+  if (frozen) LSB_ADJ_QB(Q, true, k_adj_macro, L, C, glevel, F, lamO, MA, grad, ncase);
+  LSB_ADJ_QB(Q, false, k_adj_macro, L, C, glevel, F, lamO, MA, grad, ncase);
 }
 
 cudaError_t run_copy_blocks(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *src,

@@ -1169,17 +1169,19 @@ lsb_status adj_lb(lsb_grid *g, int l, const float *F, float *lamN, float *lamO, 
   if (kappa) C.kappa = kappa;
   BlockShape S = shape(g);
   const int Q = g->Q;
-  const bool fine = l == g->Lmax - 1;
-  if (fine)
+  const bool fine = l == g->Lmax - 1, frozen = !g->rec_moving;
+  if (fine) {
+    if (frozen) RUN(KADJ_LINKS, 0, 1, 128, run_adj_moments, Q, LN(g, DYN_GRID, 128), C, l, F);
     RUN(KADJ_LINKS, 0, 1, 128, run_adj_links, Q, LN(g, DYN_GRID, 128), C, l, F, lamN, g->d_linkadj, g->d_madj,
-        g->d_grad, g->ncase, G);
+        g->d_grad, g->ncase, G, frozen);
+  }
   const int grid = std::min(g->cs[l].n, 152 * LSB_ADJ_MINB);  // the resident CTAs
   RUN(KADJ_COLLIDE, 3.0 * Q * sizeof(float) * g->leaf_cells[l], g->cs[l].n, g->nthreads, run_adj_collide, Q,
       LN(g, grid, g->nthreads), C, S, (const int *)g->cs[l].d, g->cs[l].n, F, (const float *)lamN, lamO,
-      (const float *)g->d_linkadj, g->d_grad, g->rec_moving ? 0 : 1);
+      (const float *)g->d_linkadj, g->d_grad, frozen ? 1 : 0);
   if (fine)
     RUN(KADJ_MACRO, 0, 1, 128, run_adj_macro, Q, LN(g, DYN_GRID, 128), C, l, F, lamO, g->d_madj, g->d_grad,
-        g->ncase);
+        g->ncase, frozen);
   return LSB_OK;
 }
 

@@ -133,14 +133,15 @@ struct GeoAdj {
 };
 cudaError_t run_adj_seed(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *F, float *lam,
                          const double *wobs, const double *obs, int stride, float eps, float *lphi);
+cudaError_t run_adj_moments(int Q, Launch L, Ctx C, int glevel, const float *F);
 cudaError_t run_adj_links(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamN, float *LA, float *MA,
-                          double *grad, int ncase, GeoAdj G);
+                          double *grad, int ncase, GeoAdj G, bool frozen);
 cudaError_t run_adj_geometry(int D, Launch L, Ctx C, int glevel, GeoAdj G);
 // moments: the transposed collision through lambda's weighted moments (see k_adj_collide)
 cudaError_t run_adj_collide(int Q, Launch L, Ctx C, BlockShape S, const int *list, int n, const float *F,
                             const float *lamN, float *lamO, const float *LA, double *grad, int moments);
 cudaError_t run_adj_macro(int Q, Launch L, Ctx C, int glevel, const float *F, float *lamO, float *MA, double *grad,
-                          int ncase);
+                          int ncase, bool frozen);
 // Multi-level grids: transposes of the ghost-ring transfer (per ghost cell of a
 // fine level, coarse states at t and t + 1 blended by theta), of its coarse
 // share's hand-over after the coarse sub-step, and of the restriction (per
