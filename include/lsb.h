@@ -202,7 +202,8 @@ lsb_status lsb_get_fields(lsb_grid *g, int case_idx, int field, int level, void 
 /*
  * Allocation-free variant of lsb_get_fields for LSB_FIELD_RHO, LSB_FIELD_U and
  * LSB_FIELD_F (the paper has no counterpart: this is a service of the library).
- * lsb_get_fields stages these fields in a temporary cudaMalloc buffer; this
+ * lsb_get_fields stages these fields in a temporary cudaMalloc buffer (unless dst is
+ * memory of the current device, which the export then writes itself); this
  * entry point stages them in a fixed 16 MiB array that the library reserves
  * on every GPU it is loaded on, held until the process exits.  It is meant
  * for callers that cannot allocate device memory at the point of the call:
