@@ -46,6 +46,8 @@ struct WorkList {
   int n = 0;
   int cap = 0;
   std::vector<int> h;
+  int4 *info = nullptr;  // beside each block id, for the lists that have hinfo: its blk_info entry
+  std::vector<int4> hinfo;
 };
 
 struct CellList {
@@ -221,8 +223,11 @@ lsb_status upload_list(lsb_grid *g, WorkList &w) {
     lsb_status s = dalloc(g, &p, sizeof(int) * (size_t)cap);
     if (s) return s;
     w.d = p;
+    if (!w.hinfo.empty() && (s = dalloc(g, &w.info, sizeof(int4) * (size_t)cap))) return s;
     w.cap = cap;
   }
+  if (!w.hinfo.empty())
+    CU(cudaMemcpyAsync(w.info, w.hinfo.data(), sizeof(int4) * w.n, cudaMemcpyHostToDevice, g->stream));
   if (w.n) CU(cudaMemcpyAsync(w.d, w.h.data(), sizeof(int) * w.n, cudaMemcpyHostToDevice, g->stream));
   return LSB_OK;
 }
@@ -437,6 +442,7 @@ bool any_neighbor(const lsb_grid *g, const LevelDev &L, const std::vector<int8_t
 lsb_status build_lists(lsb_grid *g) {
   for (int l = 0; l < MAXL; ++l) {
     g->cs[l].h.clear();
+    g->cs[l].hinfo.clear();
     g->rst[l].h.clear();
     g->ghost[l].h.clear();
     g->finest[l].h.clear();
@@ -454,19 +460,23 @@ lsb_status build_lists(lsb_grid *g) {
       const int8_t s = st[b];
       bool near_leaf = any_neighbor(g, L, st, b, BLK_LEAF, false);
       bool near_active = any_neighbor(g, L, st, b, 0, true);
-      if (s == BLK_LEAF) {
-        int bc[3];
+      auto collides = [&](int bc[3]) {
         block_coords(L, b, bc);
+        g->cs[l].h.push_back(gb);
+        g->cs[l].hinfo.push_back(make_int4((int)ld, bc[0], bc[1], bc[2]));
+      };
+      int bc[3];
+      if (s == BLK_LEAF) {
+        collides(bc);
         double cnt = 1;
         for (int a = 0; a < 3; ++a) cnt *= std::min(g->bs[a], L.n[a] - bc[a] * g->bs[a]);
         g->leaf_cells[l] += cnt;
-        g->cs[l].h.push_back(gb);
         g->leaf.h.push_back(gb);
         if (L.finest) g->finest[l].h.push_back(gb);
       }
       if (s != BLK_INACTIVE) g->all_active.h.push_back(gb);
       if (s == BLK_REFINED && near_leaf) {
-        g->cs[l].h.push_back(gb);
+        collides(bc);
         g->rst[l].h.push_back(gb);
       }
       if (s == BLK_INACTIVE && near_active && l > 0) g->ghost[l].h.push_back(gb);
@@ -681,7 +691,7 @@ lsb_status coarse_side(lsb_grid *g, int l) {
   const int grid = std::min(g->cs[l].n, std::max(1, g->tma_grid / LSB_SIDE_DIV));
   const CUtensorMap *tm = (const CUtensorMap *)g->d_tmaps;
   RUN(collide_kid(l), cs_bytes, g->cs[l].n, nt, run_collide_stream_tma, Q, st, Launch{grid, nt, g->side[l]}, C, S,
-      (const int *)g->cs[l].d, g->cs[l].n, tm, g->tma_tags ? tm + 2 * g->lds.size() : nullptr, work_counters(g, l));
+      (const int4 *)g->cs[l].info, g->cs[l].n, tm, g->tma_tags ? tm + 2 * g->lds.size() : nullptr, work_counters(g, l));
   CU(cudaEventRecord(g->ev_join[l], g->side[l]));
   return LSB_OK;
 }
@@ -722,7 +732,7 @@ lsb_status advance(lsb_grid *g, int l) {
     const int grid = std::min(g->cs[l].n, g->tma_grid);
     const CUtensorMap *tm = (const CUtensorMap *)g->d_tmaps;
     RUN(collide_kid(l), cs_bytes, g->cs[l].n, nt, run_collide_stream_tma, Q, st, LN(g, grid, nt), C, S,
-        (const int *)g->cs[l].d, g->cs[l].n, g->tma_a ? g->tma_a : tm, g->tma_tags ? tm + 2 * g->lds.size() : nullptr,
+        (const int4 *)g->cs[l].info, g->cs[l].n, g->tma_a ? g->tma_a : tm, g->tma_tags ? tm + 2 * g->lds.size() : nullptr,
         work_counters(g, l));
   } else {
     RUN(collide_kid(l), cs_bytes, g->cs[l].n, nt, run_collide_stream, Q, st, LN(g, g->cs[l].n, nt), C, S, (const int *)g->cs[l].d,

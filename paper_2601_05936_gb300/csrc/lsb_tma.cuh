@@ -49,6 +49,11 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const void *tmap, int c0,
       "l"(tmap), "r"(c0), "r"(c1), "r"(c2), "r"(smem_u32(bar))
       : "memory");
 }
+// 16 bytes to shared memory without a register; visible to the issuing thread after cp_async_wait.
+__device__ __forceinline__ void cp_async_16(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 constexpr unsigned kWaitLimit = 1u << 24;
 
