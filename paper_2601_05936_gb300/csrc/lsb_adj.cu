@@ -164,8 +164,8 @@ __global__ void k_adj_seed(Ctx C, BlockShape S, const int *list, int nlist, cons
 // its links.  Per link their order varies from run to run, and reinitialisation's transpose
 // turns that round-off into 2e-5 of dJ/dphi (41 x 92, 8 steps) where it was 1e-8.
 
-// Moments and strain rate of every interface cell's populations in F, into the macro planes
-// (drho, u[D], S): scratch during a reverse sweep, every forward step writes them before it
+// Moments and strain rate of every interface cell's populations in F, into their
+// MacroRec (drho, u[D], S): scratch during a reverse sweep, every forward step writes them before it
 // reads them.
 template <int Q>
 __global__ void k_adj_moments(Ctx C, int glevel, const float *__restrict__ F) {
@@ -184,11 +184,15 @@ __global__ void k_adj_moments(Ctx C, int glevel, const float *__restrict__ F) {
 #pragma unroll
     for (int j = 0; j < Q; ++j) f[j] = Fl[j * N + c];
     moments_strain<Q>(f, L.omega[A], r, u, S);
-    C.macro[fc] = r;
+    MacroRec<D> M;
+    M.v[0] = r;
 #pragma unroll
-    for (int a = 0; a < D; ++a) C.macro[(1 + a) * NF + fc] = u[a];
+    for (int a = 0; a < D; ++a) M.v[1 + a] = u[a];
 #pragma unroll
-    for (int k = 0; k < NS; ++k) C.macro[(1 + D + k) * NF + fc] = S[k];
+    for (int k = 0; k < NS; ++k) M.v[1 + D + k] = S[k];
+#pragma unroll
+    for (int k = 1 + D + NS; k < MacroRec<D>::N; ++k) M.v[k] = 0.f;
+    M.store(C.macro, fc);
   }
 }
 
@@ -206,7 +210,6 @@ __global__ void __launch_bounds__(128) k_adj_links(Ctx C, int glevel, const floa
                            : (long long)min(C.counters[glevel * NCOUNT + 1], (int)C.list_cap);
   const int2 *lst = LINK ? C.link_cell + C.link_list_off[glevel] : C.iface_list + (long long)glevel * C.list_cap;
   const long long NF = C.nfine;
-  const float *M = C.macro;
   // (every lane of a warp makes the same rounds: the parameter partials are summed over it)
   for (long long e0 = blockIdx.x * (long long)blockDim.x; e0 < n; e0 += (long long)gridDim.x * blockDim.x) {
     const long long e = e0 + threadIdx.x;
@@ -232,11 +235,13 @@ __global__ void __launch_bounds__(128) k_adj_links(Ctx C, int glevel, const floa
       float f[Q];
       float rA, uA[3] = {0.f, 0.f, 0.f}, SA[6];
       if (LINK) {
-        rA = M[fo + c];
+        MacroRec<D> M;
+        M.load(C.macro, fo + c);
+        rA = M.rho();
 #pragma unroll
-        for (int a = 0; a < D; ++a) uA[a] = M[(1 + a) * NF + fo + c];
+        for (int a = 0; a < D; ++a) uA[a] = M.u(a);
 #pragma unroll
-        for (int s = 0; s < NS; ++s) SA[s] = M[(1 + D + s) * NF + fo + c];
+        for (int s = 0; s < NS; ++s) SA[s] = M.S(s);
       } else {
 #pragma unroll
         for (int j = 0; j < Q; ++j) f[j] = Fl[j * N + c];
@@ -286,11 +291,13 @@ __global__ void __launch_bounds__(128) k_adj_links(Ctx C, int glevel, const floa
         // forward pieces of Eq. bb_cc at this link
         float rB, uB[3] = {0.f, 0.f, 0.f}, SB[6];
         if (LINK) {
-          rB = M[my];
+          MacroRec<D> M;
+          M.load(C.macro, my);
+          rB = M.rho();
 #pragma unroll
-          for (int a = 0; a < D; ++a) uB[a] = M[(1 + a) * NF + my];
+          for (int a = 0; a < D; ++a) uB[a] = M.u(a);
 #pragma unroll
-          for (int s = 0; s < NS; ++s) SB[s] = M[(1 + D + s) * NF + my];
+          for (int s = 0; s < NS; ++s) SB[s] = M.S(s);
         } else {
           float fy[Q];
 #pragma unroll
@@ -710,7 +717,7 @@ __global__ void __launch_bounds__(512, LSB_ADJ_MINB) k_adj_collide(Ctx C, BlockS
 //
 // Latency-bound: lamO's values are loaded before the sums they join (loads and stores of one
 // array would wait for one another).  Frozen level set (MOM): drho, u and S come from
-// k_adj_moments' planes, Pi_ab = S_ab / k, and F is not read: 37 -> 31 us on the 33 k cells of
+// k_adj_moments, Pi_ab = S_ab / k, and F is not read: 37 -> 31 us on the 33 k cells of
 // the 3D bubble.  Moving: from F as the oracle has it (round-off is amplified, see k_adj_links).
 template <int Q, bool MOM>
 __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, float *lamO, float *MA, double *grad,
@@ -746,11 +753,13 @@ __global__ void k_adj_macro(Ctx C, int glevel, const float *__restrict__ F, floa
     float d = 0.f, j[3] = {0.f, 0.f, 0.f}, m2[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     float uM[3] = {0.f, 0.f, 0.f};
     if (MOM) {
-      d = C.macro[fc];
+      MacroRec<D> M;
+      M.load(C.macro, fc);
+      d = M.rho();
 #pragma unroll
-      for (int a = 0; a < D; ++a) uM[a] = C.macro[(1 + a) * NF + fc];
+      for (int a = 0; a < D; ++a) uM[a] = M.u(a);
 #pragma unroll
-      for (int k = 0; k < NS; ++k) m2[k] = C.macro[(1 + D + k) * NF + fc];
+      for (int k = 0; k < NS; ++k) m2[k] = M.S(k);
     }
 #pragma unroll
     for (int i = 0; i < (MOM ? 0 : Q); ++i) {

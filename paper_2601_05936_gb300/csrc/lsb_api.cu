@@ -219,11 +219,12 @@ lsb_status upload_list(lsb_grid *g, WorkList &w) {
   w.n = (int)w.h.size();
   if (w.n > w.cap) {
     int cap = std::max(w.n, 64);
-    int *p = nullptr;
-    lsb_status s = dalloc(g, &p, sizeof(int) * (size_t)cap);
+    const size_t info = w.hinfo.empty() ? 0 : sizeof(int4) * (size_t)cap;  // in front of the ids
+    char *p = nullptr;
+    lsb_status s = dalloc(g, &p, info + sizeof(int) * (size_t)cap);
     if (s) return s;
-    w.d = p;
-    if (!w.hinfo.empty() && (s = dalloc(g, &w.info, sizeof(int4) * (size_t)cap))) return s;
+    w.info = info ? (int4 *)p : nullptr;
+    w.d = (int *)(p + info);
     w.cap = cap;
   }
   if (!w.hinfo.empty())
@@ -1497,7 +1498,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
   const long long nf = g->nfine;
   const int Q = g->Q;
   const size_t fsz = g->storage == LSB_FP32 ? 4 : 2;
-  const int MF = 1 + D + D * (D + 1) / 2;
+  const int MREC = D == 2 ? MacroRec<2>::N : MacroRec<3>::N;
   g->list_cap = std::min<long long>(nf, std::max<long long>(1 << 16, nf / 4));
   g->link_cap = std::min<long long>((long long)Q * nf, std::max<long long>(1 << 18, 2 * nf));
   g->band_cap = 0;
@@ -1529,7 +1530,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
   ALLOC(g->d_plan_f, nf);
   ALLOC(g->d_cmask, 4 * nf);
   ALLOC(g->d_cbase, 4 * nf);
-  ALLOC(g->d_macro, 4 * (size_t)MF * nf);
+  ALLOC(g->d_macro, 4 * (size_t)MREC * nf);
   ALLOC(g->d_nvec, 4 * D * nf);
   ALLOC(g->d_kappa, 4 * nf);
   ALLOC(g->d_linkbuf, 8 * g->link_cap);
@@ -1592,7 +1593,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
       cuerr(cudaMemset(g->d_cmask, 0, 4 * nf), "cmask") ||
       cuerr(cudaMemset(g->d_nvec, 0, 4 * D * nf), "nvec") ||
       cuerr(cudaMemset(g->d_kappa, 0, 4 * nf), "kappa") ||
-      cuerr(cudaMemset(g->d_macro, 0, 4 * (size_t)MF * nf), "macro") ||
+      cuerr(cudaMemset(g->d_macro, 0, 4 * (size_t)MREC * nf), "macro") ||
       cuerr(cudaMemset(g->d_buf[0], 0, fsz * Q * g->ncell_total), "buf0") ||
       cuerr(cudaMemset(g->d_buf[1], 0, fsz * Q * g->ncell_total), "buf1")) {
     lsb_destroy(g);

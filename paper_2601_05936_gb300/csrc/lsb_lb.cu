@@ -135,7 +135,7 @@ __device__ __forceinline__ void cumulant_collide27(float *f, float om, const flo
 }
 
 // drho, u and the strain rate of an interface cell's pre-collision populations, kept for the
-// interface condition (Eq. bb_cc, Sdecomp) in the finest-level macro planes (drho, u[D], S):
+// interface condition (Eq. bb_cc, Sdecomp) in the cell's MacroRec (drho, u[D], S):
 // S = -(om / (2 rho c_s^2)) sum_i c_i c_i (f_i - feq_i).  In deviation form the equilibrium's
 // second moments are sum_i c_a c_b f~eq_i = drho c_s^2 delta_ab + rho u_a u_b, for the BGK
 // equilibrium and for the cumulant model's Gaussian alike, so no per-population feq is needed.
@@ -164,19 +164,22 @@ __device__ __forceinline__ void store_iface_macro(const Ctx &C, long long fc, Ld
   const float drho = d, inv = 1.0f / (1.0f + d);
   const float u[3] = {jx * inv, jy * inv, jz * inv};
   const float rho = 1.0f + drho, s = -1.5f * om / rho, iso = CS2 * drho;
-  const long long NF = C.nfine;
-  float *M = C.macro;
-  M[fc] = drho;
-  for (int a = 0; a < D; ++a) M[(1 + a) * NF + fc] = u[a];
+  MacroRec<D> M;
+  M.v[0] = drho;
+#pragma unroll
+  for (int a = 0; a < D; ++a) M.v[1 + a] = u[a];
   const float sxx = s * (pxx - iso - rho * u[0] * u[0]), sxy = s * (pxy - rho * u[0] * u[1]);
   const float syy = s * (pyy - iso - rho * u[1] * u[1]);
   if (D == 2) {
-    M[3 * NF + fc] = sxx; M[4 * NF + fc] = sxy; M[5 * NF + fc] = syy;
+    M.v[3] = sxx; M.v[4] = sxy; M.v[5] = syy;
+    M.v[6] = M.v[7] = 0.f;
   } else {
-    M[4 * NF + fc] = sxx; M[5 * NF + fc] = sxy; M[6 * NF + fc] = s * (pxz - rho * u[0] * u[2]);
-    M[7 * NF + fc] = syy; M[8 * NF + fc] = s * (pyz - rho * u[1] * u[2]);
-    M[9 * NF + fc] = s * (pzz - iso - rho * u[2] * u[2]);
+    M.v[4] = sxx; M.v[5] = sxy; M.v[6] = s * (pxz - rho * u[0] * u[2]);
+    M.v[7] = syy; M.v[8] = s * (pyz - rho * u[1] * u[2]);
+    M.v[9] = s * (pzz - iso - rho * u[2] * u[2]);
+    M.v[10] = M.v[11] = 0.f;
   }
+  M.store(C.macro, fc);
 }
 
 // The cell's phase operator: BGK, or on D3Q27 the cumulant model where the level asks for it.
@@ -636,16 +639,17 @@ __device__ __forceinline__ void d_interface_bc(const Ctx &C, int glevel, int b0,
     const int Bp = 1 - A;
     const long long N = L.ncell;
     T *Bf = fB<T, Q>(C, L);
-    const float *M = C.macro;
+    MacroRec<D> MA, MB;
+    MA.load(C.macro, fo + c);
     const float phx = C.phi[fo + c];
-    const float rA = M[fo + c];
+    const float rA = MA.rho();
     float uA[3] = {0.f, 0.f, 0.f}, SA[6] = {0, 0, 0, 0, 0, 0}, nx[3] = {0.f, 0.f, 0.f};
     for (int a = 0; a < D; ++a) {
-      uA[a] = M[(1 + a) * NF + fo + c];
+      uA[a] = MA.u(a);
       nx[a] = C.nvec[a * NF + fo + c];
     }
-    const int MS = 1 + D;
-    for (int s = 0; s < D * (D + 1) / 2; ++s) SA[s] = M[(MS + s) * NF + fo + c];
+#pragma unroll
+    for (int s = 0; s < D * (D + 1) / 2; ++s) SA[s] = MA.S(s);
     const float kx = C.kappa[fo + c];
     const float etaA = L.eta[A], etaB = L.eta[Bp];
     const float eta_bar = 0.5f * (etaA + etaB);
@@ -658,6 +662,7 @@ __device__ __forceinline__ void d_interface_bc(const Ctx &C, int glevel, int b0,
       int yx = x + LT::cx(i), yy = y + LT::cy(i), yz = z + LT::cz(i);
       wrap(L, 0, yx); wrap(L, 1, yy); if (D == 3) wrap(L, 2, yz);
       const long long cy_ = cidx(L, yx, yy, yz);
+      MB.load(C.macro, fo + cy_);
       const float phy = C.phi[fo + cy_];
       const float q = phx / (phx - phy);
       // u_I, n, kappa along the link; Sbar, [p], eta from the two nodes
@@ -665,15 +670,16 @@ __device__ __forceinline__ void d_interface_bc(const Ctx &C, int glevel, int b0,
       float nn = 0.f;
       for (int a = 0; a < 3; ++a) { uI[a] = 0.f; nv[a] = 0.f; }
       for (int a = 0; a < D; ++a) {
-        uI[a] = (1.0f - q) * uA[a] + q * M[(1 + a) * NF + fo + cy_];
+        uI[a] = (1.0f - q) * uA[a] + q * MB.u(a);
         nv[a] = (1.0f - q) * nx[a] + q * C.nvec[a * NF + fo + cy_];
         nn += nv[a] * nv[a];
       }
       nn = sqrtf(nn);
       for (int a = 0; a < D; ++a) nv[a] = nn > 0.f ? sgn * nv[a] / nn : 0.f;
       const float kap = sgn * ((1.0f - q) * kx + q * C.kappa[fo + cy_]);
-      for (int s = 0; s < D * (D + 1) / 2; ++s) Sb[s] = 0.5f * (SA[s] + M[(MS + s) * NF + fo + cy_]);
-      const float rB = M[fo + cy_];
+#pragma unroll
+      for (int s = 0; s < D * (D + 1) / 2; ++s) Sb[s] = 0.5f * (SA[s] + MB.S(s));
+      const float rB = MB.rho();
       const float jp = CS2 * (L.rho_phys[Bp] * rB - L.rho_phys[A] * rA);
       // symmetric tensor access
       auto Sget = [&](int a, int b) -> float {

@@ -1486,11 +1486,23 @@ cudaError_t lsf_prepare(LsfLimits *out) {
   e = cudaFuncSetAttribute(k_levelset_fused<Q, 0>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_levelset_fused<Q, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e == cudaSuccess) e = cudaFuncSetAttribute(k_levelset_fused<Q, 0>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_levelset_fused<Q, 1>, 1024, smem);
+  if (e != cudaSuccess) return e;
+  out->max_ld = kLsfMaxLd;
+  // what fits on a device is asked once per device, not for every handle (64 x 32 channel: a handle's
+  // creation 0.55 ms; 0.53 without this launch to prepare at all)
+  constexpr int kDevs = 64;
+  static std::mutex mu;
+  static LsfLimits known[kDevs];  // (grid, cluster; cluster 0: not asked yet)
+  std::lock_guard<std::mutex> lock(mu);
+  if (dev < kDevs && known[dev].cluster) {
+    out->grid = known[dev].grid;
+    out->cluster = known[dev].cluster;
+    return cudaSuccess;
+  }
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_levelset_fused<Q, 1>, 1024, smem);
   if (e != cudaSuccess) return e;
   out->grid = coop && nb > 0 ? sms : 0;
   out->cluster = 8;
-  out->max_ld = kLsfMaxLd;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute at;
   at.id = cudaLaunchAttributeClusterDimension;
@@ -1504,6 +1516,7 @@ cudaError_t lsf_prepare(LsfLimits *out) {
   int nc = 0;
   if (cudaOccupancyMaxActiveClusters(&nc, k_levelset_fused<Q, 0>, &cfg) == cudaSuccess && nc > 0) out->cluster = 16;
   else cudaGetLastError();
+  if (dev < kDevs) known[dev] = *out;
   return cudaSuccess;
 }
 cudaError_t prepare_levelset_fused(int Q, LsfLimits *out) {
