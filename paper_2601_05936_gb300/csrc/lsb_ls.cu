@@ -529,8 +529,8 @@ __device__ __forceinline__ void ext_sweep_cell(const Ctx &C, const LevelDev &L, 
 }
 
 // TVD-RK3 transport stage at one band cell (as d_adv_stage).  Stage 1 takes u~ from the
-// last extension sweep (ufin; nullptr: ut0, no sweeps) and commits it to ut0 and both
-// sweep buffers at the cell.
+// last extension sweep (ufin; nullptr: ut0, no sweeps) and commits it to ut0; stage 2 also to
+// both sweep buffers at the cell.
 template <int D>
 __device__ __forceinline__ void adv_cell(const Ctx &C, const LevelDev &L, int x, int y, int z, int stage,
                                          const typename UVec<D>::T *ufin, typename UVec<D>::T *ub1,
@@ -543,8 +543,9 @@ __device__ __forceinline__ void adv_cell(const Ctx &C, const LevelDev &L, int x,
   if (stage == 1 && ufin) u_get(ufin[fc], ua);
   else
     for (int a = 0; a < D; ++a) ua[a] = C.ut0[a * NF + fc];
-  if (stage == 1) {
+  if (stage == 1)
     for (int a = 0; a < D; ++a) C.ut0[a * NF + fc] = ua[a];
+  if (stage == 2) {  // (not in stage 1, beside which the last sweep may still run)
     u_put(ub1[fc], ua, 0.f);
     u_put(ub2[fc], ua, 0.f);
   }
@@ -635,7 +636,9 @@ __device__ __forceinline__ void reinit_cell(const Ctx &C, const LevelDev &L, int
 // Everything the level set does in a finest sub-step after the interface pass, in one
 // launch: n_ext extension sweeps, three transport stages, the reinitialisation, and the
 // phase and cut-link passes of the classification (16 passes by default), with a barrier
-// between passes.  As launches of their own the passes are bound by their chains: ~1 us
+// between them but for two places where a pass needs its own cells' values only: the first
+// transport stage behind the last sweep, and the phases behind the last stage (barriers there
+// cost 3 us of the launch's 47 over the 2D ensemble, 6 of 157 on the 3D bubble).  As launches of their own the passes are bound by their chains: ~1 us
 // for the launch, then band count, band entry, level descriptor, plan, neighbours, one L2
 // round trip each.  Here a CTA's cells stay its own for all passes: each thread sets up
 // its band cells once (slots) and keeps their offsets, flags, extension velocity and
@@ -910,7 +913,8 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       if (ok) ext_sweep_cell<D>(C, L, x, y, z, uin, uout);
     }
     uin = uout;
-    if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+    // (the first transport stage reads phi and its own cells' u~: no barrier before it)
+    if (it < n_ext - 1 && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
   }
   // values around a cell (at pc) along axis a at offsets -3..+3, or mirrored; last: the
   // highest index wanted
@@ -943,9 +947,12 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
 #pragma unroll
       for (int a = 0; a < D; ++a)  // upwind side by the sign of u~: the mirrored stencil is the same sum negated
         gather(pin + fc, g, fl, a, !(ua[a] >= 0.f), v[a], 5);
-      if (stage == 1) {  // commit u~ (the buffer of the last sweep holds it)
+      // commit u~ (the buffer of the last sweep holds it; the other one's old values are read
+      // until the barrier behind stage 1)
+      if (stage == 1) {
 #pragma unroll
         for (int a = 0; a < D; ++a) C.ut0[a * NF + fc] = ua[a];
+      } else if (stage == 2) {
         if (uin != ub1) u_put(ub1[fc], ua, 0.f);
         if (uin != ub2) u_put(ub2[fc], ua, 0.f);
       }
@@ -977,7 +984,9 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       const LevelDev &L = beyond(k, x, y, z, ok);
       if (ok) adv_cell<D>(C, L, x, y, z, stage, uin, ub1, ub2);
     }
-    if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+    // (the phases read their own cells' phi and leave p2, which the last stage's neighbours
+    // read, as it is: no barrier between them)
+    if ((stage < 3 || n_re > 0) && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
   }
   // ---- reinitialisation
   for (int r = 0; r < n_re; ++r)
@@ -1030,9 +1039,9 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
         const LevelDev &L = beyond(k, x, y, z, ok);
         if (ok) reinit_cell<Q>(C, L, x, y, z, stage, prep);
       }
-      if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+      if ((stage < 3 || r < n_re - 1) && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
     }
-  // ---- phases (k_classify_phase without init): p1, p2 back to phi, tags, flips
+  // ---- phases (k_classify_phase without init): p1 (p2 below) back to phi, tags, flips
   for (int k = 0; k < kn; ++k) {
     const int w = w0 + k * GB;
     unsigned fc;
@@ -1060,7 +1069,6 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     const uint8_t tg = C.tag[tc];
     if (!(tg & TAG_LEAF)) continue;
     C.p1[fc] = ph;
-    C.p2[fc] = ph;
     const int gas = ph >= 0.0f ? 1 : 0, prev = tg & TAG_GAS;
     C.tag[tc] = (tg & (TAG_LEAF | TAG_RLAYER | TAG_GHOST)) | (gas ? TAG_GAS : 0) | (prev ? TAG_PREVGAS : 0) |
                 (gas != prev ? TAG_FLIP : 0);
@@ -1088,14 +1096,17 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       uint8_t tg = 0;
       int ld = 0;
       bool cell, edge;
+      float ph = 0.f;
       gb = w < nl ? lst[w] : chk[w - nl];
       if (k < ks && w < nl) {
         const unsigned fl = SM[k].fl[tid];
+        ph = SM[k].v[tid].x;
         ld = (int)(fl >> SL_LD);
         cell = (fl & SL_CELL) != 0;
         edge = (fl & SL_EDGE) != 0;
         dist = fl >> SL_DIST;
         if (cell) fc = SM[k].fc[tid];
+        if (cell && !(fl & SL_LIVE)) ph = C.phi[fc];
       } else {
         const int4 b = C.blk_info[gb];
         ld = b.x;
@@ -1107,6 +1118,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
         if (cell) {
           fc = g.fo + (unsigned)crd[0] + (unsigned)(g.p0 * crd[1] + g.p01 * crd[2]);
           dist = lsf_dist<D>(crd, g.n);
+          if (w < nl) ph = C.phi[fc];
         }
       }
       const LsfGeo g = geo_of((unsigned)ld);
@@ -1114,6 +1126,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       if (cell) {
         tg = C.tag[tc];
         if (tg & TAG_LEAF) {
+          if (w < nl) C.p2[fc] = ph;
           m = edge ? cut_mask<Q>(C.tag + tc, tg, lsf_near<D>(g, dist)) : cut_mask_inner<Q>(C.tag + tc, tg, g.p0, g.p01);
           C.cmask[fc] = m;
         }
