@@ -161,11 +161,11 @@ def cpu_baseline(budget_s=20.0, warmup=0, compare_storage=None):
 # dram__bytes_write.sum per level's launch class) on a workload, with the sha1 of the kernel
 # sources the capture was taken on: a change to them voids the figure (traffic null).
 TRAFFIC = dict(
-    sources_sha1="2a97239a19b27e02f71529324b044a1e865e204e",
+    sources_sha1="dcaa2f4e5d8d4ca455eb483f9e5948f4a3848571",
     # 3D rising bubble 128x128x256, two levels, FP32: one coarse step after the warm-up
-    # (level 0, then the two level-1 sub-steps: 260.6 and 260.2 MB)
-    per_launch={("bubble3d", 1.0, "fp32"): {"k_collide_stream": 327672064 + 251297280,
-                                            "k_collide_stream_l1": (161361408 + 99237632 + 161222400 + 98941696) / 2}})
+    # (level 0, then the two level-1 sub-steps: 255.4 and 256.5 MB)
+    per_launch={("bubble3d", 1.0, "fp32"): {"k_collide_stream": 329013504 + 251797760,
+                                            "k_collide_stream_l1": (159134976 + 96259072 + 159558400 + 96927744) / 2}})
 
 
 def kernel_sources_sha1():

@@ -254,7 +254,8 @@ class Grid:
         self._check(self.lib.lsb_use_graphs(self.h, 1 if enable else 0))
 
     def set_driver(self, mode):
-        """0: one launch per level-set pass; 1: one persistent cooperative launch per finest step."""
+        """0: the level-set update and the cell classification in one launch per finest step; 1: the persistent
+        cooperative level-set launch, whose passes look the band up per stencil point."""
         self._check(self.lib.lsb_set_driver(self.h, int(mode)))
 
     def set_objective(self, eps=1.5):
