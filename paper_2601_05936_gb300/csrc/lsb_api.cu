@@ -1822,6 +1822,7 @@ lsb_status lsb_get_fields(lsb_grid *g, int case_idx, int field, int level, void 
     const int fcode = field == LSB_FIELD_RHO ? 0 : (field == LSB_FIELD_U ? 1 : 4);
     const int grid = (int)std::min<size_t>((n + 255) / 256, EXPORT_CTAS);
     if (!dst_on_host && device_writable(g, dst, need)) {
+      TRY(pin_host(g));  // (nothing may fail between the launch and lsb_sync's wait for it)
       TRY(launched(g, run_export(g->Q, g->storage, LN(g, grid, 256), make_ctx(g), ld, fcode, (float *)dst)));
       return lsb_sync(g);
     }
