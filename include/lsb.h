@@ -164,7 +164,8 @@ lsb_status lsb_use_graphs(lsb_grid *g, int enable);
  * TVD-RK3 transport, reinitialisation).  mode 0 (default): the passes and the
  * classification's phase and cut-link passes in one launch per finest step, on
  * stage arrays that need no band lookups (one thread-block cluster for a small
- * band, a cooperative launch with bounded device-wide barriers otherwise).
+ * band, a cooperative launch with device-wide barriers otherwise, bounded by
+ * lsb_set_wait_limit as those of mode 1).
  * mode 1: one persistent cooperative launch per finest step that runs the
  * level-set passes over the band work list of all cases with a lookup per
  * stencil point, and a device-wide barrier between passes; the barrier's wait
@@ -175,14 +176,16 @@ lsb_status lsb_use_graphs(lsb_grid *g, int enable);
 lsb_status lsb_set_driver(lsb_grid *g, int mode);
 
 /*
- * Iteration limit of the library's bounded device-side waits (the grid barrier
- * of lsb_set_driver mode 1; the paper has no counterpart).  A waiting CTA
- * sleeps ~64 ns per iteration and, after `spins` iterations, records the
- * timeout, leaves the kernel, and the next synchronising call returns
- * LSB_ETIMEOUT (a latched error: the handle stays in error; the CUDA context
- * stays usable).  Default 2^22 (~0.3 s).  0 makes every wait that would have to
- * wait give up at once, which exercises the timeout path without a stalled
- * GPU.  Errors: LSB_EINVAL (negative spins).
+ * Iteration limit of the library's device-wide barriers: those of the level-set
+ * update (lsb_set_driver mode 1, and mode 0 where its launch is the cooperative one)
+ * and of the reverse sweep over a moving level set (the paper has no counterpart).  A
+ * waiting CTA reads the barrier's word once per iteration (mode 1 sleeps ~64 ns
+ * between) and, after `spins` iterations, records the timeout, leaves the kernel, and
+ * the next synchronising call (lsb_backward among them) returns LSB_ETIMEOUT (a
+ * latched error: the handle stays in error; the CUDA context stays usable).  Default
+ * 2^22 (0.3 s or more).  0 makes every such barrier give up at once, which exercises
+ * the timeout path without a stalled GPU.  Not covered: the hardware barrier of a
+ * thread-block cluster (mode 0 with a small band).  Errors: LSB_EINVAL (negative spins).
  */
 lsb_status lsb_set_wait_limit(lsb_grid *g, long long spins);
 

@@ -105,7 +105,7 @@ struct lsb_grid {
   LsfLimits lsf_lim;
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
   int band_est[MAXL] = {0, 0, 0, 0};  // band blocks when it was planned
-  long long wait_limit = 1LL << 22;  // sleeps of ~64 ns before a device-side wait gives up
+  long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
   int driver = 0;             // 0: one launch per level-set pass, 1: one persistent launch
@@ -591,7 +591,7 @@ lsb_status levelset(lsb_grid *g, int l) {
   }
   const bool due = g->reinit_every > 0 && ((g->fine_steps[l] + 1) % g->reinit_every == 0);
   RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
-      (int)g->lds.size(), g->d_bar + 2);
+      (int)g->lds.size(), g->d_bar + 2, g->wait_limit);
   g->classified[l] = true;
   return LSB_OK;
 }
@@ -1223,7 +1223,7 @@ lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *u
   RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l);
   const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
   RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, g->band_est[l]), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
-      g->d_bar + 2);
+      g->d_bar + 2, g->wait_limit);
   RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, P.A.LU, g->d_madj, P.A.LP);
   // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LP
   const GeoAdj G{P.A.LP, g->d_gn, g->d_gk};
@@ -1742,9 +1742,10 @@ lsb_status lsb_sync(lsb_grid *g) {
   CU(cudaStreamSynchronize(g->stream));
   const int e = *g->h_err;
   g->latched |= e;
+  // first the timeout: the lists of an update that gave up are half made, and may overflow after it
+  if (g->latched & ERR_TIMEOUT) return fail(g, LSB_ETIMEOUT, "a bounded device-side wait gave up");
   if (g->latched & (ERR_LINK_OVF | ERR_LIST_OVF | ERR_BAND_OVF))
     return fail(g, LSB_ENOMEM, "device work list overflow (flags %d)", g->latched);
-  if (g->latched & ERR_TIMEOUT) return fail(g, LSB_ETIMEOUT, "a bounded device-side wait gave up");
   if (g->latched & ERR_NONFINITE) return fail(g, LSB_EUNSTABLE, "non-finite density or velocity");
   return LSB_OK;
 }

@@ -646,7 +646,7 @@ __device__ __forceinline__ void reinit_cell(const Ctx &C, const LevelDev &L, int
 //
 // MODE 0: the grid is one thread-block cluster and the barrier is the cluster's.
 // MODE 1: a cooperative launch; the barrier counts arrivals in bar[0] (one release-add per
-// CTA, polled with an iteration limit; a barrier that gives up sets ERR_TIMEOUT and ends
+// CTA, polled up to the handle's wait limit; a barrier that gives up sets ERR_TIMEOUT and ends
 // the CTA).  bar[1] counts CTAs that left: the last one clears both words for the next launch.
 // Measured per pass, one store and two neighbour loads per thread: a launch of its own in a
 // captured graph 3.8 us, grid barrier 1.4 us (152 CTAs), cluster barrier 0.6 - 1.0 us
@@ -739,7 +739,7 @@ template <int D> struct LsfSlot {
 };
 template <int Q, int MODE>
 __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                                                            int kcap, unsigned *bar) {
+                                                            int kcap, unsigned *bar, long long limit) {
   constexpr int D = Lat<Q>::D;
   using V = typename UVec<D>::T;
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -858,7 +858,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     if (ok && n_ext > 0) ext_first_cell<D>(C, L, x, y, z, ub1);
   }
   const V *uin = n_ext > 0 ? ub1 : nullptr;
-  if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  if (!lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
   // start the classification's counters (every CTA has read the band count; the lists are
   // filled after the next barriers): the band count into the previous-band slot
   if (blockIdx.x == 0 && tid == 0) {
@@ -914,7 +914,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     }
     uin = uout;
     // (the first transport stage reads phi and its own cells' u~: no barrier before it)
-    if (it < n_ext - 1 && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
+    if (it < n_ext - 1 && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
   }
   // values around a cell (at pc) along axis a at offsets -3..+3, or mirrored; last: the
   // highest index wanted
@@ -986,7 +986,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     }
     // (the phases read their own cells' phi and leave p2, which the last stage's neighbours
     // read, as it is: no barrier between them)
-    if ((stage < 3 || n_re > 0) && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
+    if ((stage < 3 || n_re > 0) && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
   }
   // ---- reinitialisation
   for (int r = 0; r < n_re; ++r)
@@ -1039,7 +1039,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
         const LevelDev &L = beyond(k, x, y, z, ok);
         if (ok) reinit_cell<Q>(C, L, x, y, z, stage, prep);
       }
-      if ((stage < 3 || r < n_re - 1) && !lsf_barrier<MODE>(bar, target, C.err)) return leave();
+      if ((stage < 3 || r < n_re - 1) && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
     }
   // ---- phases (k_classify_phase without init): p1 (p2 below) back to phi, tags, flips
   for (int k = 0; k < kn; ++k) {
@@ -1079,7 +1079,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       list_flip<Q>(C, L, S, glevel, ld, fc - L.fine_off, x, y, z);
     }
   }
-  if (!lsf_barrier<MODE>(bar, target, C.err)) return leave();
+  if (!lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
   // ---- cut links (k_classify_links without full): the previous band, then the check list
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int *lst = C.band_list + (long long)glevel * C.band_cap, *chk = C.check_list + (long long)glevel * C.band_cap;
@@ -1537,7 +1537,7 @@ cudaError_t prepare_levelset_fused(int Q, LsfLimits *out) {
 }
 template <int Q>
 cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                       unsigned *bar) {
+                       unsigned *bar, long long limit) {
   cudaLaunchAttribute at[3];
   unsigned na = 0;
   if (P.coop) {
@@ -1567,14 +1567,14 @@ cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, i
   cfg.stream = L.stream;
   cfg.attrs = at;
   cfg.numAttrs = na;
-  if (P.coop) return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 1>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar);
-  return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 0>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar);
+  if (P.coop) return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 1>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
+  return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 0>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
 }
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                               unsigned *bar) {
-  if (Q == 9) return lsf_launch<9>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
-  if (Q == 19) return lsf_launch<19>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
-  return lsf_launch<27>(L, P, C, S, glevel, n_ext, n_re, nld, bar);
+                               unsigned *bar, long long limit) {
+  if (Q == 9) return lsf_launch<9>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
+  if (Q == 19) return lsf_launch<19>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
+  return lsf_launch<27>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
 }
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,
                               int refill) {

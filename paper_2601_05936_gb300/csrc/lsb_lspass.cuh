@@ -330,11 +330,13 @@ __device__ __forceinline__ void d_reinit_stage(const Ctx &C, BlockShape S, int g
   }
 }
 // ------------------------------------------------------------------ barriers between passes of a launch
-constexpr unsigned kLsfLimit = 1u << 23;  // polls of a grid barrier before it gives up (seconds)
-// MODE 0: the grid is one thread-block cluster; 1: a cooperative launch (bar[0] counts
-// arrivals; false: the wait gave up, ERR_TIMEOUT is set).
+// MODE 0: the grid is one thread-block cluster and the barrier is the hardware's, without a limit;
+// 1: a cooperative launch (bar[0] counts arrivals).  limit: reads of the count before the wait
+// gives up (the handle's wait limit; 0 gives up at once unless the CTA is alone).  false: it gave
+// up, ERR_TIMEOUT is set, and the CTA has to leave: it arrives at no later barrier, so no CTA gets
+// past the next one either.
 template <int MODE>
-__device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err) {
+__device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err, long long limit) {
   if (MODE == 0) {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     return true;
@@ -343,17 +345,18 @@ __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
-    gave_up = 0;
-    unsigned v, spins = 0;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    do {
+    bool there = gridDim.x == 1;
+    for (long long i = 0; !there && i < limit; ++i) {
+      unsigned v;
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if (++spins > kLsfLimit) {
-        gave_up = 1;
-        atomicOr(err, ERR_TIMEOUT);
-        break;
-      }
-    } while ((int)(v - target) < 0);
+      there = (int)(v - target) >= 0;
+    }
+    gave_up = !there;
+    if (!there) {
+      atomicOr(err, ERR_TIMEOUT);
+      __threadfence();  // the arrival, which no read has seen yet, before the count in lsf_leave
+    }
   }
   __syncthreads();
   return gave_up == 0;
@@ -363,6 +366,7 @@ __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int
 // clears both words for the next launch.
 __device__ __forceinline__ void lsf_leave(unsigned *bar) {
   if (threadIdx.x == 0 && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
+    __threadfence();
     bar[0] = 0;
     bar[1] = 0;
   }

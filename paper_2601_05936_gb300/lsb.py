@@ -263,7 +263,7 @@ class Grid:
         self._check(self.lib.lsb_set_objective(self.h, float(eps)))
 
     def set_wait_limit(self, spins):
-        """Iteration limit of the bounded device-side waits (~64 ns each; 0 gives up at once)."""
+        """Iteration limit of the device-wide barriers, forward and reverse (0 gives up at once)."""
         self._check(self.lib.lsb_set_wait_limit(self.h, int(spins)))
 
     def refine(self):
