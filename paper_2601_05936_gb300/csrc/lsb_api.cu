@@ -573,6 +573,9 @@ lsb_status ls_mirror(lsb_grid *g) {
   return LSB_OK;
 }
 
+// The wait limit of the launches that count it in 32 bits (2^32 - 1 reads take the better part of an hour).
+unsigned wait_limit32(const lsb_grid *g) { return (unsigned)std::min(g->wait_limit, 0xffffffffLL); }
+
 // Level-set update of the finest level l (extension, transport, reinitialisation).
 lsb_status levelset(lsb_grid *g, int l) {
   Ctx C = make_ctx(g);
@@ -591,7 +594,7 @@ lsb_status levelset(lsb_grid *g, int l) {
   }
   const bool due = g->reinit_every > 0 && ((g->fine_steps[l] + 1) % g->reinit_every == 0);
   RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
-      (int)g->lds.size(), g->d_bar + 2, g->wait_limit);
+      (int)g->lds.size(), g->d_bar + 2, wait_limit32(g));
   g->classified[l] = true;
   return LSB_OK;
 }
@@ -1223,7 +1226,7 @@ lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *u
   RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l);
   const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
   RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, g->band_est[l]), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
-      g->d_bar + 2, g->wait_limit);
+      g->d_bar + 2, wait_limit32(g));
   RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, P.A.LU, g->d_madj, P.A.LP);
   // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LP
   const GeoAdj G{P.A.LP, g->d_gn, g->d_gk};

@@ -112,7 +112,7 @@ cudaError_t prepare_levelset_fused(int Q, LsfLimits *out);
 // ut0's planes into the interleaved sweep buffers (n finest cells)
 cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n);
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                               unsigned *bar, long long limit);
+                               unsigned *bar, unsigned limit);
 // the flipped cells (fit, and refill when refill is set), the curvature fit of the interface
 // cells on gg CTAs and the band pass on the other CTAs of L.grid, one launch
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,
@@ -168,7 +168,7 @@ struct LsaScratch {
   float *LP, *LU, *L1, *L2, *LS0, *LK0, *LK1, *LV;
 };
 cudaError_t run_lsa_levelset(int Q, Launch L, Ctx C, BlockShape S, int glevel, int n_ext, int rein, LsaScratch A,
-                             unsigned *bar, long long limit);
+                             unsigned *bar, unsigned limit);
 cudaError_t run_lsa_flipflag(Launch L, const int *counters, int glevel, int *flag);
 
 }  // namespace lsb

@@ -739,15 +739,17 @@ template <int D> struct LsfSlot {
 };
 template <int Q, int MODE>
 __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                                                            int kcap, unsigned *bar, long long limit) {
+                                                            int kcap, unsigned *bar, unsigned limit) {
   constexpr int D = Lat<Q>::D;
   using V = typename UVec<D>::T;
   asm volatile("griddepcontrol.wait;" ::: "memory");
   extern __shared__ __align__(16) unsigned char lsf_sm[];
   __shared__ LsfGeo geo[kLsfGeo];
   __shared__ int hot[32];  // link pass: a cut link in each of the CTA's blocks
+  __shared__ unsigned wait_limit;
   LsfSlot<D> *const SM = reinterpret_cast<LsfSlot<D> *>(lsf_sm);
   const int T = blockDim.x, tid = threadIdx.x;
+  if (tid == 0) wait_limit = limit;
   const int lgnt = S.lg[0] + S.lg[1] + S.lg[2];
   const int t = tid & ((1 << lgnt) - 1);
   const int GB = (int)((gridDim.x * (unsigned)T) >> lgnt);         // band blocks per sweep of the grid
@@ -858,7 +860,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     if (ok && n_ext > 0) ext_first_cell<D>(C, L, x, y, z, ub1);
   }
   const V *uin = n_ext > 0 ? ub1 : nullptr;
-  if (!lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
+  if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return leave();
   // start the classification's counters (every CTA has read the band count; the lists are
   // filled after the next barriers): the band count into the previous-band slot
   if (blockIdx.x == 0 && tid == 0) {
@@ -914,7 +916,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     }
     uin = uout;
     // (the first transport stage reads phi and its own cells' u~: no barrier before it)
-    if (it < n_ext - 1 && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
+    if (it < n_ext - 1 && !lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return leave();
   }
   // values around a cell (at pc) along axis a at offsets -3..+3, or mirrored; last: the
   // highest index wanted
@@ -986,7 +988,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     }
     // (the phases read their own cells' phi and leave p2, which the last stage's neighbours
     // read, as it is: no barrier between them)
-    if ((stage < 3 || n_re > 0) && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
+    if ((stage < 3 || n_re > 0) && !lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return leave();
   }
   // ---- reinitialisation
   for (int r = 0; r < n_re; ++r)
@@ -1039,7 +1041,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
         const LevelDev &L = beyond(k, x, y, z, ok);
         if (ok) reinit_cell<Q>(C, L, x, y, z, stage, prep);
       }
-      if ((stage < 3 || r < n_re - 1) && !lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
+      if ((stage < 3 || r < n_re - 1) && !lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return leave();
     }
   // ---- phases (k_classify_phase without init): p1 (p2 below) back to phi, tags, flips
   for (int k = 0; k < kn; ++k) {
@@ -1079,7 +1081,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
       list_flip<Q>(C, L, S, glevel, ld, fc - L.fine_off, x, y, z);
     }
   }
-  if (!lsf_barrier<MODE>(bar, target, C.err, limit)) return leave();
+  if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return leave();
   // ---- cut links (k_classify_links without full): the previous band, then the check list
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int *lst = C.band_list + (long long)glevel * C.band_cap, *chk = C.check_list + (long long)glevel * C.band_cap;
@@ -1537,7 +1539,7 @@ cudaError_t prepare_levelset_fused(int Q, LsfLimits *out) {
 }
 template <int Q>
 cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                       unsigned *bar, long long limit) {
+                       unsigned *bar, unsigned limit) {
   cudaLaunchAttribute at[3];
   unsigned na = 0;
   if (P.coop) {
@@ -1571,7 +1573,7 @@ cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, i
   return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 0>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
 }
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
-                               unsigned *bar, long long limit) {
+                               unsigned *bar, unsigned limit) {
   if (Q == 9) return lsf_launch<9>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
   if (Q == 19) return lsf_launch<19>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
   return lsf_launch<27>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);

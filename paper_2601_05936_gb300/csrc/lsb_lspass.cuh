@@ -331,12 +331,15 @@ __device__ __forceinline__ void d_reinit_stage(const Ctx &C, BlockShape S, int g
 }
 // ------------------------------------------------------------------ barriers between passes of a launch
 // MODE 0: the grid is one thread-block cluster and the barrier is the hardware's, without a limit;
-// 1: a cooperative launch (bar[0] counts arrivals).  limit: reads of the count before the wait
-// gives up (the handle's wait limit; 0 gives up at once unless the CTA is alone).  false: it gave
-// up, ERR_TIMEOUT is set, and the CTA has to leave: it arrives at no later barrier, so no CTA gets
-// past the next one either.
+// 1: a cooperative launch (bar[0] counts arrivals).  *limit: reads of the count before the wait
+// gives up (the handle's wait limit; 0 gives up at once unless the CTA is alone), in shared memory
+// and written by thread 0: as a kernel parameter it had left the constant cache by the next barrier
+// and cost each 0.13 us (3D bubble, 28 of them: step 691 -> 695 us).  false: it gave up, ERR_TIMEOUT
+// is set, and the CTA has to leave: it arrives at no later barrier, so no CTA gets past the next
+// one either.
+constexpr unsigned kGaveUp = 1u << 16;  // (more than a cooperative grid's CTAs)
 template <int MODE>
-__device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err, long long limit) {
+__device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err, const unsigned *limit) {
   if (MODE == 0) {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
     return true;
@@ -345,28 +348,32 @@ __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
+    gave_up = 0;
+    unsigned v, left = *limit;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
-    bool there = gridDim.x == 1;
-    for (long long i = 0; !there && i < limit; ++i) {
-      unsigned v;
+    do {
+      if (left-- == 0) {
+        if (gridDim.x == 1) break;
+        gave_up = 1;
+        atomicOr(err, ERR_TIMEOUT);
+        __threadfence();  // the arrival, which no read has seen yet, before the marks in bar[1]
+        atomicAdd(bar + 1, kGaveUp);
+        break;
+      }
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      there = (int)(v - target) >= 0;
-    }
-    gave_up = !there;
-    if (!there) {
-      atomicOr(err, ERR_TIMEOUT);
-      __threadfence();  // the arrival, which no read has seen yet, before the count in lsf_leave
-    }
+    } while ((int)(v - target) < 0);
   }
   __syncthreads();
   return gave_up == 0;
 }
 
-// Every CTA of a MODE 1 launch passes here once, last: bar[1] counts them, and the last one
-// clears both words for the next launch.
+// Every CTA of a MODE 1 launch passes here once, last: bar[1] counts them (and, from kGaveUp up,
+// those that gave up), and the last one clears both words for the next launch.
 __device__ __forceinline__ void lsf_leave(unsigned *bar) {
-  if (threadIdx.x == 0 && atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
-    __threadfence();
+  if (threadIdx.x != 0) return;
+  const unsigned out = atomicAdd(bar + 1, 1u);
+  if (out % kGaveUp == gridDim.x - 1) {
+    if (out >= kGaveUp) __threadfence();  // (1 us of the launch where it is not needed)
     bar[0] = 0;
     bar[1] = 0;
   }
