@@ -288,10 +288,14 @@ lsb_status lsb_cell_updates(const lsb_grid *g, double *per_coarse_step, double *
  * out[1] band cells (band blocks x block cells), out[2] interface cells,
  * out[3] cut links, out[4] cells flipped at the last finest step (1..4: the
  * finest level of a case only, else 0), out[5] ghost-ring cells filled from
- * the coarser level, out[6] covered cells restricted from the finer level.
+ * the coarser level, out[6] covered cells restricted from the finer level;
+ * out[7 .. 10] the shape that the level-set update of the next step launches with
+ * (finest level of a case only, else 0): 0 one thread-block cluster or 1 a
+ * cooperative grid, its CTAs, its threads per CTA, and the band cells it holds in
+ * shared memory (the shape follows the band; it changes no result).
  * Host array of n <= LSB_NWORK values.  Synchronises.  Errors: LSB_EINVAL.
  */
-enum { LSB_NWORK = 7 };
+enum { LSB_NWORK = 11 };
 lsb_status lsb_work_counts(lsb_grid *g, int level, long long *out, int n);
 
 /* Velocity-set tables compiled into the library (Sec. 2.1, Fig. 1): c receives

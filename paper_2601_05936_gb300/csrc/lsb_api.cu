@@ -94,9 +94,12 @@ struct lsb_grid {
   int2 *d_linkcell = nullptr;
   uint8_t *d_linkdir = nullptr;
   long long link_list_off[MAXL] = {0, 0, 0, 0};
-  // pinned host words the synchronising calls read back into: the error word, then the
-  // observables of every case (allocated at the first use)
-  int *h_err = nullptr;
+  // pinned host words: the counters of every level and the error word, as they lie behind
+  // d_counters (read back by the synchronising calls and, between them, by follow_band), then
+  // the observables of every case
+  int *h_words = nullptr;
+  enum { WORDS_NONE, WORDS_ASKED, WORDS_HERE } words = WORDS_NONE;  // the band counts in h_words
+  int unseen_steps = 0;  // coarse steps since they were last asked for
   double *h_obs = nullptr;
   int *d_work = nullptr;  // per level: the collide-and-stream's block counters (next, finished)
   int *d_counters = nullptr, *d_err = nullptr, *d_band = nullptr, *d_check = nullptr;
@@ -104,7 +107,7 @@ struct lsb_grid {
   unsigned *d_bar = nullptr;  // grid barriers: of the persistent level-set kernel, of the one-launch update
   LsfLimits lsf_lim;
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
-  int band_est[MAXL] = {0, 0, 0, 0};  // band blocks when it was planned
+  int band_est[MAXL] = {0, 0, 0, 0};  // band blocks it was planned for
   long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
@@ -180,6 +183,7 @@ struct lsb_grid {
   int rec_moving = 0;
   int *d_recflip = nullptr;  // set when a recorded step flipped a cell
   float *d_lsa = nullptr;    // one allocation, carved by lsa_ptrs()
+  int lsa_band = 0;          // band blocks of the window
   size_t lsa_floats = 0;
   float *d_phisave = nullptr, *d_utsave = nullptr;
   double *d_grad = nullptr, *d_wobs = nullptr;
@@ -364,6 +368,10 @@ constexpr int EXPORT_CTAS = 152 * 8;  // resident at 256 threads: a cell a threa
 #ifndef LSB_GEO_CTAS
 #define LSB_GEO_CTAS 512
 #endif
+
+constexpr int NWORDS = MAXL * NCOUNT + 1;  // counters of every level, error word
+constexpr int kBandRoom = 16;    // a plan has room for 1 / kBandRoom more band blocks
+constexpr int kWordsEvery = 64;  // coarse steps between looks at the band without a synchronising call
 
 #define TRY(x)                   \
   do {                           \
@@ -599,18 +607,12 @@ lsb_status levelset(lsb_grid *g, int l) {
   return LSB_OK;
 }
 
-// Shape of the one-launch level-set update of level l from the band its classification
-// just listed (the launch is right for any band; the shape only sets its speed).  Up to two
-// cells per thread of a 16-CTA cluster of 1024 threads the cluster's barrier wins (0.6 -
-// 1.0 us a pass against 1.4 us of the grid's); beyond, a pass is bound by its loads and a
-// grid over all SMs takes over.
-lsb_status plan_levelset(lsb_grid *g, int l) {
-  int nb = 0;
-  CU(cudaMemcpyAsync(&nb, g->d_counters + l * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
-  CU(cudaStreamSynchronize(g->stream));
-  nb = std::max(1, std::min(nb, g->band_cap));
-  g->band_est[l] = nb;
-  nb += nb / 16;  // room for the band to grow until the next regrid
+// Shape of the one-launch level-set update for a band of nb blocks (the launch is right for
+// any band; the shape only sets its speed).  Up to two cells per thread of a 16-CTA cluster of
+// 1024 threads the cluster's barrier wins (0.6 - 1.0 us a pass against 1.4 us of the grid's);
+// beyond, a pass is bound by its loads and a grid over all SMs takes over.
+LsfPlan plan_levelset(const lsb_grid *g, int nb) {
+  nb += nb / kBandRoom;
   const int nt = g->nthreads, per = 1024 / nt;  // blocks of a full CTA
   const LsfLimits &M = g->lsf_lim;
   LsfPlan P;
@@ -629,7 +631,76 @@ lsb_status plan_levelset(lsb_grid *g, int l) {
     P.kcap = std::min(M.kmax, (nb + P.grid * each - 1) / (P.grid * each));
   }
   if ((int)g->lds.size() > M.max_ld) P.kcap = 0;
-  g->lsf[l] = P;
+  return P;
+}
+
+// The plan of level l for the band that its classification just listed.
+lsb_status plan_for_band(lsb_grid *g, int l) {
+  int nb = 0;
+  CU(cudaMemcpyAsync(&nb, g->d_counters + l * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  CU(cudaStreamSynchronize(g->stream));
+  g->band_est[l] = std::max(1, std::min(nb, g->band_cap));
+  g->lsf[l] = plan_levelset(g, g->band_est[l]);
+  return LSB_OK;
+}
+
+// Copy the device's words (the counters of every level, then the error word) into h_words.
+lsb_status read_words(lsb_grid *g) {
+  CU(cudaMemcpyAsync(g->h_words, g->d_counters, sizeof(int) * NWORDS, cudaMemcpyDeviceToHost, g->stream));
+  return LSB_OK;
+}
+
+void drop_graphs(lsb_grid *g);
+
+// Keeps the plans to the band there is, where no regrid does (one level, regrid_every = 0, a
+// regrid that changes no block).  A 1024 x 128 flow whose interface is sheared from 128 to 460
+// band blocks: 128 us a step on the plan of its creation, 67 - 71 when followed (the launch per
+// pass that knew no plan: 97), and 30.5 against 17 us once the interface was gone (25).
+// Called before the launches of a coarse step.  The band counts come with every synchronising
+// call, and on stretches without one by a copy every kWordsEvery steps that nothing waits for
+// (2 us): the words are set to -1 before it and looked at again until they changed (how far the
+// plan then lags is how far the launches run ahead of the GPU).  Captured graphs are dropped
+// only when a plan differs, once what runs has ended; nothing is done while the caller captures
+// the stream.
+lsb_status follow_band(lsb_grid *g) {
+  if (g->driver != 0) return LSB_OK;
+  auto word = [&](int l) -> volatile int & { return g->h_words[l * NCOUNT + 3]; };
+  auto capturing = [&]() {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaError_t e = cudaStreamIsCapturing(g->stream, &st);
+    if (e != cudaSuccess) cudaGetLastError();
+    return e != cudaSuccess || st != cudaStreamCaptureStatusNone;
+  };
+  if (g->words == lsb_grid::WORDS_ASKED) {
+    bool here = true;
+    for (int l = 0; l < g->Lmax; ++l) here = here && (!has_finest(g, l) || word(l) >= 0);
+    if (here) g->words = lsb_grid::WORDS_HERE;
+  }
+  if (g->words == lsb_grid::WORDS_HERE) {
+    g->words = lsb_grid::WORDS_NONE;
+    bool changed = false;
+    for (int l = 0; l < g->Lmax; ++l) {
+      if (!has_finest(g, l)) continue;
+      const int nb = std::max(1, std::min((int)word(l), g->band_cap)), est = g->band_est[l];
+      if (nb <= est + est / kBandRoom && 2 * nb >= est) continue;
+      const LsfPlan P = plan_levelset(g, nb), &O = g->lsf[l];
+      const bool same = P.coop == O.coop && P.grid == O.grid && P.threads == O.threads && P.kcap == O.kcap;
+      if (!same && !changed) {
+        if (capturing()) return LSB_OK;
+        CU(cudaStreamSynchronize(g->stream));
+        drop_graphs(g);
+        changed = true;
+      }
+      g->band_est[l] = nb;
+      g->lsf[l] = P;
+    }
+  }
+  if (g->words == lsb_grid::WORDS_NONE && g->unseen_steps >= kWordsEvery && !capturing()) {
+    for (int l = 0; l < g->Lmax; ++l) word(l) = -1;
+    TRY(read_words(g));
+    g->words = lsb_grid::WORDS_ASKED;
+    g->unseen_steps = 0;
+  }
   return LSB_OK;
 }
 
@@ -820,14 +891,14 @@ lsb_status advance(lsb_grid *g, int l) {
 }
 
 lsb_status regrid(lsb_grid *g, bool initial);
-// Pinned read-back words (one allocation: the error word, then room for the observables).
+// Pinned read-back words (one allocation: the device's words, then room for the observables).
 lsb_status pin_host(lsb_grid *g) {
-  if (g->h_err) return LSB_OK;
-  const size_t nobs = (size_t)(4 + 2 * g->D) * g->ncase;
+  if (g->h_words) return LSB_OK;
+  const size_t nobs = (size_t)(4 + 2 * g->D) * g->ncase, words = (sizeof(int) * NWORDS + 15) / 16 * 16;
   void *p = nullptr;
-  CU(cudaMallocHost(&p, 16 + sizeof(double) * nobs));
-  g->h_err = static_cast<int *>(p);
-  g->h_obs = reinterpret_cast<double *>(static_cast<char *>(p) + 16);
+  CU(cudaMallocHost(&p, words + sizeof(double) * nobs));
+  g->h_words = static_cast<int *>(p);
+  g->h_obs = reinterpret_cast<double *>(static_cast<char *>(p) + words);
   return LSB_OK;
 }
 
@@ -1225,7 +1296,7 @@ lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *u
   Gm.kappa = P.KP;
   RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l);
   const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
-  RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, g->band_est[l]), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
+  RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, std::min(g->lsa_band, g->band_cap)), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
       g->d_bar + 2, wait_limit32(g));
   RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, P.A.LU, g->d_madj, P.A.LP);
   // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LP
@@ -1550,8 +1621,8 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
     ALLOC(g->d_linkcell, 8 * g->link_cap * nl);
     ALLOC(g->d_linkdir, g->link_cap * nl);
   }
-  ALLOC(g->d_counters, sizeof(int) * MAXL * NCOUNT);
-  ALLOC(g->d_err, sizeof(int));
+  ALLOC(g->d_counters, sizeof(int) * NWORDS);
+  g->d_err = g->d_counters + MAXL * NCOUNT;
   ALLOC(g->d_work, sizeof(int) * 2 * MAXL);
   s = pin_host(g);
   if (s) { g_create_error = g->err; lsb_destroy(g); return s; }
@@ -1589,10 +1660,9 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
       cuerr(cudaMemcpy(g->d_blk_info, binfo.data(), sizeof(int4) * binfo.size(), cudaMemcpyHostToDevice), "blk_info") ||
       cuerr(cudaMemset(g->d_tag, 0, g->ncell_total), "tag") ||
       cuerr(cudaMemset(g->d_bflag, 0, g->nblock_total), "bflag") ||
-      cuerr(cudaMemset(g->d_err, 0, sizeof(int)), "err") ||
       cuerr(cudaMemset(g->d_work, 0, sizeof(int) * 2 * MAXL), "work") ||
       cuerr(cudaMemset(g->d_bar, 0, 4 * sizeof(unsigned)), "barrier") ||
-      cuerr(cudaMemset(g->d_counters, 0, sizeof(int) * MAXL * NCOUNT), "counters") ||
+      cuerr(cudaMemset(g->d_counters, 0, sizeof(int) * NWORDS), "counters") ||
       cuerr(cudaMemset(g->d_cmask, 0, 4 * nf), "cmask") ||
       cuerr(cudaMemset(g->d_nvec, 0, 4 * D * nf), "nvec") ||
       cuerr(cudaMemset(g->d_kappa, 0, 4 * nf), "kappa") ||
@@ -1663,7 +1733,9 @@ lsb_status lsb_step(lsb_grid *g, int n) {
     for (int k = 0; k < n; ++k) {
       if (g->rec_steps % g->rec_every == 0 && (size_t)(g->rec_steps / g->rec_every) == g->rec_ckpt.size())
         TRY(rec_checkpoint(g));
+      TRY(follow_band(g));
       TRY(advance(g, 0));
+      g->unseen_steps++;
       if (g->rec_moving)
         TRY(launched(g, run_lsa_flipflag(LN(g, 1, 32), g->d_counters, g->Lmax - 1, g->d_recflip)));
       g->updates_done += updates_per_step(g);
@@ -1678,11 +1750,14 @@ lsb_status lsb_step(lsb_grid *g, int n) {
     const bool regrid_on = g->regrid_every > 0 && g->Lmax > 1;
     const bool regrid_soon =
         regrid_on && ((g->coarse_steps + 1) % g->regrid_every == 0 || (g->coarse_steps + 2) % g->regrid_every == 0);
+    TRY(follow_band(g));
     if (n - k >= 2 && !regrid_soon && graphs_usable(g)) {
       TRY(replay_steps(g, 2));
       k += 2;
+      g->unseen_steps += 2;
       continue;
     }
+    g->unseen_steps++;
     if (graphs_usable(g)) {  // one step (a regrid, if due, follows it as after an eager step)
       TRY(replay_steps(g, 1));
     } else {
@@ -1740,10 +1815,12 @@ lsb_status lsb_refine(lsb_grid *g) {
 lsb_status lsb_sync(lsb_grid *g) {
   if (!g) return LSB_EINVAL;
   TRY(pin_host(g));
-  // the error word comes back with the stream's work: one wait for both
-  CU(cudaMemcpyAsync(g->h_err, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
+  // the words come back with the stream's work: one wait for both
+  TRY(read_words(g));
   CU(cudaStreamSynchronize(g->stream));
-  const int e = *g->h_err;
+  g->words = lsb_grid::WORDS_HERE;
+  g->unseen_steps = 0;
+  const int e = g->h_words[MAXL * NCOUNT];
   g->latched |= e;
   // first the timeout: the lists of an update that gave up are half made, and may overflow after it
   if (g->latched & ERR_TIMEOUT) return fail(g, LSB_ETIMEOUT, "a bounded device-side wait gave up");
@@ -2004,6 +2081,11 @@ lsb_status lsb_work_counts(lsb_grid *g, int level, long long *out, int n) {
     v[2] = std::min<long long>(h[1], g->list_cap);
     v[3] = std::min<long long>(h[0], g->link_cap);
     v[4] = std::min<long long>(h[2], g->list_cap);
+    const LsfPlan &P = g->lsf[level];
+    v[7] = P.coop;
+    v[8] = P.grid;
+    v[9] = P.threads;
+    v[10] = (long long)P.grid * P.threads * P.kcap;
   }
   for (int k = 0; k < n && k < LSB_NWORK; ++k) out[k] = v[k];
   return LSB_OK;
@@ -2084,6 +2166,8 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
     CU(cudaStreamSynchronize(g->stream));
     CU(cudaMemcpy(&flip, g->d_recflip, sizeof(int), cudaMemcpyDeviceToHost));
     if (flip) return fail(g, LSB_ESTATE, "a cell changed phase during the recorded window");
+    // the reverse launch's grid: a CTA per band block of the window (no flips: the same all through)
+    CU(cudaMemcpy(&g->lsa_band, g->d_counters + (g->Lmax - 1) * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost));
   }
   TRY(adj_buffers(g, (int)std::min<long long>(every, std::max<long long>(T, 1))));
   const size_t sf = state_floats(g), sb = sizeof(float) * sf, sl = slot_floats(g);
@@ -2301,7 +2385,7 @@ void lsb_destroy(lsb_grid *g) {
     cudaEventDestroy(r.b);
   }
   for (cudaEvent_t e : g->ev_pool) cudaEventDestroy(e);
-  if (g->h_err) cudaFreeHost(g->h_err);
+  if (g->h_words) cudaFreeHost(g->h_words);
   delete g;
 }
 
@@ -2508,8 +2592,10 @@ lsb_status regrid(lsb_grid *g, bool initial) {
   CU(cudaMemsetAsync(g->d_bflag, 0, g->nblock_total, g->stream));
   for (int l = 0; l < g->Lmax; ++l) {
     TRY(classify(g, l, 1));
-    if (has_finest(g, l)) TRY(plan_levelset(g, l));
+    if (has_finest(g, l)) TRY(plan_for_band(g, l));
   }
+  g->words = lsb_grid::WORDS_NONE;
+  g->unseen_steps = 0;
   return LSB_OK;
 }
 

@@ -343,6 +343,12 @@ class Grid:
         self._check(self.lib.lsb_work_counts(self.h, int(level), out, len(names)))
         return dict(zip(names, (int(v) for v in out)))
 
+    def levelset_launch(self, level):
+        """Shape of the next level-set launch of finest level ``level`` (see lsb_work_counts)."""
+        out = (ctypes.c_longlong * 11)()
+        self._check(self.lib.lsb_work_counts(self.h, int(level), out, 11))
+        return dict(zip(("form", "ctas", "threads", "cells"), (int(v) for v in out[7:])))
+
     def kernel_launches(self):
         return int(self.lib.lsb_kernel_launches(self.h))
 
