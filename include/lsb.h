@@ -165,7 +165,8 @@ lsb_status lsb_use_graphs(lsb_grid *g, int enable);
  * classification's phase and cut-link passes in one launch per finest step, on
  * stage arrays that need no band lookups (one thread-block cluster for a small
  * band, a cooperative launch with device-wide barriers otherwise, bounded by
- * lsb_set_wait_limit as those of mode 1).
+ * lsb_set_wait_limit as those of mode 1; a launch per pass for bands of millions of
+ * cells).
  * mode 1: one persistent cooperative launch per finest step that runs the
  * level-set passes over the band work list of all cases with a lookup per
  * stencil point, and a device-wide barrier between passes; the barrier's wait
@@ -290,9 +291,10 @@ lsb_status lsb_cell_updates(const lsb_grid *g, double *per_coarse_step, double *
  * finest level of a case only, else 0), out[5] ghost-ring cells filled from
  * the coarser level, out[6] covered cells restricted from the finer level;
  * out[7 .. 10] the shape that the level-set update of the next step launches with
- * (finest level of a case only, else 0): 0 one thread-block cluster or 1 a
- * cooperative grid, its CTAs, its threads per CTA, and the band cells it holds in
- * shared memory (the shape follows the band; it changes no result).
+ * (finest level of a case only, else 0): 0 one thread-block cluster, 1 a
+ * cooperative grid or 2 a launch per pass (very large bands), its CTAs, its threads
+ * per CTA, and the band cells it holds in shared memory (the shape follows the
+ * band; it changes no result).
  * Host array of n <= LSB_NWORK values.  Synchronises.  Errors: LSB_EINVAL.
  */
 enum { LSB_NWORK = 11 };

@@ -370,6 +370,14 @@ constexpr int EXPORT_CTAS = 152 * 8;  // resident at 256 threads: a cell a threa
 #endif
 
 constexpr int NWORDS = MAXL * NCOUNT + 1;  // counters of every level, error word
+// Band cells, in multiples of the one-launch update's slots (3D: 778 k, 2D: 1.4 M), from which a
+// launch per pass wins.  us a step with one launch / a launch per pass:
+//   3D   1.37 M cells (two levels) 1217 / 1305, 2.36 M 1062 / 1052, 4.06 M 1902 / 1788, 16 M 7418 / 6499
+//   2D   1.97 M                     444 /  464, 3.93 M  950 /  924, 7.86 M 2120 / 1833
+#ifndef LSB_PASSES_FROM
+#define LSB_PASSES_FROM 2.5
+#endif
+constexpr double kPassesFrom = LSB_PASSES_FROM;
 constexpr int kBandRoom = 16;    // a plan has room for 1 / kBandRoom more band blocks
 constexpr int kWordsEvery = 64;  // coarse steps between looks at the band without a synchronising call
 
@@ -601,6 +609,20 @@ lsb_status levelset(lsb_grid *g, int l) {
     return LSB_OK;
   }
   const bool due = g->reinit_every > 0 && ((g->fine_steps[l] + 1) % g->reinit_every == 0);
+  if (g->lsf[l].form == LSF_PASSES) {
+    const int n_re = due ? g->n_reinit : 0;
+    const void *uin = nullptr;
+    for (int it = 0; it < g->n_ext; ++it) {
+      void *uout = g->d_ut[1 + (it & 1)];
+      RUN(13, 0, nb, nt, run_ext_pass, Q, LN(g, nb, nt), C, S, l, uin, uout);
+      uin = uout;
+    }
+    for (int st = 1; st <= 3; ++st) RUN(14, 0, nb, nt, run_adv_pass, Q, LN(g, nb, nt), C, S, l, st, uin);
+    for (int r = 0; r < n_re; ++r)
+      for (int st = 1; st <= 3; ++st)
+        RUN(16, 0, nb, nt, run_reinit_pass, Q, LN(g, nb, nt), C, S, l, st, r == 0 && st == 1 ? 1 : 0);
+    return LSB_OK;
+  }
   RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
       (int)g->lds.size(), g->d_bar + 2, wait_limit32(g));
   g->classified[l] = true;
@@ -610,27 +632,36 @@ lsb_status levelset(lsb_grid *g, int l) {
 // Shape of the one-launch level-set update for a band of nb blocks (the launch is right for
 // any band; the shape only sets its speed).  Up to two cells per thread of a 16-CTA cluster of
 // 1024 threads the cluster's barrier wins (0.6 - 1.0 us a pass against 1.4 us of the grid's);
-// beyond, a pass is bound by its loads and a grid over all SMs takes over.
+// beyond, a pass is bound by its loads and a grid over all SMs takes over; with most of the band
+// beyond that grid's slots, or more level descriptors than a slot can name, the passes are
+// launches of their own.
 LsfPlan plan_levelset(const lsb_grid *g, int nb) {
   nb += nb / kBandRoom;
   const int nt = g->nthreads, per = 1024 / nt;  // blocks of a full CTA
   const LsfLimits &M = g->lsf_lim;
   LsfPlan P;
+  // cells in the shared memory of all CTAs (with more level descriptors than a slot can name, none)
+  const double slots = (int)g->lds.size() > M.max_ld ? 0.0 : 1024.0 * M.kmax * std::max(M.grid, M.cluster);
+  if ((double)nb * nt > kPassesFrom * slots) {
+    P.form = LSF_PASSES;
+    P.grid = std::min(g->band_cap, 152 * 16);
+    P.threads = nt;
+    P.kcap = 0;
+    return P;
+  }
   if (nb <= M.cluster * per * 2 || M.grid == 0) {
-    P.coop = 0;
     P.grid = 1;
     while (P.grid < M.cluster && P.grid < nb) P.grid *= 2;
     const int each = (nb + P.grid - 1) / P.grid;  // blocks per CTA
     P.threads = nt * std::min(per, each);
     P.kcap = std::min(M.kmax, (each + per - 1) / per);
   } else {
-    P.coop = 1;
+    P.form = LSF_GRID;
     const int each = std::min(per, (nb + M.grid - 1) / M.grid);
     P.threads = nt * each;
     P.grid = std::min(M.grid, (nb + each - 1) / each);
     P.kcap = std::min(M.kmax, (nb + P.grid * each - 1) / (P.grid * each));
   }
-  if ((int)g->lds.size() > M.max_ld) P.kcap = 0;
   return P;
 }
 
@@ -684,7 +715,7 @@ lsb_status follow_band(lsb_grid *g) {
       const int nb = std::max(1, std::min((int)word(l), g->band_cap)), est = g->band_est[l];
       if (nb <= est + est / kBandRoom && 2 * nb >= est) continue;
       const LsfPlan P = plan_levelset(g, nb), &O = g->lsf[l];
-      const bool same = P.coop == O.coop && P.grid == O.grid && P.threads == O.threads && P.kcap == O.kcap;
+      const bool same = P.form == O.form && P.grid == O.grid && P.threads == O.threads && P.kcap == O.kcap;
       if (!same && !changed) {
         if (capturing()) return LSB_OK;
         CU(cudaStreamSynchronize(g->stream));
@@ -2082,7 +2113,7 @@ lsb_status lsb_work_counts(lsb_grid *g, int level, long long *out, int n) {
     v[3] = std::min<long long>(h[0], g->link_cap);
     v[4] = std::min<long long>(h[2], g->list_cap);
     const LsfPlan &P = g->lsf[level];
-    v[7] = P.coop;
+    v[7] = P.form;
     v[8] = P.grid;
     v[9] = P.threads;
     v[10] = (long long)P.grid * P.threads * P.kcap;

@@ -105,14 +105,21 @@ cudaError_t run_geometry(int D, Launch L, Ctx C, int glevel);
 struct LsfLimits {
   int kmax = 0, grid = 0, cluster = 0, max_ld = 0;
 };
+enum { LSF_CLUSTER, LSF_GRID, LSF_PASSES };  // one cluster; a cooperative grid; a launch per pass
 struct LsfPlan {
-  int coop = 0, grid = 1, threads = 0, kcap = 1;
+  int form = LSF_CLUSTER, grid = 1, threads = 0, kcap = 1;
 };
 cudaError_t prepare_levelset_fused(int Q, LsfLimits *out);
 // ut0's planes into the interleaved sweep buffers (n finest cells)
 cudaError_t run_ut_pack(int D, Launch L, const float *ut0, float *ut1, float *ut2, long long n);
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
                                unsigned *bar, unsigned limit);
+// The passes of the same update as launches of their own (LSF_PASSES): an extension sweep from
+// uin into uout (nullptr: the first sweep, from ut0, which stores the plan), a transport stage
+// from the last sweep's buffer (nullptr: no sweeps), a reinitialisation stage.
+cudaError_t run_ext_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, const void *uin, void *uout);
+cudaError_t run_adv_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, const void *ufin);
+cudaError_t run_reinit_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, int prep);
 // the flipped cells (fit, and refill when refill is set), the curvature fit of the interface
 // cells on gg CTAs and the band pass on the other CTAs of L.grid, one launch
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,

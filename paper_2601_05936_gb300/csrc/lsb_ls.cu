@@ -411,8 +411,8 @@ __global__ void k_geometry(Ctx C, int glevel) {
 
 // seven values of the stage array along axis a at offsets -3..+3 (clamped or
 // wrapped at the box faces like gather7)
-__device__ __forceinline__ void gather7m(const LevelDev &L, const float *__restrict__ pinL, int x, int y, int z,
-                                         unsigned c, int a, float v[7]) {
+__device__ __forceinline__ void gather7m(const LevelDev &L, const float *pinL, int x, int y, int z, unsigned c, int a,
+                                         float v[7]) {
   const int crd = a == 0 ? x : (a == 1 ? y : z);
   if (crd >= 3 && crd + 3 < L.n[a]) {
     const int str = a == 0 ? 1 : (a == 1 ? L.p[0] : L.p[0] * L.p[1]);
@@ -1142,6 +1142,42 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
   leave();
 }
 
+// ------------------------------------------------------------------ a launch per pass
+// One pass of the update over the band list, for bands so large that most cells lie beyond the
+// slots of the launch above: there every pass loads a cell's descriptor and plan again on 1024
+// threads per SM, here on 1536, and the launches and their chains (~4 us each, 14 of them) weigh
+// little.  A layer of 16 M band cells (1024 x 1024 x 64): 7418 -> 6499 us a step.  The
+// reinitialisation is built for two CTAs of 512 threads per SM: with three (its stages 873
+// instead of 934 us there) the compiler contracts its arithmetic otherwise, an ulp in one of 500
+// cells, and the shape of the launch changes no result.  The counters are started by the
+// classification (no pass here touches them).
+enum { LS_EXT_FIRST, LS_EXT_SWEEP, LS_ADVECT, LS_REINIT };
+template <int Q, int PASS>
+__global__ void __launch_bounds__(512, PASS == LS_REINIT ? 2 : 3) k_levelset_pass(Ctx C, BlockShape S, int glevel, int stage, int prep,
+                                                          const void *uin_, void *uout_) {
+  LSB_GRID_WAIT();
+  constexpr int D = Lat<Q>::D;
+  using V = typename UVec<D>::T;
+  const V *uin = static_cast<const V *>(uin_);
+  V *uout = static_cast<V *>(uout_);
+  const int nl = min(C.counters[glevel * NCOUNT + 3], C.band_cap);
+  // the next entry of the band list is loaded while this one is processed
+  const int4 *info = C.band_info + (long long)glevel * C.band_cap;
+  int4 next = (int)blockIdx.x < nl ? __ldg(info + blockIdx.x) : make_int4(0, 0, 0, 0);
+  for (int w = blockIdx.x; w < nl; w += gridDim.x) {
+    const int4 bi = next;
+    if (w + (int)gridDim.x < nl) next = __ldg(info + w + gridDim.x);
+    int x, y, z;
+    const LevelDev &L = band_cell_at(C, S, bi, threadIdx.x, x, y, z);
+    if (!L.ls_active || x >= L.n[0] || y >= L.n[1] || z >= L.n[2]) continue;
+    if constexpr (PASS == LS_EXT_FIRST) ext_first_cell<D>(C, L, x, y, z, uout);
+    else if constexpr (PASS == LS_EXT_SWEEP) ext_sweep_cell<D>(C, L, x, y, z, uin, uout);
+    else if constexpr (PASS == LS_ADVECT)
+      adv_cell<D>(C, L, x, y, z, stage, uin, reinterpret_cast<V *>(C.ut1), reinterpret_cast<V *>(C.ut2));
+    else reinit_cell<Q>(C, L, x, y, z, stage, prep);
+  }
+}
+
 // Both sweep buffers from ut0 at every finest cell (their state between updates).
 template <int D>
 __global__ void k_ut_pack(const float *__restrict__ ut0, typename UVec<D>::T *ub1, typename UVec<D>::T *ub2,
@@ -1542,7 +1578,7 @@ cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, i
                        unsigned *bar, unsigned limit) {
   cudaLaunchAttribute at[3];
   unsigned na = 0;
-  if (P.coop) {
+  if (P.form == LSF_GRID) {
     at[na].id = cudaLaunchAttributeCooperative;
     at[na++].val.cooperative = 1;
   } else {
@@ -1554,7 +1590,7 @@ cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, i
   // a cooperative launch is no programmatic dependent: launched early it loses the guarantee
   // that its CTAs become resident together (steps of 1 to 80 ms seen beside a side stream's
   // collide, 0.77 without)
-  if (L.pdl && !P.coop) {
+  if (L.pdl && P.form != LSF_GRID) {
     at[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at[na++].val.programmaticStreamSerializationAllowed = 1;
   }
@@ -1569,7 +1605,7 @@ cudaError_t lsf_launch(const Launch &L, const LsfPlan &P, Ctx C, BlockShape S, i
   cfg.stream = L.stream;
   cfg.attrs = at;
   cfg.numAttrs = na;
-  if (P.coop) return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 1>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
+  if (P.form == LSF_GRID) return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 1>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
   return cudaLaunchKernelEx(&cfg, k_levelset_fused<Q, 0>, C, S, glevel, n_ext, n_re, nld, P.kcap, bar, limit);
 }
 cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, int glevel, int n_ext, int n_re, int nld,
@@ -1577,6 +1613,24 @@ cudaError_t run_levelset_fused(int Q, Launch L, LsfPlan P, Ctx C, BlockShape S, 
   if (Q == 9) return lsf_launch<9>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
   if (Q == 19) return lsf_launch<19>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
   return lsf_launch<27>(L, P, C, S, glevel, n_ext, n_re, nld, bar, limit);
+}
+template <int PASS>
+cudaError_t pass_launch(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, int prep, const void *uin,
+                        void *uout) {
+  if (Q == 9) launcher(k_levelset_pass<9, PASS>, L, 0)(C, S, glevel, stage, prep, uin, uout);
+  else if (Q == 19) launcher(k_levelset_pass<19, PASS>, L, 0)(C, S, glevel, stage, prep, uin, uout);
+  else launcher(k_levelset_pass<27, PASS>, L, 0)(C, S, glevel, stage, prep, uin, uout);
+  return cudaGetLastError();
+}
+cudaError_t run_ext_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, const void *uin, void *uout) {
+  return uin ? pass_launch<LS_EXT_SWEEP>(Q, L, C, S, glevel, 0, 0, uin, uout)
+             : pass_launch<LS_EXT_FIRST>(Q, L, C, S, glevel, 0, 0, uin, uout);
+}
+cudaError_t run_adv_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, const void *ufin) {
+  return pass_launch<LS_ADVECT>(Q, L, C, S, glevel, stage, 0, ufin, nullptr);
+}
+cudaError_t run_reinit_pass(int Q, Launch L, Ctx C, BlockShape S, int glevel, int stage, int prep) {
+  return pass_launch<LS_REINIT>(Q, L, C, S, glevel, stage, prep, nullptr, nullptr);
 }
 cudaError_t run_post_classify(int Q, int st, Launch L, Ctx C, const int *list, int n, int glevel, int gg,
                               int refill) {
