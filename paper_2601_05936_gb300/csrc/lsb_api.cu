@@ -84,16 +84,15 @@ struct lsb_grid {
   int8_t *d_bstat = nullptr, *d_bstat_old = nullptr;
   uint8_t *d_bflag = nullptr, *d_tag = nullptr, *d_frozen = nullptr;
   void *d_buf[2] = {nullptr, nullptr};
-  float *d_phi = nullptr, *d_p1 = nullptr, *d_p2 = nullptr, *d_s0 = nullptr;
+  float *d_phi = nullptr, *d_p1 = nullptr, *d_p2 = nullptr, *d_s0 = nullptr;  // (p1, p2, s0: one allocation)
   float *d_ut[3] = {nullptr, nullptr, nullptr};
-  float *d_plan_v = nullptr;
-  uint8_t *d_plan_f = nullptr;
   uint32_t *d_cmask = nullptr;
   int *d_cbase = nullptr;
   float *d_macro = nullptr, *d_nvec = nullptr, *d_kappa = nullptr, *d_linkbuf = nullptr;
   int2 *d_linkcell = nullptr;
   uint8_t *d_linkdir = nullptr;
   long long link_list_off[MAXL] = {0, 0, 0, 0};
+  int list_l0 = 0;  // first level at which a case ends: the lists' memory starts with its region
   // pinned host words: the counters of every level and the error word, as they lie behind
   // d_counters (read back by the synchronising calls and, between them, by follow_band), then
   // the observables of every case
@@ -258,8 +257,8 @@ Ctx make_ctx(lsb_grid *g) {
   C.ut0 = g->d_ut[0];
   C.ut1 = g->d_ut[1];
   C.ut2 = g->d_ut[2];
-  C.plan_v = g->d_plan_v;
-  C.plan_f = g->d_plan_f;
+  C.plan_v = g->d_p1;
+  C.plan_f = g->d_frozen;
   C.cmask = g->d_cmask;
   C.cbase = g->d_cbase;
   C.macro = g->d_macro;
@@ -272,11 +271,15 @@ Ctx make_ctx(lsb_grid *g) {
   C.link_dir = g->d_linkdir;
   for (int l = 0; l < MAXL; ++l) C.link_list_off[l] = g->link_list_off[l];
   C.counters = g->d_counters;
-  C.iface_list = g->d_iface;
-  C.flip_list = g->d_flip;
-  C.band_list = g->d_band;
-  C.check_list = g->d_check;
-  C.band_info = g->d_band_info;
+  // (the kernels count regions from level 0)
+  auto from0 = [&](auto *p, long long cap) {
+    return reinterpret_cast<decltype(p)>(reinterpret_cast<uintptr_t>(p) - (size_t)(g->list_l0 * cap) * sizeof *p);
+  };
+  C.iface_list = from0(g->d_iface, g->list_cap);
+  C.flip_list = from0(g->d_flip, g->list_cap);
+  C.band_list = from0(g->d_band, g->band_cap);
+  C.check_list = from0(g->d_check, g->band_cap);
+  C.band_info = from0(g->d_band_info, g->band_cap);
   C.list_cap = g->list_cap;
   C.band_cap = g->band_cap;
   C.err = g->d_err;
@@ -1625,33 +1628,37 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
   ALLOC(g->d_buf[0], fsz * Q * g->ncell_total);
   ALLOC(g->d_buf[1], fsz * Q * g->ncell_total);
   ALLOC(g->d_phi, 4 * nf);
-  ALLOC(g->d_p1, 4 * nf);
-  ALLOC(g->d_p2, 4 * nf);
-  ALLOC(g->d_s0, 4 * nf);
+  ALLOC(g->d_p1, 3 * 4 * nf);
+  g->d_p2 = g->d_p1 + nf;
+  g->d_s0 = g->d_p2 + nf;
   ALLOC(g->d_frozen, nf);
   ALLOC(g->d_ut[0], 4 * D * nf);
   for (int k = 1; k < 3; ++k) ALLOC(g->d_ut[k], (D == 2 ? 8 : 16) * nf);  // sweep buffers: a vector per cell
-  ALLOC(g->d_plan_v, 4 * D * nf);
-  ALLOC(g->d_plan_f, nf);
   ALLOC(g->d_cmask, 4 * nf);
   ALLOC(g->d_cbase, 4 * nf);
   ALLOC(g->d_macro, 4 * (size_t)MREC * nf);
   ALLOC(g->d_nvec, 4 * D * nf);
   ALLOC(g->d_kappa, 4 * nf);
   ALLOC(g->d_linkbuf, 8 * g->link_cap);
+  int l1 = 0;  // the levels [list_l0, l1) have lists
   {
     // the link list lives from one classification to the next step's bounce-back, so
     // every finest global level keeps its own region (the link buffer is shared)
     long long nl = 0;
+    g->list_l0 = MAXL;
     for (int l = 0; l < MAXL; ++l) {
       g->link_list_off[l] = nl * g->link_cap;
       bool fin = false;
       for (int c = 0; c < n_cases; ++c) fin = fin || (g->cases[c].L - 1 == l);
-      if (fin) ++nl;
+      if (!fin) continue;
+      ++nl;
+      l1 = l + 1;
+      g->list_l0 = std::min(g->list_l0, l);
     }
     ALLOC(g->d_linkcell, 8 * g->link_cap * nl);
     ALLOC(g->d_linkdir, g->link_cap * nl);
   }
+  const size_t nlist = (size_t)(l1 - g->list_l0);
   ALLOC(g->d_counters, sizeof(int) * NWORDS);
   g->d_err = g->d_counters + MAXL * NCOUNT;
   ALLOC(g->d_work, sizeof(int) * 2 * MAXL);
@@ -1663,11 +1670,11 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
     else cudaGetLastError();
   }
   ALLOC(g->d_bar, 4 * sizeof(unsigned));
-  ALLOC(g->d_iface, sizeof(int2) * MAXL * g->list_cap);
-  ALLOC(g->d_flip, sizeof(int2) * MAXL * g->list_cap);
-  ALLOC(g->d_band, sizeof(int) * MAXL * (size_t)std::max(1, g->band_cap));
-  ALLOC(g->d_check, sizeof(int) * MAXL * (size_t)std::max(1, g->band_cap));
-  ALLOC(g->d_band_info, sizeof(int4) * MAXL * (size_t)std::max(1, g->band_cap));
+  ALLOC(g->d_iface, sizeof(int2) * nlist * g->list_cap);
+  ALLOC(g->d_flip, sizeof(int2) * nlist * g->list_cap);
+  ALLOC(g->d_band, sizeof(int) * nlist * (size_t)std::max(1, g->band_cap));
+  ALLOC(g->d_check, sizeof(int) * nlist * (size_t)std::max(1, g->band_cap));
+  ALLOC(g->d_band_info, sizeof(int4) * nlist * (size_t)std::max(1, g->band_cap));
   ALLOC(g->d_obs, sizeof(double) * n_cases * 16);
   ALLOC(g->d_sens, sizeof(float) * g->nblock_total);
 #undef ALLOC

@@ -189,9 +189,14 @@ struct Ctx {
   // finest-level arrays (indexed fine_off + cell)
   float *phi, *p1, *p2, *s0;
   uint8_t *frozen;
-  float *ut0, *ut1, *ut2;  // extension velocity (D planes of nfine each)
-  float *plan_v;           // extension plan: upwind velocity (D planes of nfine)
-  uint8_t *plan_f;         // extension plan: side / band / interface / boundary bits
+  // extension velocity: ut0 in D planes of nfine; ut1 and ut2, the sweeps' buffers, interleaved (a
+  // float2 or float4 per cell), but D planes to the persistent driver, which fills them anew
+  float *ut0, *ut1, *ut2;
+  // extension plan of a band cell: upwind velocity (D planes of nfine), side / band / interface /
+  // boundary bits.  They lie in p1, p2, s0 and in frozen, which a band cell does not use before
+  // its extension is done (and the classification after it sets p1 and p2 back to phi).
+  float *plan_v;
+  uint8_t *plan_f;
   uint32_t *cmask;
   int *cbase;
   float *macro;            // a MacroRec per finest cell: drho, u[D], S (sym, D(D+1)/2)
@@ -203,6 +208,8 @@ struct Ctx {
   long long nfine;         // finest-level cells over all cases
   long long link_cap;
   int *counters;           // per global level: [0] links, [1] iface cells, [2] flipped, [3] band blocks
+  // lists of the finest global levels, level l from l * list_cap (band lists: l * band_cap) on;
+  // there is memory for the levels from the first to the last at which a case ends
   int2 *iface_list, *flip_list;   // (ld, cell)
   int *band_list;          // global block ids
   int *check_list;         // blocks next to a flipped cell outside the previous band
