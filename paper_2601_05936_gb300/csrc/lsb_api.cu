@@ -26,12 +26,12 @@ using namespace lsb;
 namespace {
 
 constexpr int MAXL = 4;
-const char *const KNAMES[] = {"k_collide_stream", "k_interface_bc", "k_restrict", "k_ghost", "k_prolong", "k_level_tags", "k_observables", "k_export", "k_classify_phase", "k_classify_links", "k_post_classify", "k_geometry", "k_ext_init", "k_ext_iter", "k_adv_stage", "k_reinit_prep", "k_reinit_stage", "k_refill", "k_sensor", "k_init", "k_collect",
+const char *const KNAMES[] = {"k_collide_stream", "k_interface_bc", "k_restrict", "k_ghost", "k_prolong", "k_level_tags", "k_observables", "k_export", "k_classify_phase", "k_classify_links", "k_post_classify", "k_geometry", "k_levelset_fused", "k_ext_pass", "k_adv_pass", "k_adj_moments", "k_reinit_pass", "k_lsa_levelset", "k_sensor", "k_init", "k_collect",
                                "k_collide_stream_l1", "k_collide_stream_l2", "k_collide_stream_l3", "k_adj_seed",
                                "k_adj_links", "k_adj_collide", "k_adj_macro", "k_adj_geometry",
                                "k_levelset_persistent", "k_lsa", "k_adj_ghost", "k_adj_ghost_apply",
                                "k_adj_restrict", "k_tape"};
-constexpr int KADJ_SEED = 24, KADJ_LINKS = 25, KADJ_COLLIDE = 26, KADJ_MACRO = 27, KADJ_GEOM = 28, KLS_PERSIST = 29,
+constexpr int KLS_FUSED = 12, KADJ_MOMENTS = 15, KLSA_LEVELSET = 17, KADJ_SEED = 24, KADJ_LINKS = 25, KADJ_COLLIDE = 26, KADJ_MACRO = 27, KADJ_GEOM = 28, KLS_PERSIST = 29,
               KLSA = 30, KADJ_GHOST = 31, KADJ_GAPPLY = 32, KADJ_RESTRICT = 33, KTAPE = 34;
 constexpr int NKERN = sizeof(KNAMES) / sizeof(KNAMES[0]);
 
@@ -110,7 +110,7 @@ struct lsb_grid {
   long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
-  int driver = 0;             // 0: one launch per level-set pass, 1: one persistent launch
+  int driver = 0;             // 0: the planned level-set launch, 1: the persistent one
   int2 *d_iface = nullptr, *d_flip = nullptr;
   double *d_obs = nullptr;
   float *d_sens = nullptr;
@@ -626,7 +626,7 @@ lsb_status levelset(lsb_grid *g, int l) {
         RUN(16, 0, nb, nt, run_reinit_pass, Q, LN(g, nb, nt), C, S, l, st, r == 0 && st == 1 ? 1 : 0);
     return LSB_OK;
   }
-  RUN(KLS_PERSIST, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
+  RUN(KLS_FUSED, 0, 1, nt, run_levelset_fused, Q, LN(g, 1, nt), g->lsf[l], C, S, l, g->n_ext, due ? g->n_reinit : 0,
       (int)g->lds.size(), g->d_bar + 2, wait_limit32(g));
   g->classified[l] = true;
   return LSB_OK;
@@ -1292,7 +1292,7 @@ lsb_status adj_lb(lsb_grid *g, int l, const float *F, float *lamN, float *lamO, 
   const int Q = g->Q;
   const bool fine = l == g->Lmax - 1, frozen = !g->rec_moving;
   if (fine) {
-    if (frozen) RUN(KADJ_LINKS, 0, 1, 128, run_adj_moments, Q, LN(g, DYN_GRID, 128), C, l, F);
+    if (frozen) RUN(KADJ_MOMENTS, 0, 1, 128, run_adj_moments, Q, LN(g, DYN_GRID, 128), C, l, F);
     RUN(KADJ_LINKS, 0, 1, 128, run_adj_links, Q, LN(g, DYN_GRID, 128), C, l, F, lamN, g->d_linkadj, g->d_madj,
         g->d_grad, g->ncase, G, frozen);
   }
@@ -1330,7 +1330,7 @@ lsb_status adj_moving(lsb_grid *g, int l, const float *F, float *phi_n, float *u
   Gm.kappa = P.KP;
   RUN(11, 0, 1, 128, run_geometry, D, LN(g, DYN_GRID, 128), Gm, l);
   const bool rein = g->reinit_every == 1 && g->n_reinit > 0;
-  RUN(KLSA, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, std::min(g->lsa_band, g->band_cap)), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
+  RUN(KLSA_LEVELSET, 0, 1, nt, run_lsa_levelset, Q, LN(g, std::max(1, std::min(g->lsa_band, g->band_cap)), nt), R, S, l, g->n_ext, rein ? 1 : 0, P.A,
       g->d_bar + 2, wait_limit32(g));
   RUN(KLSA, 0, 1, 128, run_lsa_init_T, Q, LN(g, DYN_GRID, 128), R, l, F, P.A.LU, g->d_madj, P.A.LP);
   // lattice Boltzmann part with the geometry of phi_n; its phi adjoint goes to LP
