@@ -101,7 +101,7 @@ __device__ __forceinline__ float weno5_grad(const float v[5], float g[5]) {
 // ------------------------------------------------------------------ forward replay: interface velocity
 // u~ on interface cells = mean over cut links of (1 - q) u(x) + q u(y), with the
 // pre-collision moments of the stored state F (= f_n) and q from C.phi (= phi_n):
-// the values k_ext_init writes from the collide kernel's moments.
+// the values d_ext_init writes from the collide kernel's moments.
 template <int Q>
 __global__ void k_lsa_init(Ctx C, int glevel, const float *__restrict__ F, float *U0) {
   using LT = Lat<Q>;

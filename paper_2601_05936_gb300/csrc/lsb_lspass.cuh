@@ -13,9 +13,9 @@ __device__ __forceinline__ bool in_band(const Ctx &C, const LevelDev &L, const B
 
 // One Jacobi sweep of first-order upwind extension on the band (interface cells
 // copy their value).  Neighbours outside the band read the committed field ut0.
-// mode 0: sweep; 2: sweep and store the plan (velocity S(phi) n, upwind side and
-// band membership of each upwind neighbour, interface / boundary bits), which phi
-// fixes for all sweeps of a step; 3: sweep from the plan; 1: copy uin into ut0 on
+// mode 2: the first sweep, which stores the plan (velocity S(phi) n, upwind side and
+// band membership of each upwind neighbour, interface / boundary bits) that phi
+// fixes for all sweeps of a step; 3: a sweep from the plan; 1: copy uin into ut0 on
 // the band (commit).
 template <int D>
 __device__ __forceinline__ void d_ext_iter(const Ctx &C, BlockShape S, int glevel, const float *uin, float *uout, int mode) {
@@ -68,7 +68,7 @@ __device__ __forceinline__ void d_ext_iter(const Ctx &C, BlockShape S, int gleve
     const uint8_t tg = C.tag[L.cell_off + c];
     if (tg & TAG_IFACE) {
       for (int a = 0; a < D; ++a) uout[a * NF + fo + c] = uin[a * NF + fo + c];
-      if (mode == 2) C.plan_f[fo + c] = 64;
+      C.plan_f[fo + c] = 64;
       continue;
     }
     // interior: all +-1 neighbours inside the box (direct offsets, face-neighbour band flags)
@@ -120,14 +120,12 @@ __device__ __forceinline__ void d_ext_iter(const Ctx &C, BlockShape S, int gleve
         const float un = src[b * NF + fo + cn];
         acc[b] += va * (va > 0.f ? (u0[b] - un) : (un - u0[b]));
       }
-      if (mode == 2) {
-        C.plan_v[a * NF + fo + c] = va;
-        pf |= (dir < 0 ? 1 : 0) << a;
-        pf |= (inb ? 1 : 0) << (3 + a);
-      }
+      C.plan_v[a * NF + fo + c] = va;
+      pf |= (dir < 0 ? 1 : 0) << a;
+      pf |= (inb ? 1 : 0) << (3 + a);
     }
     for (int b = 0; b < D; ++b) uout[b * NF + fo + c] = u0[b] - L.dtau_ext * acc[b];
-    if (mode == 2) C.plan_f[fo + c] = pf;
+    C.plan_f[fo + c] = pf;
   }
 }
 // ------------------------------------------------------------------ transport
