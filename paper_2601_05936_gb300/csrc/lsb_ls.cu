@@ -690,7 +690,7 @@ enum : unsigned {  // slot flags
   SL_DIST = 8,      // 12 bits from here: lsf_dist
   SL_LD = 20        // the bits above: the cell's level descriptor
 };
-constexpr int kLsfMaxLd = 1 << (32 - SL_LD);  // more level descriptors: no slots (kcap 0)
+constexpr int kLsfMaxLd = 1 << (32 - SL_LD);  // more level descriptors: a launch per pass
 // How far a cell lies from the box faces, up to three cells: per axis 2 bits towards the low
 // face, 2 towards the high one.
 template <int D>

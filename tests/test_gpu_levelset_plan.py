@@ -11,6 +11,8 @@ import pytest
 
 pytestmark = pytest.mark.gpu
 
+CLUSTER, GRID = 0, 1
+
 
 def _sheared(nx=512, ny=96, U=0.08):
     X = np.broadcast_to(np.arange(nx) + 0.5, (ny, nx))
@@ -85,22 +87,41 @@ def test_band_that_vanishes():
 
 
 def test_stepping_inside_a_capture():
-    """Steps captured by the caller are recorded as they are: no copy, query or new plan meanwhile."""
+    """Steps captured by the caller keep the plan they were captured with: no copy, query or new
+    plan meanwhile.  Replayed while the band outgrows the slots of its cluster, the cells beyond them
+    take the per-cell functions beside a pass without a barrier before it."""
     import torch
 
     from paper_2601_05936_gb300 import lsb
     s = torch.cuda.Stream()
     g = lsb.Grid(_sheared(), stream=s)
     ref = lsb.Grid(_sheared(), stream=torch.cuda.Stream())
+    ref.set_driver(1)
     g.step(2)
     g.sync()
     graph = torch.cuda.CUDAGraph()
     with torch.cuda.graph(graph, stream=s):
         g.step(80)  # beyond the steps after which the band is looked at
-    for _ in range(10):
+    for _ in range(26):
         graph.replay()
     torch.cuda.synchronize()
-    ref.step(802)
+    shape = g.levelset_launch(0)
+    assert shape["form"] == CLUSTER and g.work_counts(0)["band"] > shape["cells"]
+    ref.step(2082)
     _same(g, ref)
     g.close()
     ref.close()
+
+
+@pytest.mark.parametrize("dims, block, form, slots", [
+    ((8, 8), (8, 4), CLUSTER, 1), ((256, 48), (32, 8), CLUSTER, 1), ((1000, 48), (32, 8), CLUSTER, 2),
+    ((3000, 48), (32, 8), GRID, 1), ((64, 64, 24), (16, 8, 4), GRID, 1), ((256, 256, 32), (32, 4, 4), GRID, 5)])
+def test_shapes_that_the_launch_tests_cover(dims, block, form, slots):
+    """The sizes of test_gpu_levelset_launch.py reach the forms they stand for; the last one has more
+    band cells than the grid holds."""
+    from test_gpu_levelset_launch import _layers
+    g = _grid(_layers(dims, (True,) * (len(dims) - 1) + (False,), block))
+    shape, band = g.levelset_launch(0), g.work_counts(0)["band"]
+    assert shape["form"] == form and shape["cells"] == slots * shape["ctas"] * shape["threads"], (shape, band)
+    assert (band > shape["cells"]) == (dims == (256, 256, 32)), (shape, band)
+    g.close()
