@@ -107,6 +107,7 @@ struct lsb_grid {
   LsfLimits lsf_lim;
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
   int band_est[MAXL] = {0, 0, 0, 0};  // band blocks it was planned for
+  bool full_launch = false;           // a plan takes a full CTA on every SM
   long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
@@ -308,7 +309,13 @@ lsb_status launched(lsb_grid *g, cudaError_t e) {
 
 // Kernels of a handle with a stream of its own launch as programmatic dependents of the
 // kernel before them (off while kernel timing is on, so that each launch's events
-// bracket that launch alone).
+// bracket that launch alone), unless a level-set launch needs a full CTA on every SM at once:
+// CTAs that sit on an SM waiting for their predecessor then keep it out, of this handle and of
+// others.  Two (four) handles of a 96 x 96 x 192 bubble on streams of their own, a step of all: 1050
+// (2720) us with dependents, 837 (1700) without, 835 (1665) with the launch per pass that the one
+// launch replaced.  One handle, dependents / plain launches: 2D 126 CTAs x 512 threads 58.5 / 58.5,
+// 152 x 1024 100.7 / 93.3 and 149 / 142; 3D 136 x 512 84.1 / 81.6, 152 x 1024 112.6 / 102.0 and
+// 158 / 146; a cluster 64.5 / 65.5.
 #ifndef LSB_PDL
 #define LSB_PDL 1
 #endif
@@ -318,7 +325,7 @@ lsb_status launched(lsb_grid *g, cudaError_t e) {
 #define LSB_PRIO 1
 #endif
 Launch LN(const lsb_grid *g, int grid, int block) {
-  return Launch{grid, block, g->stream, LSB_PDL && g->stream != nullptr && g->prof_mode == 0 ? 1 : 0,
+  return Launch{grid, block, g->stream, LSB_PDL && g->stream != nullptr && g->prof_mode == 0 && !g->full_launch ? 1 : 0,
                 LSB_PRIO ? g->prio_hi : 0};
 }
 
@@ -668,13 +675,23 @@ LsfPlan plan_levelset(const lsb_grid *g, int nb) {
   return P;
 }
 
+// The plan of level l, for a band of nb blocks.
+void set_plan(lsb_grid *g, int l, int nb, const LsfPlan &P) {
+  g->band_est[l] = nb;
+  g->lsf[l] = P;
+  g->full_launch = false;
+  for (int k = 0; k < g->Lmax; ++k)
+    if (has_finest(g, k) && g->lsf[k].form == LSF_GRID && g->lsf[k].grid == g->lsf_lim.grid && g->lsf[k].threads == 1024)
+      g->full_launch = true;
+}
+
 // The plan of level l for the band that its classification just listed.
 lsb_status plan_for_band(lsb_grid *g, int l) {
   int nb = 0;
   CU(cudaMemcpyAsync(&nb, g->d_counters + l * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost, g->stream));
   CU(cudaStreamSynchronize(g->stream));
-  g->band_est[l] = std::max(1, std::min(nb, g->band_cap));
-  g->lsf[l] = plan_levelset(g, g->band_est[l]);
+  nb = std::max(1, std::min(nb, g->band_cap));
+  set_plan(g, l, nb, plan_levelset(g, nb));
   return LSB_OK;
 }
 
@@ -725,8 +742,7 @@ lsb_status follow_band(lsb_grid *g) {
         drop_graphs(g);
         changed = true;
       }
-      g->band_est[l] = nb;
-      g->lsf[l] = P;
+      set_plan(g, l, nb, P);
     }
   }
   if (g->words == lsb_grid::WORDS_NONE && g->unseen_steps >= kWordsEvery && !capturing()) {
