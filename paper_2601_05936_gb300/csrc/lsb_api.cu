@@ -107,7 +107,7 @@ struct lsb_grid {
   LsfLimits lsf_lim;
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
   int band_est[MAXL] = {0, 0, 0, 0};  // band blocks it was planned for
-  bool full_launch = false;           // a plan takes a full CTA on every SM
+  bool full_launch = false;           // a plan that runs takes a full CTA on every SM
   long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
@@ -325,7 +325,7 @@ lsb_status launched(lsb_grid *g, cudaError_t e) {
 #define LSB_PRIO 1
 #endif
 Launch LN(const lsb_grid *g, int grid, int block) {
-  return Launch{grid, block, g->stream, LSB_PDL && g->stream != nullptr && g->prof_mode == 0 && !g->full_launch ? 1 : 0,
+  return Launch{grid, block, g->stream, LSB_PDL && g->stream != nullptr && g->prof_mode == 0 && !(g->full_launch && g->driver == 0) ? 1 : 0,
                 LSB_PRIO ? g->prio_hi : 0};
 }
 
@@ -639,6 +639,21 @@ lsb_status levelset(lsb_grid *g, int l) {
   return LSB_OK;
 }
 
+bool ls_active_any(const lsb_grid *g, int l) {
+  for (const CaseHost &c : g->cases)
+    if (c.L - 1 == l && c.p.ls_active) return true;
+  return false;
+}
+
+// Whether a level-set launch of the step takes a full CTA on every SM (see LN).
+void find_full_launch(lsb_grid *g) {
+  g->full_launch = false;
+  for (int l = 0; l < g->Lmax; ++l) {
+    const LsfPlan &P = g->lsf[l];
+    if (ls_active_any(g, l) && P.form == LSF_GRID && P.grid == g->lsf_lim.grid && P.threads == 1024) g->full_launch = true;
+  }
+}
+
 // Shape of the one-launch level-set update for a band of nb blocks (the launch is right for
 // any band; the shape only sets its speed).  Up to two cells per thread of a 16-CTA cluster of
 // 1024 threads the cluster's barrier wins (0.6 - 1.0 us a pass against 1.4 us of the grid's);
@@ -679,10 +694,7 @@ LsfPlan plan_levelset(const lsb_grid *g, int nb) {
 void set_plan(lsb_grid *g, int l, int nb, const LsfPlan &P) {
   g->band_est[l] = nb;
   g->lsf[l] = P;
-  g->full_launch = false;
-  for (int k = 0; k < g->Lmax; ++k)
-    if (has_finest(g, k) && g->lsf[k].form == LSF_GRID && g->lsf[k].grid == g->lsf_lim.grid && g->lsf[k].threads == 1024)
-      g->full_launch = true;
+  find_full_launch(g);
 }
 
 // The plan of level l for the band that its classification just listed.
@@ -752,12 +764,6 @@ lsb_status follow_band(lsb_grid *g) {
     g->unseen_steps = 0;
   }
   return LSB_OK;
-}
-
-bool ls_active_any(const lsb_grid *g, int l) {
-  for (const CaseHost &c : g->cases)
-    if (c.L - 1 == l && c.p.ls_active) return true;
-  return false;
 }
 
 // Copy every case's level-l populations from src to dst (same offsets: each level's
@@ -1774,6 +1780,7 @@ lsb_status lsb_set_params(lsb_grid *g, int case_idx, const lsb_params *params) {
   g->n_reinit = params->n_reinit;
   g->regrid_every = params->regrid_every;
   if (relaunch) drop_graphs(g);
+  find_full_launch(g);  // (the level set may have been frozen, or set free)
   // stream-ordered before the next step; a copy from pageable memory returns once the
   // source is staged, so the host descriptors may change again right away
   CU(cudaMemcpyAsync(g->d_lds, g->lds.data(), sizeof(LevelDev) * g->lds.size(), cudaMemcpyHostToDevice, g->stream));
