@@ -493,7 +493,7 @@ __device__ __forceinline__ void d_lsa_ext_v(const Ctx &C, const BlockShape &S, i
 // The adjoints LP (of phi) and LU (of u~) change in place; phi_n is overwritten by phi* on the
 // band while the reinitialisation is transposed and written back from PB.
 // A: scratch of the sweep (LsaScratch); rein: the step reinitialised.
-template <int Q>
+template <int Q, int MODE>  // MODE of the barriers
 __global__ void __launch_bounds__(512, LSA_MINB) k_lsa_levelset(Ctx C, BlockShape S, int glevel, int n_ext, int rein,
                                                                 LsaScratch A, unsigned *bar, unsigned limit) {
   constexpr int D = Lat<Q>::D;
@@ -509,16 +509,16 @@ __global__ void __launch_bounds__(512, LSA_MINB) k_lsa_levelset(Ctx C, BlockShap
   E.ut0 = A.S0;
   for (int k = 0; k < n_ext; ++k) {
     d_ext_iter<D>(E, S, glevel, Sk(k), Sk(k + 1), k == 0 ? 2 : 3);
-    if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+    if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
   }
   Ctx T = C;
   T.p1 = A.A1;
   T.p2 = A.A2;
   T.ut0 = Sk(n_ext);  // the committed u~ (read at the cells themselves only)
   d_adv_stage<D>(T, S, glevel, 1);
-  if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+  if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
   d_adv_stage<D>(T, S, glevel, 2);
-  if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+  if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
   if (rein) {
     const int nl = min(C.counters[glevel * NCOUNT + 3], C.band_cap);
     for (int w = blockIdx.x; w < nl; w += gridDim.x) {  // phi_n of the band, kept
@@ -529,7 +529,7 @@ __global__ void __launch_bounds__(512, LSA_MINB) k_lsa_levelset(Ctx C, BlockShap
       A.PB[fc] = phi_n[fc];
     }
     d_adv_stage<D>(T, S, glevel, 3);  // phi* into phi_n (each cell by the thread that kept it)
-    if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+    if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
     Ctx R = C;
     R.p1 = A.R1;
     R.p2 = A.R2;
@@ -537,29 +537,29 @@ __global__ void __launch_bounds__(512, LSA_MINB) k_lsa_levelset(Ctx C, BlockShap
     R.s0 = A.SS;
     d_reinit_prep<Q>(R, S, glevel);
     d_reinit_stage<D>(R, S, glevel, 1);  // reads only its own cell's frozen flag and S(phi*)
-    if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+    if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
     d_reinit_stage<D>(R, S, glevel, 2);
-    if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+    if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
     for (int st = 3; st >= 1; --st) {
       d_lsa_reinit<D>(R, S, glevel, st, st == 3 ? A.R2 : A.R1, A.LP, A.L1, A.L2, A.LS0);
-      if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+      if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
     }
   }
   for (int st = 3; st >= 1; --st) {
     d_lsa_adv<D>(T, S, glevel, st, st == 3 ? A.A2 : A.A1, rein ? A.PB : nullptr, A.LP, A.L1, A.L2, A.LU);
-    if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+    if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
   }
   if (n_ext > 0) {
     float *Lin = A.LU;
     for (int k = n_ext - 1; k >= 0; --k) {
       float *out = Lin == A.LK0 ? A.LK1 : A.LK0;
       d_lsa_ext_T<D>(E, S, glevel, Sk(k), A.S0, Lin, out, A.LU, A.LV);
-      if (!lsf_barrier<1>(bar, target, C.err, &wait_limit)) return lsf_leave(bar);
+      if (!lsf_barrier<MODE>(bar, target, C.err, &wait_limit)) return lsf_leave<MODE>(bar);
       Lin = out;
     }
     d_lsa_ext_v<D>(E, S, glevel, Lin, A.LU, A.LV, A.LP);
   }
-  lsf_leave(bar);
+  lsf_leave<MODE>(bar);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -576,22 +576,25 @@ cudaError_t run_lsa_init_T(int Q, Launch L, Ctx C, int glevel, const float *F, f
   LSA_Q(k_lsa_init_T, C, glevel, F, LS0, MA, LPHI);
 }
 // grid: at most the resident CTAs (a cooperative launch needs them all)
-template <int Q>
+template <int Q, int MODE>
 cudaError_t lsa_levelset_launch(Launch L, Ctx C, BlockShape S, int glevel, int n_ext, int rein, LsaScratch A,
                                 unsigned *bar, unsigned limit) {
   int per_sm = 0, dev = 0, sms = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lsa_levelset<Q>, L.block, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_lsa_levelset<Q, MODE>, L.block, 0);
   if (e != cudaSuccess) return e;
   const int grid = L.grid < per_sm * sms ? L.grid : per_sm * sms;
   void *args[] = {&C, &S, &glevel, &n_ext, &rein, &A, &bar, &limit};
-  return cudaLaunchCooperativeKernel((const void *)k_lsa_levelset<Q>, dim3(grid), dim3(L.block), args, 0, L.stream);
+  return cudaLaunchCooperativeKernel((const void *)k_lsa_levelset<Q, MODE>, dim3(grid), dim3(L.block), args, 0, L.stream);
 }
 cudaError_t run_lsa_levelset(int Q, Launch L, Ctx C, BlockShape S, int glevel, int n_ext, int rein, LsaScratch A,
                              unsigned *bar, unsigned limit) {
-  if (Q == 9) return lsa_levelset_launch<9>(L, C, S, glevel, n_ext, rein, A, bar, limit);
-  return lsa_levelset_launch<19>(L, C, S, glevel, n_ext, rein, A, bar, limit);
+  if (limit == kDefaultWait)
+    return Q == 9 ? lsa_levelset_launch<9, 2>(L, C, S, glevel, n_ext, rein, A, bar, limit)
+                  : lsa_levelset_launch<19, 2>(L, C, S, glevel, n_ext, rein, A, bar, limit);
+  return Q == 9 ? lsa_levelset_launch<9, 1>(L, C, S, glevel, n_ext, rein, A, bar, limit)
+                : lsa_levelset_launch<19, 1>(L, C, S, glevel, n_ext, rein, A, bar, limit);
 }
 
 }  // namespace lsb

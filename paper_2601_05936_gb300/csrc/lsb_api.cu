@@ -93,7 +93,7 @@ struct lsb_grid {
   uint8_t *d_linkdir = nullptr;
   long long link_list_off[MAXL] = {0, 0, 0, 0};
   int list_l0 = 0;  // first level at which a case ends: the lists' memory starts with its region
-  // pinned host words: the counters of every level and the error word, as they lie behind
+  // pinned host words: the counters of every level, the error word and d_recflip, as they lie behind
   // d_counters (read back by the synchronising calls and, between them, by follow_band), then
   // the observables of every case
   int *h_words = nullptr;
@@ -108,7 +108,7 @@ struct lsb_grid {
   LsfPlan lsf[MAXL];  // per finest global level: the one-launch level-set update
   int band_est[MAXL] = {0, 0, 0, 0};  // band blocks it was planned for
   bool full_launch = false;           // a plan that runs takes a full CTA on every SM
-  long long wait_limit = 1LL << 22;  // iterations before a grid barrier gives up
+  long long wait_limit = kDefaultWait;  // iterations before a grid barrier gives up
   bool ls_dirty = false;  // stage arrays no longer mirror phi / u~ outside the band (driver 1 ran)
   float obj_eps = 0.f;    // > 0: observables and objective with the smoothed gas indicator H_eps
   int driver = 0;             // 0: the planned level-set launch, 1: the persistent one
@@ -379,7 +379,7 @@ constexpr int EXPORT_CTAS = 152 * 8;  // resident at 256 threads: a cell a threa
 #define LSB_GEO_CTAS 512
 #endif
 
-constexpr int NWORDS = MAXL * NCOUNT + 1;  // counters of every level, error word
+constexpr int NWORDS = MAXL * NCOUNT + 2;  // counters of every level, error word, flips of a recording
 // Band cells, in multiples of the one-launch update's slots (3D: 778 k, 2D: 1.4 M), from which a
 // launch per pass wins.  us a step with one launch / a launch per pass:
 //   3D   1.37 M cells (two levels) 1217 / 1305, 2.36 M 1062 / 1052, 4.06 M 1902 / 1788, 16 M 7418 / 6499
@@ -707,7 +707,7 @@ lsb_status plan_for_band(lsb_grid *g, int l) {
   return LSB_OK;
 }
 
-// Copy the device's words (the counters of every level, then the error word) into h_words.
+// Copy the device's words into h_words.
 lsb_status read_words(lsb_grid *g) {
   CU(cudaMemcpyAsync(g->h_words, g->d_counters, sizeof(int) * NWORDS, cudaMemcpyDeviceToHost, g->stream));
   return LSB_OK;
@@ -1683,6 +1683,7 @@ lsb_status lsb_create_grid(int n_cases, const lsb_grid_desc *descs, const lsb_pa
   const size_t nlist = (size_t)(l1 - g->list_l0);
   ALLOC(g->d_counters, sizeof(int) * NWORDS);
   g->d_err = g->d_counters + MAXL * NCOUNT;
+  g->d_recflip = g->d_err + 1;
   ALLOC(g->d_work, sizeof(int) * 2 * MAXL);
   s = pin_host(g);
   if (s) { g_create_error = g->err; lsb_destroy(g); return s; }
@@ -2207,7 +2208,6 @@ lsb_status lsb_record(lsb_grid *g, int checkpoint_every) {
     return fail(g, LSB_ESTATE, "the moving-interface adjoint needs reinit_every <= 1 and n_reinit <= 1");
   CU(cudaStreamSynchronize(g->stream));
   rec_clear(g);
-  if (!g->d_recflip) TRY(dalloc(g, &g->d_recflip, sizeof(int)));
   CU(cudaMemset(g->d_recflip, 0, sizeof(int)));
   g->rec_on = 1;
   g->rec_moving = live ? 1 : 0;
@@ -2223,12 +2223,12 @@ lsb_status lsb_backward(lsb_grid *g, const double *dJ_dobs, double *dJ_dparams, 
   const int every = g->rec_every;
   const bool mv = g->rec_moving != 0;
   if (mv) {
-    int flip = 0;
+    TRY(read_words(g));
     CU(cudaStreamSynchronize(g->stream));
-    CU(cudaMemcpy(&flip, g->d_recflip, sizeof(int), cudaMemcpyDeviceToHost));
-    if (flip) return fail(g, LSB_ESTATE, "a cell changed phase during the recorded window");
+    const int flip = g->h_words[MAXL * NCOUNT + 1];
     // the reverse launch's grid: a CTA per band block of the window (no flips: the same all through)
-    CU(cudaMemcpy(&g->lsa_band, g->d_counters + (g->Lmax - 1) * NCOUNT + 3, sizeof(int), cudaMemcpyDeviceToHost));
+    g->lsa_band = g->h_words[(g->Lmax - 1) * NCOUNT + 3];
+    if (flip) return fail(g, LSB_ESTATE, "a cell changed phase during the recorded window");
   }
   TRY(adj_buffers(g, (int)std::min<long long>(every, std::max<long long>(T, 1))));
   const size_t sf = state_floats(g), sb = sizeof(float) * sf, sl = slot_floats(g);

@@ -220,6 +220,8 @@ struct Ctx {
   float fp16_scale, fp16_inv;
 };
 
+constexpr unsigned kDefaultWait = 1u << 22;  // iterations of a grid barrier before it gives up, by default
+
 enum : int { ERR_LINK_OVF = 1, ERR_LIST_OVF = 2, ERR_NONFINITE = 4, ERR_BAND_OVF = 8, ERR_TIMEOUT = 16 };
 // device counters per global level: [0] cut links, [1] interface cells, [2] flipped cells,
 // [3] band blocks, [4] blocks next to a flipped cell outside the previous band (check

@@ -774,7 +774,7 @@ __global__ void __launch_bounds__(1024, 1) k_levelset_fused(Ctx C, BlockShape S,
     return L;
   };
   auto leave = [&]() {
-    if (MODE == 1) lsf_leave(bar);
+    if (MODE == 1) lsf_leave<MODE>(bar);
   };
   __syncthreads();
   // ---- slots, and the first extension sweep with the plan

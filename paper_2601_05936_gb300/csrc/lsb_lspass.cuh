@@ -335,6 +335,9 @@ __device__ __forceinline__ void d_reinit_stage(const Ctx &C, BlockShape S, int g
 // and cost each 0.13 us (3D bubble, 28 of them: step 691 -> 695 us).  false: it gave up, ERR_TIMEOUT
 // is set, and the CTA has to leave: it arrives at no later barrier, so no CTA gets past the next
 // one either.
+// 2: a cooperative launch with the default limit, a constant: the reverse sweep's launch (28
+// barriers) is built for it too, where a limit read from memory costs 1% (2D window 7.56 and 7.64
+// ms).
 constexpr unsigned kGaveUp = 1u << 16;  // (more than a cooperative grid's CTAs)
 template <int MODE>
 __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int *err, const unsigned *limit) {
@@ -345,7 +348,19 @@ __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int
   __shared__ int gave_up;
   target += gridDim.x;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (MODE == 2 && threadIdx.x == 0) {
+    gave_up = 0;
+    unsigned v, reads = 0;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (++reads > kDefaultWait) {
+        gave_up = 1;
+        atomicOr(err, ERR_TIMEOUT);
+        break;
+      }
+    } while ((int)(v - target) < 0);
+  } else if (threadIdx.x == 0) {
     gave_up = 0;
     unsigned v, left = *limit;
     asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
@@ -365,13 +380,15 @@ __device__ __forceinline__ bool lsf_barrier(unsigned *bar, unsigned &target, int
   return gave_up == 0;
 }
 
-// Every CTA of a MODE 1 launch passes here once, last: bar[1] counts them (and, from kGaveUp up,
-// those that gave up), and the last one clears both words for the next launch.
+// Every CTA of a MODE 1 or 2 launch passes here once, last: bar[1] counts them (and, from kGaveUp
+// up, those that gave up with an arrival not read back), and the last one clears both words for
+// the next launch.
+template <int MODE>
 __device__ __forceinline__ void lsf_leave(unsigned *bar) {
   if (threadIdx.x != 0) return;
   const unsigned out = atomicAdd(bar + 1, 1u);
-  if (out % kGaveUp == gridDim.x - 1) {
-    if (out >= kGaveUp) __threadfence();  // (1 us of the launch where it is not needed)
+  if ((MODE == 2 ? out : out % kGaveUp) == gridDim.x - 1) {
+    if (MODE != 2 && out >= kGaveUp) __threadfence();  // (1 us of the launch where it is not needed)
     bar[0] = 0;
     bar[1] = 0;
   }
