@@ -368,7 +368,9 @@ __device__ __forceinline__ void d_lsa_adv(const Ctx &C, const BlockShape &S, int
 // committed u~ of the previous step, which the sweeps leave alone).  Lin holds the adjoint of
 // u_{k+1} at band cells (cleared as it is read, unless it is LU itself), Lout (zero before)
 // collects that of u_k; a neighbour outside the band gets its part in LU.  LV(a, c)
-// accumulates d/dv_a over the sweeps.
+// accumulates d/dv_a over the sweeps.  Cleared where there is something to clear: a store of zero
+// right behind the load of the same word made a sweep over 2.2 M band cells take 325 us instead of
+// 80 (and the reverse of a step on 384 x 384 x 48 cells 7.8 ms instead of 5.4).
 template <int D>
 __device__ __forceinline__ void d_lsa_ext_T(const Ctx &C, const BlockShape &S, int glevel, const float *Sk,
                                             const float *S0, float *Lin, float *Lout, float *LU, float *LV) {
@@ -382,7 +384,7 @@ __device__ __forceinline__ void d_lsa_ext_T(const Ctx &C, const BlockShape &S, i
     float lc[3] = {0.f, 0.f, 0.f};
     for (int b = 0; b < D; ++b) {
       lc[b] = Lin[b * NF + fo + c];
-      if (Lin != LU) Lin[b * NF + fo + c] = 0.f;
+      if (Lin != LU && lc[b] != 0.f) Lin[b * NF + fo + c] = 0.f;
     }
     const uint8_t pf = C.plan_f[fo + c];
     if (pf & 64) {  // interface cell: carried over
@@ -436,16 +438,19 @@ __device__ __forceinline__ void d_lsa_ext_v(const Ctx &C, const BlockShape &S, i
     const long long fo = L.fine_off;
     const long long c = cidx(L, x, y, z);
     for (int b = 0; b < D; ++b) {
-      LU[b * NF + fo + c] = Lin[b * NF + fo + c];
-      Lin[b * NF + fo + c] = 0.f;
+      const float l = Lin[b * NF + fo + c];
+      LU[b * NF + fo + c] = l;
+      if (l != 0.f) Lin[b * NF + fo + c] = 0.f;
     }
     if (C.plan_f[fo + c] & 64) continue;
     float lv[3] = {0.f, 0.f, 0.f};
     bool any = false;
     for (int a = 0; a < D; ++a) {
       lv[a] = LV[a * NF + fo + c];
-      LV[a * NF + fo + c] = 0.f;
-      any |= lv[a] != 0.f;
+      if (lv[a] != 0.f) {
+        LV[a * NF + fo + c] = 0.f;
+        any = true;
+      }
     }
     if (!any) continue;
     const int crd[3] = {x, y, z};
@@ -487,9 +492,10 @@ __device__ __forceinline__ void d_lsa_ext_v(const Ctx &C, const BlockShape &S, i
 // As launches these were 41 per sub-step beside 20 dense copies and fills; now 28 passes that
 // touch band cells only.  A window of 8 steps on 64 x 96 cells (two levels) and its reverse
 // sweep 10.4 -> 7.9 ms, 4 steps on 96 x 96 x 128 (two levels) 31.4 -> 25.4 ms; the launch
-// itself takes 130 us there in 2D (a CTA per band block) and 0.8 ms in 3D (442 k band cells:
-// the atomics of the transposes).  Two CTAs of 512 threads per SM: 0.82 ms per sub-step
-// against 0.99 with one (more chains in flight) and 0.84 with three (spills).
+// itself takes 130 us there in 2D (a CTA per band block) and 0.61 ms in 3D (442 k band cells;
+// 0.82 before the sweeps' accumulators were cleared only where they hold something).  Two CTAs of
+// 512 threads per SM: 0.82 ms per sub-step then, against 0.99 with one (more chains in flight) and
+// 0.84 with three (spills).  As a launch per pass, 2.2 M band cells: within 1%.
 // The adjoints LP (of phi) and LU (of u~) change in place; phi_n is overwritten by phi* on the
 // band while the reinitialisation is transposed and written back from PB.
 // A: scratch of the sweep (LsaScratch); rein: the step reinitialised.
